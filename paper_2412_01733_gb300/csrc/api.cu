@@ -77,7 +77,8 @@ void free_all(TreeWorkspace *ws) {
                     ws->adj_cot, ws->adj_xt, ws->adj_xg, ws->adj_mg, ws->adj_ccot, ws->pleaf, ws->nparent,
                     ws->seg_off, ws->seg_cstart, ws->seg_bchunk, ws->seg_bfirst, ws->seg_part,
                     ws->seg_digit_off, ws->cmask, ws->morder, ws->mbucket, ws->xm, ws->hs_x, ws->hs_v,
-                    ws->hs_m, ws->hs_a, ws->hs_phi, ws->hs_diag, ws->dctl};
+                    ws->hs_m, ws->hs_a, ws->hs_phi, ws->hs_diag, ws->dctl, ws->tile_hdr, ws->tile_idx,
+                    ws->tile_part, ws->tile_next, ws->ghead, ws->gtiles};
     for (void *p : ptrs)
         if (p) cudaFree(p);
     if (ws->graph_exec) cudaGraphExecDestroy(ws->graph_exec);
@@ -281,6 +282,14 @@ tree_status_t tree_workspace_create(int64_t n_max, const TreeParams *p, TreeWork
               dalloc(&ws->cmask, 2 * (size_t)chunks_max) &&
               dalloc(&ws->gscan_status, (size_t)(chunks_max / 2048 + 2)) &&
               dalloc(&ws->dmac, kLevels) && dalloc(&ws->dctl, 1);
+    if (ok && n_max > 0 && n_max <= (p->precision == TREE_F64 ? kSplitMaxN64 : kSplitMaxN32)) {
+        // tile slots of the split walk (groups of 64 use half of them: two targets per lane)
+        const size_t T = (((size_t)n_max * kTilesPer + 4096) / kTileChunk) * kTileChunk;
+        ok = dalloc(&ws->tile_hdr, T) && dalloc(&ws->tile_idx, T * 32) && dalloc(&ws->tile_next, T / kTileChunk) &&
+             dalloc((unsigned char **)&ws->tile_part, T * 32 * v4) &&
+             dalloc(&ws->ghead, (size_t)ws->groups_max) && dalloc(&ws->gtiles, (size_t)ws->groups_max);
+        ws->tile_cap = ok ? (uint32_t)T : 0u;
+    }
     ws->chunks_cap = chunks_max;
     ws->box_cap = 1;
     if (!ok) {
@@ -486,12 +495,18 @@ tree_status_t tree_moments(TreeWorkspace *ws, const void *x, const void *m, void
     return TREE_OK;
 }
 
-static tree_status_t walk(TreeWorkspace *ws, int mode, const WalkOut &out, cudaStream_t s) {
+static tree_status_t walk(TreeWorkspace *ws, int mode, WalkOut out, cudaStream_t s) {
     tree_status_t st = upload_mac(ws, s);
     if (st != TREE_OK) return st;
     PhaseScope ph(ws, mode == kWalkForce ? TREE_PHASE_WALK : TREE_PHASE_LISTS, s);
-    if (walk_widest_first(ws)) TRY_CUDA(launch_group_order(ws, s));
-    if (ws->p.precision == TREE_F64) TRY_CUDA(launch_walk_f64(ws, mode, out, s));
+    // (the split walk has no straggler to put first)
+    const bool split = mode == kWalkForce && walk_splits(ws);
+    out.ordered = walk_widest_first(ws) && !split;
+    if (out.ordered) TRY_CUDA(launch_group_order(ws, s));
+    if (split) {
+        if (ws->p.precision == TREE_F64) TRY_CUDA(launch_walk_split_f64(ws, out, s));
+        else TRY_CUDA(launch_walk_split_f32(ws, out, s));
+    } else if (ws->p.precision == TREE_F64) TRY_CUDA(launch_walk_f64(ws, mode, out, s));
     else TRY_CUDA(launch_walk_f32(ws, mode, out, s));
     return TREE_OK;
 }

@@ -2,6 +2,7 @@
 #pragma once
 
 #include <cuda_runtime.h>
+#include <math.h>
 #include <stdint.h>
 
 #include <vector>
@@ -33,6 +34,15 @@ constexpr int64_t kMaxNodes = (int64_t)1 << 29;  // node indices fit 29 bits (wa
 // same time together in L2 (measured 0.3 % faster on the galaxy at N = 1.7e7
 // and 1e8, equal at 2^20).
 constexpr int64_t kWalkOrderMaxN = (int64_t)1 << 22;
+
+// Split walk (walk.cuh): workspaces of at most this many particles (FP32,
+// FP64; the measured lines are in walk.cuh) keep tile slots for it, kTilesPer
+// for each particle, handed out kTileChunk at a time.  12 a particle serve
+// theta >= 0.43 at N = 65536 (660 B a slot in FP32).
+constexpr int64_t kSplitMaxN32 = (int64_t)1 << 16, kSplitMaxN64 = (int64_t)1 << 17;
+constexpr int kTilesPer = 12;
+constexpr int kTileChunk = 16;
+constexpr uint32_t kTilesFull = 0xffffffffu;     // group whose tiles found no slot
 
 // lookback status words: 2-bit flag + 30-bit value
 constexpr uint32_t kFlagAgg = 1u << 30;
@@ -73,8 +83,9 @@ enum CounterSlots {
     kCtrLevelTrunc = kCtrLevelRawEnd + 24,    // 23 truncation points
     kCtrGroups = kCtrLevelTrunc + 24,         // number of walk groups
     kCtrGScanTicket = kCtrGroups + 1,         // group-count scan tiles
-    kCtrWalkTicket = kCtrGroups + 2,          // walk: next group slot (reset before every walk)
-    kCtrAbort = kCtrGroups + 3,               // stage whose bounded wait gave up (0: none)
+    kCtrAbort = kCtrGroups + 2,               // stage whose bounded wait gave up (0: none)
+    kCtrWalkTicket = kCtrGroups + 3,          // walk: next group slot (reset before every walk)
+    kCtrTiles = kCtrGroups + 4,               // split walk: tile slots handed out (reset with the ticket)
     kCtrCount = kCtrGroups + 8
 };
 
@@ -179,6 +190,11 @@ struct TreeWorkspace {
     uint32_t *gkey = nullptr;          // per group: extent bucket (scratch for gorder)
     uint32_t *gbucket = nullptr;       // [2][32] bucket counts / cursors
     int64_t groups_max = 0;
+    // split walk (n_max <= kSplitMaxN32 or kSplitMaxN64): tile slots, and the groups' chains of chunks
+    uint2 *tile_hdr = nullptr;
+    uint32_t *tile_idx = nullptr, *tile_next = nullptr, *ghead = nullptr, *gtiles = nullptr;
+    void *tile_part = nullptr;
+    uint32_t tile_cap = 0;             // slots (0: no split walk)
     // interaction lists (allocated on first use)
     int64_t *list_cnt = nullptr;       // [2][groups+1] counts -> offsets
     int32_t *pc_list = nullptr, *pp_list = nullptr;
@@ -207,6 +223,20 @@ struct TreeWorkspace {
 
 namespace treegb {
 
+// Whether the force walk is split: the workspace keeps tile slots, and the
+// lists are expected to fit them.  A particle meets about 95 log2(n) / theta^2
+// sources (Plummer spheres and the galaxy, within a tenth), at most n; groups
+// hold 28 or more on average, and a chunk's unused slots come to about one per
+// particle.  Lists that do not fit after all are walked by one warp as ever,
+// but only after the traversal has been tried in vain, hence the line.
+inline bool walk_splits(const TreeWorkspace *ws) {
+    if (ws->tile_cap == 0) return false;
+    const double n = (double)ws->n, th = ws->p.theta;
+    double src = n;
+    if (th > 0.0 && 95.0 * log2(n + 2.0) / (th * th) < n) src = 95.0 * log2(n + 2.0) / (th * th);
+    const double lanes = ws->p.group_size == 16 ? 14.0 : 28.0;  // groups of 64 share a slot two targets to a lane
+    return n * (src / (32.0 * lanes) + 1.0) <= 0.9 * (double)ws->tile_cap;
+}
 inline bool walk_widest_first(const TreeWorkspace *ws) { return ws->n < kWalkOrderMaxN; }
 
 // ---------------------------------------------------------------- device helpers
@@ -442,7 +472,8 @@ cudaError_t launch_export_tree(TreeWorkspace *ws, int64_t nn, int32_t *level, ui
 // moments.cu
 cudaError_t launch_moments(TreeWorkspace *ws, cudaStream_t s);
 // walk_f32.cu / walk_f64.cu
-enum WalkMode { kWalkForce = 0, kWalkCount = 1, kWalkEmit = 2 };
+// kWalkTiles, kWalkFold: first and last kernel of the split walk
+enum WalkMode { kWalkForce = 0, kWalkCount = 1, kWalkEmit = 2, kWalkTiles = 3, kWalkFold = 4 };
 struct WalkOut {
     void *a;            // [3][n] caller order (or NULL in count/emit modes)
     void *phi;          // [n] or NULL
@@ -450,9 +481,13 @@ struct WalkOut {
     double half_tau;    // leapfrog kick
     void *v_mirror = nullptr;    // also receives the kicked v (e.g. mapped host memory), or NULL
     void *phi_mirror = nullptr;  // also receives phi, or NULL
+    bool ordered = false;        // groups in gorder's order (launch_group_order), else in key order
 };
 cudaError_t launch_walk_f32(TreeWorkspace *ws, int mode, const WalkOut &out, cudaStream_t s);
 cudaError_t launch_walk_f64(TreeWorkspace *ws, int mode, const WalkOut &out, cudaStream_t s);
+// walk_split_f32.cu / walk_split_f64.cu
+cudaError_t launch_walk_split_f32(TreeWorkspace *ws, const WalkOut &out, cudaStream_t s);
+cudaError_t launch_walk_split_f64(TreeWorkspace *ws, const WalkOut &out, cudaStream_t s);
 // adjoint.cu
 cudaError_t launch_adjoint(TreeWorkspace *ws, const void *abar, const void *phibar, void *xbar, void *mbar,
                            cudaStream_t s);

@@ -1,6 +1,22 @@
 // walk.cuh -- the tree walk and force evaluation (Sec. 2 TreeCode; Eq. 1 for
 // the near part), one warp per group of Gs key-ordered particles.
 //
+// Small systems leave most of the chip idle in this form: a group is one
+// warp's serial chain (at N = 30011 there are 989 groups for 3648 resident
+// warps, and the group with the longest lists sets the time), and in FP64 one
+// SM's pipe does 2 lanes a clock.  They take the split walk, three kernels:
+// the traversal writes each group's tiles of 32 sources, in the order in which
+// it would have evaluated them, into tile slots (kWalkTiles); every slot is
+// then evaluated by whichever warp of the chip comes to it (k_eval_tiles); and
+// the partial sums are folded, group by group, in the order of the tiles
+// (kWalkFold).  Each tile's partial sums and the order of the folds are those
+// of the one-warp walk, so the results are the same bits, alone or in an
+// ensemble.  Walk of a Plummer sphere, theta = 0.7 (one-warp -> split): FP32
+// N = 1031 62 -> 39 us, 16384 334 -> 172, 65536 495 -> 415, but 100003 560 ->
+// 592 (1.25 KB of slot traffic per tile, and the traversal no longer hides
+// behind the arithmetic); FP64 N = 16384 12.8 -> 2.7 ms, 65536 21.6 -> 13.1,
+// 131072 32.6 -> 28.7.  walk_splits() draws the lines there.
+//
 // Traversal (per warp, depth first, stack in shared memory):
 //   the stack holds ranges of sibling nodes (children are contiguous in the
 //   breadth-first numbering), one entry per opened cell.  Each step pops up
@@ -21,6 +37,8 @@
 // cancel in FP32 against a potential that can be far smaller than m_i/eps);
 // with eps = 0 a guarded variant also skips other r = 0 pairs.
 #pragma once
+
+#include <cfloat>
 
 #include "common.cuh"
 
@@ -56,6 +74,13 @@ struct WalkArgs {
     const int64_t *seg_off;   // segment offsets (nseg > 1): a group walks its own segment's tree
     int64_t nseg;
     const DevBox *box;        // per segment: the tree's cube (side 2^k)
+    // split walk (kWalkTiles, k_eval_tiles, kWalkFold): tile slots and the groups' chains of them
+    uint2 *tile_hdr;          // per slot: {group, sources | far cells << 8}; 0 sources: unused
+    uint32_t *tile_idx;       // per slot: 32 source indices
+    void *tile_part;          // per slot: Vec4 partial sums of 32 TPL targets
+    uint32_t *tile_next;      // per chunk of kTileChunk slots: first slot of the group's next chunk
+    uint32_t tile_cap;        // slots, a multiple of kTileChunk
+    uint32_t *ghead, *gtiles; // per group: first slot; tiles, or kTilesFull
 };
 
 template <typename Real> __device__ __forceinline__ Real rsqrt_r(Real x);
@@ -91,7 +116,7 @@ __device__ __forceinline__ void pp_term(Real px, Real py, Real pz, const typenam
     acc[0] = fma(mr3, dx, acc[0]);
     acc[1] = fma(mr3, dy, acc[1]);
     acc[2] = fma(mr3, dz, acc[2]);
-    acc[3] -= mr;
+    acc[3] = fma(-s.w, rinv, acc[3]);  // explicit: every kernel rounds it alike
 }
 
 // PC: y = r_i - R, r_s^2 = |y|^2 + eps^2;
@@ -126,7 +151,7 @@ __device__ __forceinline__ void pc_term(Real px, Real py, Real pz, const typenam
         acc[0] = fma(-Mr3, yx, acc[0]);
         acc[1] = fma(-Mr3, yy, acc[1]);
         acc[2] = fma(-Mr3, yz, acc[2]);
-        acc[3] -= Mr;
+        acc[3] = fma(-A.w, rinv, acc[3]);
     }
 }
 
@@ -249,8 +274,250 @@ __device__ __forceinline__ uint32_t warp_incl_scan(uint32_t v, int lane) {
     return v;
 }
 
+// --- evaluation of one tile (whole warp) -----------------------------------
+// A warp's targets: its group's particles, lane l holding l (and l + 32).
+template <typename Real, int TPL>
+struct Targets {
+    Real px[TPL], py[TPL], pz[TPL];
+    float2 nX[TPL], nY[TPL], nZ[TPL];  // negated and duplicated (packed FP32 terms)
+    __device__ __forceinline__ void set_packed() {
+#pragma unroll
+        for (int t = 0; t < TPL; ++t) {
+            nX[t] = make_float2(-(float)px[t], -(float)px[t]);
+            nY[t] = make_float2(-(float)py[t], -(float)py[t]);
+            nZ[t] = make_float2(-(float)pz[t], -(float)pz[t]);
+        }
+    }
+};
+
+// A warp's staging area.  FP32: sources are staged as pairs, pair k in
+// F[5k .. 5k+4]:
+//   PP: (x0, x1, y0, y1), (z0, z1, m0, m1)
+//   PC: (Rx0, Rx1, Ry0, Ry1), (Rz0, Rz1, M0, M1), -(Qxx, Qyy), -(Qzz, Qxy), -(Qxz, Qyz)
+// with an odd count padded by a massless source at the origin.  FP64: A, B, C
+// one record per source.
+template <typename Real>
+struct Stage {
+    float4 *F;
+    typename Vec4<Real>::T *A, *B;
+    typename Vec2<Real>::T *C;
+    uint32_t *sidx;  // sorted index of each staged near source
+    __device__ __forceinline__ Stage(unsigned char *wb, uint32_t *si) : sidx(si) {
+        F = reinterpret_cast<float4 *>(wb);
+        A = reinterpret_cast<typename Vec4<Real>::T *>(wb);
+        B = A + 32;
+        C = reinterpret_cast<typename Vec2<Real>::T *>(B + 32);
+    }
+};
+
+// Stages ns near sources (lane l: src, sorted index si); true when some of
+// them is one of the group's own particles [s0, s0 + cnt).
+template <typename Real>
+__device__ __forceinline__ bool stage_pp(const Stage<Real> &S, int lane, const typename Vec4<Real>::T &src,
+                                         uint32_t si, int ns, uint32_t s0, int cnt) {
+    S.sidx[lane] = lane < ns ? si : 0xffffffffu;
+    const bool own = __any_sync(0xffffffffu, lane < ns && si - s0 < (uint32_t)cnt);
+    if constexpr (sizeof(Real) == 4) {
+        const int ne = (ns + 1) & ~1;
+        if (lane < ne) {
+            float *a = reinterpret_cast<float *>(S.F + 5 * (lane >> 1));
+            const int sl = lane & 1;
+            const bool v = lane < ns;
+            a[sl] = v ? (float)src.x : 0.f;
+            a[2 + sl] = v ? (float)src.y : 0.f;
+            a[4 + sl] = v ? (float)src.z : 0.f;
+            a[6 + sl] = v ? (float)src.w : 0.f;
+        }
+    } else {
+        if (lane < ns) S.A[lane] = src;
+    }
+    return own;
+}
+
+// Partial sums of the staged near sources.  UNROLL: the full tile's loop.
+template <typename Real, int TPL, bool SOFT, int UNROLL>
+__device__ __forceinline__ void part_pp(const Stage<Real> &S, const Targets<Real, TPL> &T, int lane, int ns, bool own,
+                                        uint32_t s0, Real eps2, float2 eps2v, Real (&p1)[TPL][4]) {
+    using V4 = typename Vec4<Real>::T;
+    if constexpr (sizeof(Real) == 4) {
+        const float2 neg1 = make_float2(-1.f, -1.f);
+        const float4 *stF = S.F;
+        const uint32_t *sidx = S.sidx;
+        float2 part[TPL][4];
+#pragma unroll
+        for (int t = 0; t < TPL; ++t)
+#pragma unroll
+            for (int c = 0; c < 4; ++c) part[t][c] = make_float2(0.f, 0.f);
+        const int np = (ns + 1) >> 1;
+        if (own) {
+            // the group's own particles are in this tile: each lane drops its own index
+            for (int k = 0; k < np; ++k) {
+                const float4 a = stF[5 * k], b = stF[5 * k + 1];
+                const uint32_t i0 = sidx[2 * k], i1 = sidx[2 * k + 1];
+#pragma unroll
+                for (int t = 0; t < TPL; ++t) {
+                    const uint32_t me = s0 + (uint32_t)(lane + 32 * t);
+                    const float2 mm = make_float2(i0 == me ? 0.f : b.z, i1 == me ? 0.f : b.w);
+                    pp_pair<SOFT>(T.nX[t], T.nY[t], T.nZ[t], make_float2(a.x, a.y), make_float2(a.z, a.w),
+                                  make_float2(b.x, b.y), mm, eps2v, neg1, part[t]);
+                }
+            }
+        } else if (np == 16) {
+#pragma unroll UNROLL
+            for (int k = 0; k < 16; ++k) {
+                const float4 a = stF[5 * k], b = stF[5 * k + 1];
+#pragma unroll
+                for (int t = 0; t < TPL; ++t)
+                    pp_pair<SOFT>(T.nX[t], T.nY[t], T.nZ[t], make_float2(a.x, a.y), make_float2(a.z, a.w),
+                                  make_float2(b.x, b.y), make_float2(b.z, b.w), eps2v, neg1, part[t]);
+            }
+        } else {
+            for (int k = 0; k < np; ++k) {
+                const float4 a = stF[5 * k], b = stF[5 * k + 1];
+#pragma unroll
+                for (int t = 0; t < TPL; ++t)
+                    pp_pair<SOFT>(T.nX[t], T.nY[t], T.nZ[t], make_float2(a.x, a.y), make_float2(a.z, a.w),
+                                  make_float2(b.x, b.y), make_float2(b.z, b.w), eps2v, neg1, part[t]);
+            }
+        }
+#pragma unroll
+        for (int t = 0; t < TPL; ++t)
+#pragma unroll
+            for (int c = 0; c < 4; ++c) p1[t][c] = (Real)(part[t][c].x + part[t][c].y);
+    } else {
+#pragma unroll
+        for (int t = 0; t < TPL; ++t)
+#pragma unroll
+            for (int c = 0; c < 4; ++c) p1[t][c] = Real(0);
+        for (int j = 0; j < ns; ++j) {
+            const V4 s = S.A[j];
+            const uint32_t sj = S.sidx[j];
+#pragma unroll
+            for (int t = 0; t < TPL; ++t) {
+                V4 st = s;
+                if (own && sj == s0 + (uint32_t)(lane + 32 * t)) st.w = Real(0);
+                pp_term<Real, SOFT>(T.px[t], T.py[t], T.pz[t], st, eps2, p1[t]);
+            }
+        }
+    }
+}
+
+// Stages ns far cells (lane l: cell index `cell`).
+template <typename Real, bool QUAD>
+__device__ __forceinline__ void stage_pc(const Stage<Real> &S, int lane, uint32_t cell, int ns,
+                                         const typename Vec4<Real>::T *__restrict__ momA,
+                                         const typename Vec4<Real>::T *__restrict__ momB,
+                                         const typename Vec2<Real>::T *__restrict__ momC) {
+    using V4 = typename Vec4<Real>::T;
+    using V2 = typename Vec2<Real>::T;
+    if constexpr (sizeof(Real) == 4) {
+        const int ne = (ns + 1) & ~1;
+        if (lane < ne) {
+            float *q = reinterpret_cast<float *>(S.F + 5 * (lane >> 1));
+            const int sl = lane & 1;
+            V4 a{};
+            V4 b{};
+            V2 c{};
+            if (lane < ns) {
+                a = momA[cell];
+                if (QUAD) { b = momB[cell]; c = momC[cell]; }
+            }
+            q[sl] = a.x; q[2 + sl] = a.y; q[4 + sl] = a.z; q[6 + sl] = a.w;
+            if (QUAD) {  // the FP32 cell copies already hold -Q
+                q[8 + sl] = b.x; q[10 + sl] = b.y; q[12 + sl] = b.z; q[14 + sl] = b.w;
+                q[16 + sl] = c.x; q[18 + sl] = c.y;
+            }
+        }
+    } else {
+        if (lane < ns) {
+            S.A[lane] = momA[cell];
+            if (QUAD) { S.B[lane] = momB[cell]; S.C[lane] = momC[cell]; }
+        }
+    }
+}
+
+// Partial sums of the staged far cells; r5: a full tile takes the r^-5 form.
+template <typename Real, int TPL, bool QUAD, bool SOFT, int UNROLL5, int UNROLL>
+__device__ __forceinline__ void part_pc(const Stage<Real> &S, const Targets<Real, TPL> &T, int ns, bool r5, Real eps2,
+                                        float2 eps2v, Real (&p1)[TPL][4]) {
+    using V4 = typename Vec4<Real>::T;
+    using V2 = typename Vec2<Real>::T;
+    if constexpr (sizeof(Real) == 4) {
+        const float2 neg1 = make_float2(-1.f, -1.f), halfv = make_float2(0.5f, 0.5f), m25 = make_float2(-2.5f, -2.5f),
+                     mhalf = make_float2(-0.5f, -0.5f);
+        const float4 *stF = S.F;
+        float2 part[TPL][4];
+#pragma unroll
+        for (int t = 0; t < TPL; ++t)
+#pragma unroll
+            for (int c = 0; c < 4; ++c) part[t][c] = make_float2(0.f, 0.f);
+        const int np = (ns + 1) >> 1;
+        const float4 z4 = make_float4(0.f, 0.f, 0.f, 0.f);
+        const bool tile_r5 = np == 16 && r5;  // part[t][3] then holds -phi
+        if (tile_r5) {
+#pragma unroll UNROLL5
+            for (int k = 0; k < 16; ++k) {
+                const float4 a = stF[5 * k], b = stF[5 * k + 1];
+                const float4 c = stF[5 * k + 2], d = stF[5 * k + 3], e = stF[5 * k + 4];
+#pragma unroll
+                for (int t = 0; t < TPL; ++t)
+                    pc_pair<QUAD, SOFT, true>(T.nX[t], T.nY[t], T.nZ[t], a, b, c, d, e, eps2v, mhalf, halfv, m25,
+                                              part[t]);
+            }
+        } else if (np == 16) {
+#pragma unroll UNROLL
+            for (int k = 0; k < 16; ++k) {
+                const float4 a = stF[5 * k], b = stF[5 * k + 1];
+                const float4 c = QUAD ? stF[5 * k + 2] : z4, d = QUAD ? stF[5 * k + 3] : z4,
+                             e = QUAD ? stF[5 * k + 4] : z4;
+#pragma unroll
+                for (int t = 0; t < TPL; ++t)
+                    pc_pair<QUAD, SOFT>(T.nX[t], T.nY[t], T.nZ[t], a, b, c, d, e, eps2v, neg1, halfv, m25, part[t]);
+            }
+        } else {
+            for (int k = 0; k < np; ++k) {
+                const float4 a = stF[5 * k], b = stF[5 * k + 1];
+                const float4 c = QUAD ? stF[5 * k + 2] : z4, d = QUAD ? stF[5 * k + 3] : z4,
+                             e = QUAD ? stF[5 * k + 4] : z4;
+#pragma unroll
+                for (int t = 0; t < TPL; ++t)
+                    pc_pair<QUAD, SOFT>(T.nX[t], T.nY[t], T.nZ[t], a, b, c, d, e, eps2v, neg1, halfv, m25, part[t]);
+            }
+        }
+#pragma unroll
+        for (int t = 0; t < TPL; ++t) {
+#pragma unroll
+            for (int c = 0; c < 4; ++c) p1[t][c] = (Real)(part[t][c].x + part[t][c].y);
+            if (tile_r5) p1[t][3] = -p1[t][3];
+        }
+    } else {
+#pragma unroll
+        for (int t = 0; t < TPL; ++t)
+#pragma unroll
+            for (int c = 0; c < 4; ++c) p1[t][c] = Real(0);
+        V4 b0{};
+        V2 c0{};
+        for (int j = 0; j < ns; ++j) {
+            const V4 a = S.A[j];
+            const V4 b = QUAD ? S.B[j] : b0;
+            const V2 c = QUAD ? S.C[j] : c0;
+#pragma unroll
+            for (int t = 0; t < TPL; ++t)
+                pc_term<Real, QUAD, SOFT>(T.px[t], T.py[t], T.pz[t], a, b, c, eps2, p1[t]);
+        }
+    }
+}
+
+// Resident blocks per SM the registers are held to.  kWalkFold keeps two
+// batches of partial sums in registers (the fold of the longest group is a
+// chain of loads: 65 us at N = 16384 with one batch that spilled, 20 with two
+// that fit) and runs few groups: 3 blocks.
+constexpr int walk_blocks(int mode, int tpl, size_t real) {
+    return mode == kWalkFold ? 3 : tpl == 2 ? 4 : real == 4 ? 6 : 5;
+}
+
 template <typename Real, int TPL, bool QUAD, bool KAHAN, bool SOFT, int MODE>
-__global__ void __launch_bounds__(kWalkWarps * 32, TPL == 2 ? 4 : sizeof(Real) == 4 ? 6 : 5) k_walk(const WalkArgs A) {
+__global__ void __launch_bounds__(kWalkWarps * 32, walk_blocks(MODE, TPL, sizeof(Real))) k_walk(const WalkArgs A) {
     using V4 = typename Vec4<Real>::T;
     using V2 = typename Vec2<Real>::T;
     extern __shared__ __align__(32) unsigned char smem[];
@@ -262,14 +529,10 @@ __global__ void __launch_bounds__(kWalkWarps * 32, TPL == 2 ? 4 : sizeof(Real) =
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int SD = A.stack_depth;
     unsigned char *wb = smem + (size_t)warp * walk_warp_bytes<Real>(SD);
-    V4 *stA = reinterpret_cast<V4 *>(wb);            // FP64 layout
-    V4 *stB = stA + 32;
-    V2 *stC = reinterpret_cast<V2 *>(stB + 32);
-    float4 *stF = reinterpret_cast<float4 *>(wb);    // FP32 pair-interleaved layout
     uint32_t *stack = reinterpret_cast<uint32_t *>(wb + walk_stage_bytes<Real>());
     uint32_t *ppbuf = stack + SD;
     uint32_t *pcbuf = ppbuf + kPPCap;
-    uint32_t *sidx = pcbuf + kPCCap;  // sorted index of each staged near source
+    const Stage<Real> S(wb, pcbuf + kPCCap);
     const uint32_t lt = lanemask_lt();
 
     const V4 *__restrict__ spos = reinterpret_cast<const V4 *>(A.spos);
@@ -281,6 +544,8 @@ __global__ void __launch_bounds__(kWalkWarps * 32, TPL == 2 ? 4 : sizeof(Real) =
     // full far-cell tiles of one-target-per-lane groups take pc_pair's R5 form
     // where it fits the segment's cube (flag set per segment after the moments)
     constexpr bool kR5 = sizeof(Real) == 4 && QUAD && TPL == 1;
+    // tiles are filled and consumed (evaluated or emitted)
+    constexpr bool kTiles = MODE == kWalkForce || MODE == kWalkFold || MODE == kWalkTiles;
 
     // persistent warps: each takes the next group slot until all are done
     const uint32_t ngroups = A.ctr[kCtrGroups];
@@ -296,15 +561,15 @@ __global__ void __launch_bounds__(kWalkWarps * 32, TPL == 2 ? 4 : sizeof(Real) =
     const uint32_t gseg = A.nseg > 1 ? seg_find(A.seg_off, A.nseg, s0) : 0u;
 
     // targets and the group's integer box
-    Real px[TPL], py[TPL], pz[TPL], pm[TPL];
+    Targets<Real, TPL> T;
     uint32_t lo0 = 0xffffffffu, lo1 = 0xffffffffu, lo2 = 0xffffffffu, hi0 = 0, hi1 = 0, hi2 = 0;
 #pragma unroll
     for (int t = 0; t < TPL; ++t) {
         const int li = lane + 32 * t;
-        px[t] = py[t] = pz[t] = pm[t] = Real(0);
+        T.px[t] = T.py[t] = T.pz[t] = Real(0);
         if (li < cnt) {
             const V4 p = spos[s0 + li];
-            px[t] = p.x; py[t] = p.y; pz[t] = p.z; pm[t] = p.w;
+            T.px[t] = p.x; T.py[t] = p.y; T.pz[t] = p.z;
             const uint64_t k = A.skey[s0 + li];
             const uint32_t qx = compact3(k >> 2), qy = compact3(k >> 1), qz = compact3(k);
             lo0 = min(lo0, qx); lo1 = min(lo1, qy); lo2 = min(lo2, qz);
@@ -322,221 +587,65 @@ __global__ void __launch_bounds__(kWalkWarps * 32, TPL == 2 ? 4 : sizeof(Real) =
 #pragma unroll
         for (int c = 0; c < 4; ++c) { sum[t][c] = Real(0); cmp[t][c] = Real(0); }
 
-    // --- evaluation helpers (whole warp) ---
-    // FP32: sources are staged as pairs, pair k in stF[5k .. 5k+4]:
-    //   PP: (x0, x1, y0, y1), (z0, z1, m0, m1)
-    //   PC: (Rx0, Rx1, Ry0, Ry1), (Rz0, Rz1, M0, M1), -(Qxx, Qyy), -(Qzz, Qxy), -(Qxz, Qyz)
-    // with an odd count padded by a massless source at the origin.
-    float2 nX[TPL], nY[TPL], nZ[TPL];
-#pragma unroll
-    for (int t = 0; t < TPL; ++t) {
-        nX[t] = make_float2(-(float)px[t], -(float)px[t]);
-        nY[t] = make_float2(-(float)py[t], -(float)py[t]);
-        nZ[t] = make_float2(-(float)pz[t], -(float)pz[t]);
-    }
+    T.set_packed();
     const float2 eps2v = make_float2((float)A.eps2, (float)A.eps2);
-    const float2 neg1 = make_float2(-1.f, -1.f), halfv = make_float2(0.5f, 0.5f), m25 = make_float2(-2.5f, -2.5f),
-                 mhalf = make_float2(-0.5f, -0.5f);
     const bool r5 = kR5 && A.box[gseg].r5fit != 0;
 
-    // true when some staged source is one of the group's own particles
-    auto stage_pp = [&](const V4 &src, uint32_t si, int ns) -> bool {
-        sidx[lane] = lane < ns ? si : 0xffffffffu;
-        const bool own = __any_sync(0xffffffffu, lane < ns && si - (uint32_t)s0 < (uint32_t)cnt);
-        if constexpr (sizeof(Real) == 4) {
-            const int ne = (ns + 1) & ~1;
-            if (lane < ne) {
-                float *a = reinterpret_cast<float *>(stF + 5 * (lane >> 1));
-                const int sl = lane & 1;
-                const bool v = lane < ns;
-                a[sl] = v ? (float)src.x : 0.f;
-                a[2 + sl] = v ? (float)src.y : 0.f;
-                a[4 + sl] = v ? (float)src.z : 0.f;
-                a[6 + sl] = v ? (float)src.w : 0.f;
-            }
-        } else {
-            if (lane < ns) stA[lane] = src;
-        }
-        return own;
+    // --- evaluation (whole warp) ---
+    auto fold_tile = [&](const Real(&p1)[TPL][4]) {
+#pragma unroll
+        for (int t = 0; t < TPL; ++t) fold<Real, KAHAN>(sum[t], cmp[t], p1[t]);
     };
-    auto eval_pp_stage = [&](int ns, bool own) {
-        if constexpr (sizeof(Real) == 4) {
-            float2 part[TPL][4];
-#pragma unroll
-            for (int t = 0; t < TPL; ++t)
-#pragma unroll
-                for (int c = 0; c < 4; ++c) part[t][c] = make_float2(0.f, 0.f);
-            const int np = (ns + 1) >> 1;
-            if (own) {
-                // the group's own particles are in this tile: each lane drops its own index
-                for (int k = 0; k < np; ++k) {
-                    const float4 a = stF[5 * k], b = stF[5 * k + 1];
-                    const uint32_t i0 = sidx[2 * k], i1 = sidx[2 * k + 1];
-#pragma unroll
-                    for (int t = 0; t < TPL; ++t) {
-                        const uint32_t me = (uint32_t)s0 + (uint32_t)(lane + 32 * t);
-                        const float2 mm = make_float2(i0 == me ? 0.f : b.z, i1 == me ? 0.f : b.w);
-                        pp_pair<SOFT>(nX[t], nY[t], nZ[t], make_float2(a.x, a.y), make_float2(a.z, a.w),
-                                      make_float2(b.x, b.y), mm, eps2v, neg1, part[t]);
-                    }
-                }
-            } else if (np == 16) {
-#pragma unroll 16
-                for (int k = 0; k < 16; ++k) {
-                    const float4 a = stF[5 * k], b = stF[5 * k + 1];
-#pragma unroll
-                    for (int t = 0; t < TPL; ++t)
-                        pp_pair<SOFT>(nX[t], nY[t], nZ[t], make_float2(a.x, a.y), make_float2(a.z, a.w),
-                                      make_float2(b.x, b.y), make_float2(b.z, b.w), eps2v, neg1, part[t]);
-                }
-            } else {
-                for (int k = 0; k < np; ++k) {
-                    const float4 a = stF[5 * k], b = stF[5 * k + 1];
-#pragma unroll
-                    for (int t = 0; t < TPL; ++t)
-                        pp_pair<SOFT>(nX[t], nY[t], nZ[t], make_float2(a.x, a.y), make_float2(a.z, a.w),
-                                      make_float2(b.x, b.y), make_float2(b.z, b.w), eps2v, neg1, part[t]);
-                }
-            }
-#pragma unroll
-            for (int t = 0; t < TPL; ++t) {
-                Real p1[4];
-#pragma unroll
-                for (int c = 0; c < 4; ++c) p1[c] = (Real)(part[t][c].x + part[t][c].y);
-                fold<Real, KAHAN>(sum[t], cmp[t], p1);
-            }
-        } else {
-            Real part[TPL][4];
-#pragma unroll
-            for (int t = 0; t < TPL; ++t)
-#pragma unroll
-                for (int c = 0; c < 4; ++c) part[t][c] = Real(0);
-            for (int j = 0; j < ns; ++j) {
-                const V4 s = stA[j];
-                const uint32_t sj = sidx[j];
-#pragma unroll
-                for (int t = 0; t < TPL; ++t) {
-                    V4 st = s;
-                    if (own && sj == (uint32_t)s0 + (uint32_t)(lane + 32 * t)) st.w = Real(0);
-                    pp_term<Real, SOFT>(px[t], py[t], pz[t], st, eps2, part[t]);
-                }
-            }
-#pragma unroll
-            for (int t = 0; t < TPL; ++t) fold<Real, KAHAN>(sum[t], cmp[t], part[t]);
-        }
-    };
-    auto eval_pp_list = [&](const uint32_t *buf, int ns) {
+    auto eval_pp = [&](uint32_t si, int ns) {
         V4 s{};
-        uint32_t si = 0xffffffffu;
-        if (lane < ns) { si = buf[lane]; s = spos[si]; }
+        if (lane < ns) s = spos[si];
         __syncwarp();
-        const bool own = stage_pp(s, si, ns);
+        const bool own = stage_pp<Real>(S, lane, s, si, ns, (uint32_t)s0, cnt);
         __syncwarp();
-        eval_pp_stage(ns, own);
-        __syncwarp();
-    };
-    auto eval_pp_range = [&](uint32_t first, int ns) {
-        V4 s{};
-        if (lane < ns) s = spos[first + lane];
-        __syncwarp();
-        const bool own = stage_pp(s, first + (uint32_t)lane, ns);
-        __syncwarp();
-        eval_pp_stage(ns, own);
+        Real p1[TPL][4];
+        part_pp<Real, TPL, SOFT, 16>(S, T, lane, ns, own, (uint32_t)s0, eps2, eps2v, p1);
+        fold_tile(p1);
         __syncwarp();
     };
-    auto eval_pc_list = [&](const uint32_t *buf, int ns) {
-        if constexpr (sizeof(Real) == 4) {
-            const int ne = (ns + 1) & ~1;
-            if (lane < ne) {
-                float *q = reinterpret_cast<float *>(stF + 5 * (lane >> 1));
-                const int sl = lane & 1;
-                V4 a{};
-                V4 b{};
-                V2 c{};
-                if (lane < ns) {
-                    const uint32_t cell = buf[lane];
-                    a = momA[cell];
-                    if (QUAD) { b = momB[cell]; c = momC[cell]; }
-                }
-                q[sl] = a.x; q[2 + sl] = a.y; q[4 + sl] = a.z; q[6 + sl] = a.w;
-                if (QUAD) {  // the FP32 cell copies already hold -Q
-                    q[8 + sl] = b.x; q[10 + sl] = b.y; q[12 + sl] = b.z; q[14 + sl] = b.w;
-                    q[16 + sl] = c.x; q[18 + sl] = c.y;
-                }
+    auto eval_pc = [&](const uint32_t *buf, int ns) {
+        stage_pc<Real, QUAD>(S, lane, lane < ns ? buf[lane] : 0u, ns, momA, momB, momC);
+        __syncwarp();
+        Real p1[TPL][4];
+        part_pc<Real, TPL, QUAD, SOFT, 16, 4>(S, T, ns, r5, eps2, eps2v, p1);
+        fold_tile(p1);
+        __syncwarp();
+    };
+    // --- split walk: the same tiles, in the same order, into tile slots ---
+    // (a chunk is asked for half a chunk before it is needed, so that the
+    // atomic's latency passes behind the tiles in between)
+    uint32_t ntile = 0, tbase = 0, tnext = 0;
+    bool full = false;  // out of slots: kWalkFold walks this group itself
+    if (MODE == kWalkTiles && lane == 0) tnext = atomicAdd(A.ctr + kCtrTiles, (uint32_t)kTileChunk);
+    auto emit_tile = [&](uint32_t src, int ns, uint32_t far) {
+        if (full) return;
+        if ((ntile & (kTileChunk - 1)) == 0) {
+            const uint32_t base = __shfl_sync(0xffffffffu, tnext, 0);
+            if (base > A.tile_cap - kTileChunk) { full = true; return; }
+            if (lane == 0) {
+                if (ntile == 0) A.ghead[g] = base;
+                else A.tile_next[tbase / kTileChunk] = base;
             }
-            __syncwarp();
-            float2 part[TPL][4];
-#pragma unroll
-            for (int t = 0; t < TPL; ++t)
-#pragma unroll
-                for (int c = 0; c < 4; ++c) part[t][c] = make_float2(0.f, 0.f);
-            const int np = (ns + 1) >> 1;
-            const float4 z4 = make_float4(0.f, 0.f, 0.f, 0.f);
-            const bool tile_r5 = np == 16 && r5;  // part[t][3] then holds -phi
-            if (tile_r5) {
-#pragma unroll 16
-                for (int k = 0; k < 16; ++k) {
-                    const float4 a = stF[5 * k], b = stF[5 * k + 1];
-                    const float4 c = stF[5 * k + 2], d = stF[5 * k + 3], e = stF[5 * k + 4];
-#pragma unroll
-                    for (int t = 0; t < TPL; ++t)
-                        pc_pair<QUAD, SOFT, true>(nX[t], nY[t], nZ[t], a, b, c, d, e, eps2v, mhalf, halfv, m25,
-                                                  part[t]);
-                }
-            } else if (np == 16) {
-#pragma unroll 4
-                for (int k = 0; k < 16; ++k) {
-                    const float4 a = stF[5 * k], b = stF[5 * k + 1];
-                    const float4 c = QUAD ? stF[5 * k + 2] : z4, d = QUAD ? stF[5 * k + 3] : z4,
-                                 e = QUAD ? stF[5 * k + 4] : z4;
-#pragma unroll
-                    for (int t = 0; t < TPL; ++t)
-                        pc_pair<QUAD, SOFT>(nX[t], nY[t], nZ[t], a, b, c, d, e, eps2v, neg1, halfv, m25, part[t]);
-                }
-            } else {
-                for (int k = 0; k < np; ++k) {
-                    const float4 a = stF[5 * k], b = stF[5 * k + 1];
-                    const float4 c = QUAD ? stF[5 * k + 2] : z4, d = QUAD ? stF[5 * k + 3] : z4,
-                                 e = QUAD ? stF[5 * k + 4] : z4;
-#pragma unroll
-                    for (int t = 0; t < TPL; ++t)
-                        pc_pair<QUAD, SOFT>(nX[t], nY[t], nZ[t], a, b, c, d, e, eps2v, neg1, halfv, m25, part[t]);
-                }
-            }
-#pragma unroll
-            for (int t = 0; t < TPL; ++t) {
-                Real p1[4];
-#pragma unroll
-                for (int c = 0; c < 4; ++c) p1[c] = (Real)(part[t][c].x + part[t][c].y);
-                if (tile_r5) p1[3] = -p1[3];
-                fold<Real, KAHAN>(sum[t], cmp[t], p1);
-            }
-            __syncwarp();
-        } else {
-            if (lane < ns) {
-                const uint32_t c = buf[lane];
-                stA[lane] = momA[c];
-                if (QUAD) { stB[lane] = momB[c]; stC[lane] = momC[c]; }
-            }
-            __syncwarp();
-            Real part[TPL][4];
-#pragma unroll
-            for (int t = 0; t < TPL; ++t)
-#pragma unroll
-                for (int c = 0; c < 4; ++c) part[t][c] = Real(0);
-            V4 b0{};
-            V2 c0{};
-            for (int j = 0; j < ns; ++j) {
-                const V4 a = stA[j];
-                const V4 b = QUAD ? stB[j] : b0;
-                const V2 c = QUAD ? stC[j] : c0;
-#pragma unroll
-                for (int t = 0; t < TPL; ++t) pc_term<Real, QUAD, SOFT>(px[t], py[t], pz[t], a, b, c, eps2, part[t]);
-            }
-#pragma unroll
-            for (int t = 0; t < TPL; ++t) fold<Real, KAHAN>(sum[t], cmp[t], part[t]);
-            __syncwarp();
+            tbase = base;
         }
+        const uint32_t slot = tbase + (ntile & (kTileChunk - 1));
+        if ((ntile & (kTileChunk - 1)) == kTileChunk / 2 && lane == 0)
+            tnext = atomicAdd(A.ctr + kCtrTiles, (uint32_t)kTileChunk);
+        if (lane == 0) A.tile_hdr[slot] = make_uint2((uint32_t)g, (uint32_t)ns | (far << 8));
+        A.tile_idx[(size_t)slot * 32 + lane] = lane < ns ? src : 0u;
+        ++ntile;
+    };
+    auto pc_tile = [&](const uint32_t *buf, int ns) {
+        if (MODE == kWalkTiles) emit_tile(lane < ns ? buf[lane] : 0u, ns, 1u);
+        else eval_pc(buf, ns);
+    };
+    auto pp_tile = [&](uint32_t si, int ns) {
+        if (MODE == kWalkTiles) emit_tile(si, ns, 0u);
+        else eval_pp(si, ns);
     };
 
     // --- traversal ---
@@ -547,12 +656,62 @@ __global__ void __launch_bounds__(kWalkWarps * 32, TPL == 2 ? 4 : sizeof(Real) =
     }
     uint32_t n_pc = 0, n_pp = 0, n_ppl = 0, max_top = 1;
     int top = 1, npc = 0, npp = 0;
+    bool folded = false;
+    if (MODE == kWalkFold) {
+        // the group's tiles have been evaluated: fold their partial sums in the
+        // order in which the one-warp walk would have evaluated them
+        const uint32_t nt = A.gtiles[g];
+        folded = nt != kTilesFull;
+        if (folded) {
+            const V4 *__restrict__ tp = reinterpret_cast<const V4 *>(A.tile_part);
+            // two batches of 32 registers: one is folded while the next is loaded
+            constexpr int kB = 128 / (int)(sizeof(V4) * TPL);
+            static_assert(kTileChunk % kB == 0, "a batch stays inside one chunk");
+            V4 q[kB][TPL], r[kB][TPL];
+            uint32_t base = nt ? A.ghead[g] : 0u;
+            uint32_t next = nt > kTileChunk ? A.tile_next[base / kTileChunk] : 0u;
+            auto load = [&](V4(&d)[kB][TPL], uint32_t b) {
+                if (b >= nt) return;
+                if (b != 0 && (b & (kTileChunk - 1)) == 0) {
+                    base = next;
+                    next = b + kTileChunk < nt ? A.tile_next[base / kTileChunk] : 0u;
+                }
+#pragma unroll
+                for (int k = 0; k < kB; ++k)
+#pragma unroll
+                    for (int t = 0; t < TPL; ++t)
+                        if (b + k < nt) d[k][t] = tp[((size_t)(base + (b & (kTileChunk - 1)) + k) * TPL + t) * 32 + lane];
+            };
+            auto fold_batch = [&](const V4(&d)[kB][TPL], uint32_t b) {
+#pragma unroll
+                for (int k = 0; k < kB; ++k) {
+                    if (b + k >= nt) break;
+                    Real p1[TPL][4];
+#pragma unroll
+                    for (int t = 0; t < TPL; ++t) {
+                        p1[t][0] = d[k][t].x; p1[t][1] = d[k][t].y;
+                        p1[t][2] = d[k][t].z; p1[t][3] = d[k][t].w;
+                    }
+                    fold_tile(p1);
+                }
+            };
+            load(q, 0);
+#pragma unroll 1
+            for (uint32_t b = 0; b < nt; b += 2 * kB) {
+                load(r, b + kB);
+                fold_batch(q, b);
+                load(q, b + 2 * kB);
+                fold_batch(r, b + kB);
+            }
+            top = 0;  // nothing left to walk
+        }
+    }
     // Stack entries are child ranges: first node | (count - 1) << 29.
     // the root of the group's segment (node b at level 0): range (node b, 1 node)
     if (lane == 0) stack[0] = gseg;
     __syncwarp();
     bool overflow = false;
-    while (top > 0) {
+    while (top > 0 && !(MODE == kWalkTiles && full)) {
         // pop up to 32 nodes from the top ranges; the last range may be split
         const int nr = top < 32 ? top : 32;
         uint32_t e = 0, sz = 0;
@@ -604,7 +763,7 @@ __global__ void __launch_bounds__(kWalkWarps * 32, TPL == 2 ? 4 : sizeof(Real) =
         // far cells
         const uint32_t fm = __ballot_sync(0xffffffffu, far);
         const uint32_t nf = __popc(fm);
-        if (MODE == kWalkForce) {
+        if (kTiles) {
             if (far) pcbuf[npc + __popc(fm & lt)] = node;
             npc += nf;
         } else if (MODE == kWalkEmit) {
@@ -616,7 +775,7 @@ __global__ void __launch_bounds__(kWalkWarps * 32, TPL == 2 ? 4 : sizeof(Real) =
             const uint32_t cc = allfar ? lk.y : 0u;
             const uint32_t incl = warp_incl_scan(cc, lane);
             const uint32_t tot = __shfl_sync(0xffffffffu, incl, 31);
-            if (MODE == kWalkForce) {
+            if (kTiles) {
                 if (allfar)
                     for (uint32_t c = 0; c < cc; ++c) pcbuf[npc + (incl - cc) + c] = lk.x + c;
                 npc += (int)tot;
@@ -654,7 +813,7 @@ __global__ void __launch_bounds__(kWalkWarps * 32, TPL == 2 ? 4 : sizeof(Real) =
             const uint32_t incl2 = warp_incl_scan(sc, lane);
             const uint32_t tot2 = __shfl_sync(0xffffffffu, incl2, 31);
             n_pp += __reduce_add_sync(0xffffffffu, lc);
-            if (MODE == kWalkForce) {
+            if (kTiles) {
                 if (nleaf && !big)
                     for (uint32_t c = 0; c < lc; ++c) ppbuf[npp + (incl2 - lc) + c] = lk.x + c;
                 npp += (int)tot2;
@@ -665,15 +824,15 @@ __global__ void __launch_bounds__(kWalkWarps * 32, TPL == 2 ? 4 : sizeof(Real) =
                     bm &= bm - 1;
                     const uint32_t f = __shfl_sync(0xffffffffu, lk.x, b);
                     const uint32_t c = __shfl_sync(0xffffffffu, lk.y, b);
-                    for (uint32_t o = 0; o < c; o += 32) eval_pp_range(f + o, (int)min(32u, c - o));
+                    for (uint32_t o = 0; o < c; o += 32) pp_tile(f + o + (uint32_t)lane, (int)min(32u, c - o));
                 }
             }
         }
-        if (MODE == kWalkForce) {
+        if (kTiles) {
             if (npc >= 32) {
                 __syncwarp();
                 const int ntile = npc >> 5;
-                for (int t = 0; t < ntile; ++t) eval_pc_list(pcbuf + 32 * t, 32);
+                for (int t = 0; t < ntile; ++t) pc_tile(pcbuf + 32 * t, 32);
                 const int r = npc & 31;
                 uint32_t t = lane < r ? pcbuf[32 * ntile + lane] : 0;
                 __syncwarp();
@@ -683,7 +842,7 @@ __global__ void __launch_bounds__(kWalkWarps * 32, TPL == 2 ? 4 : sizeof(Real) =
             }
             if (npp >= 32) {
                 const int ntile = npp >> 5;
-                for (int t = 0; t < ntile; ++t) eval_pp_list(ppbuf + 32 * t, 32);
+                for (int t = 0; t < ntile; ++t) pp_tile(ppbuf[32 * t + lane], 32);
                 const int r = npp & 31;
                 uint32_t t = lane < r ? ppbuf[32 * ntile + lane] : 0;
                 __syncwarp();
@@ -695,16 +854,25 @@ __global__ void __launch_bounds__(kWalkWarps * 32, TPL == 2 ? 4 : sizeof(Real) =
             __syncwarp();
         }
     }
-    if (MODE == kWalkForce) {
+    if (kTiles) {
         // every traversal step evaluates the whole tiles, so fewer than 32
         // entries are left here: the staging holds at most 32 sources
-        if (npc > 0) eval_pc_list(pcbuf, npc);
-        if (npp > 0) eval_pp_list(ppbuf, npp);
+        if (npc > 0) pc_tile(pcbuf, npc);
+        if (npp > 0) pp_tile(lane < npp ? ppbuf[lane] : 0xffffffffu, npp);
+    }
+    if (MODE == kWalkTiles) {
+        if (lane == 0) A.gtiles[g] = full ? kTilesFull : ntile;
+        // unused slots hold no sources: the rest of the last chunk, and a chunk asked for but not begun
+        const uint32_t used = ntile & (kTileChunk - 1);
+        const uint32_t ahead = __shfl_sync(0xffffffffu, tnext, 0);
+        if (used && lane >= (int)used && lane < kTileChunk) A.tile_hdr[tbase + lane] = make_uint2(0u, 0u);
+        if ((ntile == 0 || used == 0 || used > kTileChunk / 2) && ahead <= A.tile_cap - kTileChunk && lane < kTileChunk)
+            A.tile_hdr[ahead + lane] = make_uint2(0u, 0u);
     }
     if (overflow && lane == 0) set_status(A.dstatus, TREE_DEV_STACK);
-    if (lane == 0 && A.gstat) A.gstat[g] = make_uint4(n_pc, n_pp, max_top, n_ppl);
+    if (lane == 0 && A.gstat && !folded) A.gstat[g] = make_uint4(n_pc, n_pp, max_top, n_ppl);
 
-    if (MODE == kWalkForce) {
+    if (MODE == kWalkForce || MODE == kWalkFold) {
         const Real G = (Real)A.G;
 #pragma unroll
         for (int t = 0; t < TPL; ++t) {
@@ -740,9 +908,73 @@ __global__ void __launch_bounds__(kWalkWarps * 32, TPL == 2 ? 4 : sizeof(Real) =
     }  // group loop
 }
 
+// Split walk, second kernel: one warp per tile slot stages and evaluates the
+// slot's 32 sources for its group's targets and stores the partial sums.
+template <typename Real, int TPL, bool QUAD, bool SOFT>
+__global__ void __launch_bounds__(kWalkWarps * 32) k_eval_tiles(const WalkArgs A) {
+    using V4 = typename Vec4<Real>::T;
+    using V2 = typename Vec2<Real>::T;
+    __shared__ __align__(32) unsigned char s_stage[kWalkWarps][walk_stage_bytes<Real>()];
+    __shared__ uint32_t s_idx[kWalkWarps][32];
+    constexpr bool kR5 = sizeof(Real) == 4 && QUAD && TPL == 1;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    if (blockIdx.x == 0 && threadIdx.x == 0) A.ctr[kCtrWalkTicket] = 0;  // kWalkFold takes the groups again
+    if (aborted(A.ctr, kStageAfter)) return;
+    const Stage<Real> S(s_stage[warp], s_idx[warp]);
+    const V4 *__restrict__ spos = reinterpret_cast<const V4 *>(A.spos);
+    const V4 *__restrict__ momA = reinterpret_cast<const V4 *>(A.mom_a);
+    const V4 *__restrict__ momB = reinterpret_cast<const V4 *>(A.mom_b);
+    const V2 *__restrict__ momC = reinterpret_cast<const V2 *>(A.mom_c);
+    const Real eps2 = (Real)A.eps2;
+    const float2 eps2v = make_float2((float)A.eps2, (float)A.eps2);
+    const uint32_t total = min(A.ctr[kCtrTiles], A.tile_cap);
+    for (uint32_t slot = blockIdx.x * kWalkWarps + warp; slot < total; slot += gridDim.x * kWalkWarps) {
+        const uint2 h = A.tile_hdr[slot];
+        const uint32_t si = A.tile_idx[(size_t)slot * 32 + lane];
+        const int ns = (int)(h.y & 0xffu);
+        if (ns == 0) continue;
+        const uint32_t s0 = A.gfirst[h.x];
+        const int cnt = (int)(A.gfirst[h.x + 1] - s0);
+        Targets<Real, TPL> T;
+#pragma unroll
+        for (int t = 0; t < TPL; ++t) {
+            V4 p{};
+            if (lane + 32 * t < cnt) p = spos[s0 + lane + 32 * t];
+            T.px[t] = p.x; T.py[t] = p.y; T.pz[t] = p.z;
+        }
+        T.set_packed();
+        Real p1[TPL][4];
+        if (h.y >> 8) {
+            const bool r5 = kR5 && A.box[A.nseg > 1 ? seg_find(A.seg_off, A.nseg, s0) : 0u].r5fit != 0;
+            stage_pc<Real, QUAD>(S, lane, si, ns, momA, momB, momC);
+            __syncwarp();
+            part_pc<Real, TPL, QUAD, SOFT, 16, 4>(S, T, ns, r5, eps2, eps2v, p1);
+        } else {
+            V4 s{};
+            if (lane < ns) s = spos[si];
+            const bool own = stage_pp<Real>(S, lane, s, si, ns, s0, cnt);
+            __syncwarp();
+            part_pp<Real, TPL, SOFT, 16>(S, T, lane, ns, own, s0, eps2, eps2v, p1);
+        }
+        V4 *tp = reinterpret_cast<V4 *>(A.tile_part);
+#pragma unroll
+        for (int t = 0; t < TPL; ++t) {
+            V4 q;
+            q.x = p1[t][0]; q.y = p1[t][1]; q.z = p1[t][2]; q.w = p1[t][3];
+            tp[((size_t)slot * TPL + t) * 32 + lane] = q;
+        }
+        __syncwarp();
+    }
+}
+
 }  // namespace treegb
 
 namespace treegb {
+
+// The FP32 softened pair terms need eps^2 to be a normal FP32 number (see
+// rsqrt_pair); a smaller eps^2 takes the unsoftened variant, which still adds
+// it to r^2 and drops coincident pairs.
+inline bool walk_soft_f32(double eps) { return (float)(eps * eps) >= FLT_MIN; }
 
 // Host: walk arguments from the workspace.
 inline WalkArgs make_walk_args(TreeWorkspace *ws, const WalkOut &out) {
@@ -774,12 +1006,20 @@ inline WalkArgs make_walk_args(TreeWorkspace *ws, const WalkOut &out) {
     a.list_off = ws->list_cnt;
     a.pc_list = ws->pc_list;
     a.pp_list = ws->pp_list;
-    a.order = walk_widest_first(ws) ? ws->gorder : nullptr;
+    a.order = out.ordered ? ws->gorder : nullptr;
     a.gfirst = ws->gfirst;
     a.ctr = ws->ctr;
     a.seg_off = ws->seg_off;
     a.nseg = ws->nseg;
     a.box = ws->box;
+    a.tile_hdr = ws->tile_hdr;
+    a.tile_idx = ws->tile_idx;
+    a.tile_part = ws->tile_part;
+    a.tile_next = ws->tile_next;
+    // the partial sums of two targets per lane take twice the room
+    a.tile_cap = ws->p.group_size > 32 ? (ws->tile_cap / 2) & ~(uint32_t)(kTileChunk - 1) : ws->tile_cap;
+    a.ghead = ws->ghead;
+    a.gtiles = ws->gtiles;
     return a;
 }
 
@@ -800,11 +1040,26 @@ cudaError_t walk_run(TreeWorkspace *ws, const WalkArgs &a, cudaStream_t s) {
     int64_t nb = (int64_t)(per_sm > 0 ? per_sm : 1) * sms;
     if (nb > ng_bound) nb = ng_bound;
     if (nb < 1) nb = 1;
-    e = cudaMemsetAsync(ws->ctr + kCtrWalkTicket, 0, sizeof(uint32_t), s);
-    if (e != cudaSuccess) return e;
+    if (MODE != kWalkFold) {  // (k_eval_tiles has reset the ticket for kWalkFold)
+        e = cudaMemsetAsync(ws->ctr + kCtrWalkTicket, 0, 2 * sizeof(uint32_t), s);
+        if (e != cudaSuccess) return e;
+    }
     k<<<(unsigned)nb, kWalkWarps * 32, smem, s>>>(a);
     ws->launches += 1;
     return cudaGetLastError();
+}
+
+// The split walk: traversal into tile slots, evaluation of the slots, fold.
+template <typename Real, int TPL, bool QUAD, bool KAHAN, bool SOFT>
+cudaError_t walk_split(TreeWorkspace *ws, const WalkArgs &a, cudaStream_t s) {
+    cudaError_t e = walk_run<Real, TPL, false, false, true, kWalkTiles>(ws, a, s);
+    if (e != cudaSuccess || ws->n <= 0) return e;
+    auto k = k_eval_tiles<Real, TPL, QUAD, SOFT>;
+    k<<<wave_grid(k, (int64_t)ws->tile_cap * 32, kWalkWarps * 32, 1 << 20), kWalkWarps * 32, 0, s>>>(a);
+    ws->launches += 1;
+    e = cudaGetLastError();
+    if (e != cudaSuccess) return e;
+    return walk_run<Real, TPL, QUAD, KAHAN, SOFT, kWalkFold>(ws, a, s);
 }
 
 }  // namespace treegb
