@@ -78,7 +78,7 @@ void free_all(TreeWorkspace *ws) {
                     ws->seg_off, ws->seg_cstart, ws->seg_bchunk, ws->seg_bfirst, ws->seg_part,
                     ws->seg_digit_off, ws->cmask, ws->morder, ws->mbucket, ws->xm, ws->hs_x, ws->hs_v,
                     ws->hs_m, ws->hs_a, ws->hs_phi, ws->hs_diag, ws->dctl, ws->tile_hdr, ws->tile_idx,
-                    ws->tile_part, ws->tile_next, ws->ghead, ws->gtiles};
+                    ws->tile_part, ws->tile_next, ws->ghead, ws->gtiles, ws->sdig, ws->flat_cnt, ws->nraw};
     for (void *p : ptrs)
         if (p) cudaFree(p);
     if (ws->graph_exec) cudaGraphExecDestroy(ws->graph_exec);
@@ -290,6 +290,8 @@ tree_status_t tree_workspace_create(int64_t n_max, const TreeParams *p, TreeWork
              dalloc(&ws->ghead, (size_t)ws->groups_max) && dalloc(&ws->gtiles, (size_t)ws->groups_max);
         ws->tile_cap = ok ? (uint32_t)T : 0u;
     }
+    if (ok && n_max <= flat_octree_max())
+        ok = dalloc(&ws->sdig, N) && dalloc(&ws->flat_cnt, 513 * kLevels) && dalloc(&ws->nraw, NC);
     ws->chunks_cap = chunks_max;
     ws->box_cap = 1;
     if (!ok) {

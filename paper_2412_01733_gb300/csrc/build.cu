@@ -550,31 +550,6 @@ __global__ void k_tree_init(uint32_t *ctr, uint32_t *nfirst, uint32_t *ncount, u
     }
 }
 
-// Octant boundaries of a node's sorted range [first, first + count), count
-// >= 1: b[o] = first index whose octant digit at `shift` is >= o, o = 1..7
-// (keys in the range share their higher digits, so the digit is
-// non-decreasing).  Seven branchless lower-bound searches advance in lock
-// step, so each step issues seven independent loads: a large node costs
-// log2(count) load latencies, not seven times that.
-__device__ __forceinline__ void octant_bounds(const uint64_t *__restrict__ skey, uint32_t first, uint32_t count,
-                                              int shift, uint32_t (&b)[9]) {
-    uint32_t base[7];
-#pragma unroll
-    for (int o = 0; o < 7; ++o) base[o] = first;
-    uint32_t len = count;
-    while (len > 1) {
-        const uint32_t half = len >> 1;
-#pragma unroll
-        for (int o = 0; o < 7; ++o)
-            if ((uint32_t)((skey[base[o] + half] >> shift) & 7u) < (uint32_t)(o + 1)) base[o] += half;
-        len -= half;
-    }
-#pragma unroll
-    for (int o = 0; o < 7; ++o) b[o + 1] = base[o] + ((uint32_t)((skey[base[o]] >> shift) & 7u) < (uint32_t)(o + 1));
-    b[0] = first;
-    b[8] = first + count;
-}
-
 // Level L: every node decides leaf/internal; internal nodes find their
 // octant boundaries by binary search, a block scan plus a decoupled
 // look-back across tiles numbers the children breadth-first, and the
@@ -659,6 +634,7 @@ __global__ void __launch_bounds__(kLevelThreads) k_level(
 }
 
 cudaError_t launch_octree(TreeWorkspace *ws, int64_t n, cudaStream_t s) {
+    if (flat_octree(ws, n)) return launch_octree_flat(ws, n, s);
     k_tree_init<<<grid_for(ws->nseg, 128, 1 << 20), 128, 0, s>>>(ws->ctr, ws->nfirst, ws->ncount, ws->nparent, n,
                                                                  ws->seg_off, ws->nseg);
     double maxl = (double)ws->nseg;

@@ -86,6 +86,7 @@ enum CounterSlots {
     kCtrAbort = kCtrGroups + 2,               // stage whose bounded wait gave up (0: none)
     kCtrWalkTicket = kCtrGroups + 3,          // walk: next group slot (reset before every walk)
     kCtrTiles = kCtrGroups + 4,               // split walk: tile slots handed out (reset with the ticket)
+    kCtrFlatFull = kCtrGroups + 5,            // octree_flat.cu: the node array was too small
     kCtrCount = kCtrGroups + 8
 };
 
@@ -180,6 +181,9 @@ struct TreeWorkspace {
     uint32_t *gfirst = nullptr;        // walk groups: first sorted index of each, then n
     uint8_t *plev = nullptr;           // leaf level of every sorted particle
     uint32_t *pleaf = nullptr;         // leaf node of every sorted particle
+    uint8_t *sdig = nullptr;           // octree_flat.cu: digits shared with the particle before, + 1 [n_max]
+    uint32_t *flat_cnt = nullptr;      // octree_flat.cu: nodes per block and level
+    uint2 *nraw = nullptr;             // octree_flat.cu: first child or particle of every node, and the end
     uint32_t *nparent = nullptr;       // parent of every node (root: itself)
     uint32_t *ccount = nullptr, *coff = nullptr;  // groups starting in each Gs chunk / their offsets
     uint32_t *cmask = nullptr;         // group-start flags of each chunk, two 32-bit slices per chunk
@@ -427,6 +431,31 @@ __device__ __forceinline__ uint32_t seg_find(const int64_t *__restrict__ off, in
     return lo;
 }
 
+// Octant boundaries of a node's sorted range [first, first + count), count
+// >= 1: b[o] = first index whose octant digit at `shift` is >= o, o = 1..7
+// (keys in the range share their higher digits, so the digit is
+// non-decreasing).  Seven branchless lower-bound searches advance in lock
+// step, so each step issues seven independent loads: a large node costs
+// log2(count) load latencies, not seven times that.
+__device__ __forceinline__ void octant_bounds(const uint64_t *__restrict__ skey, uint32_t first, uint32_t count,
+                                              int shift, uint32_t (&b)[9]) {
+    uint32_t base[7];
+#pragma unroll
+    for (int o = 0; o < 7; ++o) base[o] = first;
+    uint32_t len = count;
+    while (len > 1) {
+        const uint32_t half = len >> 1;
+#pragma unroll
+        for (int o = 0; o < 7; ++o)
+            if ((uint32_t)((skey[base[o] + half] >> shift) & 7u) < (uint32_t)(o + 1)) base[o] += half;
+        len -= half;
+    }
+#pragma unroll
+    for (int o = 0; o < 7; ++o) b[o + 1] = base[o] + ((uint32_t)((skey[base[o]] >> shift) & 7u) < (uint32_t)(o + 1));
+    b[0] = first;
+    b[8] = first + count;
+}
+
 inline int grid_for(int64_t n, int threads, int max_blocks) {
     int64_t b = (n + threads - 1) / threads;
     if (b < 1) b = 1;
@@ -463,6 +492,14 @@ cudaError_t launch_box_segments(TreeWorkspace *ws, void *x, void *v, const void 
 cudaError_t launch_keys(TreeWorkspace *ws, const void *x, int64_t n, cudaStream_t s);
 cudaError_t launch_sort(TreeWorkspace *ws, int64_t n, cudaStream_t s);
 cudaError_t launch_octree(TreeWorkspace *ws, int64_t n, cudaStream_t s);
+// octree_flat.cu
+int64_t flat_octree_max();
+cudaError_t launch_octree_flat(TreeWorkspace *ws, int64_t n, cudaStream_t s);
+// Whether launch_octree takes the flat form: one system, in a workspace that
+// has its arrays (leaf levels then come with the octree).
+inline bool flat_octree(const TreeWorkspace *ws, int64_t n) {
+    return ws->nseg == 1 && ws->nraw && n <= flat_octree_max();
+}
 // groups.cu
 cudaError_t launch_groups(TreeWorkspace *ws, int64_t n, cudaStream_t s);
 cudaError_t launch_gather(TreeWorkspace *ws, const void *x, const void *m, int64_t n, cudaStream_t s);

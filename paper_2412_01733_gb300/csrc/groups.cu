@@ -173,8 +173,11 @@ cudaError_t launch_groups(TreeWorkspace *ws, int64_t n, cudaStream_t s) {
     const int64_t tiles = (nchunks + kGScanTile - 1) / kGScanTile;
     cudaError_t e = cudaMemsetAsync(ws->gscan_status, 0, (size_t)tiles * sizeof(uint32_t), s);
     if (e != cudaSuccess) return e;
-    k_leaf_levels<<<grid_for(ws->node_cap, 256, 152 * 8), 256, 0, s>>>(ws->ctr, ws->ngeo, ws->nlink, ws->plev,
-                                                                        ws->pleaf);
+    if (!flat_octree(ws, n)) {
+        k_leaf_levels<<<grid_for(ws->node_cap, 256, 152 * 8), 256, 0, s>>>(ws->ctr, ws->ngeo, ws->nlink, ws->plev,
+                                                                            ws->pleaf);
+        ws->launches += 1;
+    }
     const unsigned wb = (unsigned)((nchunks * 32 + 255) / 256);
     const uint32_t cmax = 128u * (uint32_t)gs;
     k_group_chunks<false><<<wb, 256, 0, s>>>(ws->key, ws->plev, ws->pleaf, ws->nparent, ws->ncount, cmax, n, gs,
@@ -185,7 +188,7 @@ cudaError_t launch_groups(TreeWorkspace *ws, int64_t n, cudaStream_t s) {
     k_group_chunks<true><<<wb, 256, 0, s>>>(ws->key, ws->plev, ws->pleaf, ws->nparent, ws->ncount, cmax, n, gs,
                                            ws->p.group_split, nchunks, ws->seg_off, ws->seg_cstart, ws->nseg, nullptr,
                                            ws->coff, ws->cmask, ws->gfirst, ws->ctr);
-    ws->launches += 4;
+    ws->launches += 3;
     return cudaGetLastError();
 }
 
