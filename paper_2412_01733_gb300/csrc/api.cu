@@ -78,7 +78,7 @@ void free_all(TreeWorkspace *ws) {
                     ws->seg_off, ws->seg_cstart, ws->seg_bchunk, ws->seg_bfirst, ws->seg_part,
                     ws->seg_digit_off, ws->cmask, ws->morder, ws->mbucket, ws->xm, ws->hs_x, ws->hs_v,
                     ws->hs_m, ws->hs_a, ws->hs_phi, ws->hs_diag, ws->dctl, ws->tile_hdr, ws->tile_idx,
-                    ws->tile_part, ws->tile_next, ws->ghead, ws->gtiles, ws->sdig, ws->flat_cnt, ws->nraw};
+                    ws->tile_part, ws->tile_next, ws->ghead, ws->gtiles, ws->sdig, ws->flat_cnt, ws->nraw, ws->marrived};
     for (void *p : ptrs)
         if (p) cudaFree(p);
     if (ws->graph_exec) cudaGraphExecDestroy(ws->graph_exec);
@@ -271,7 +271,7 @@ tree_status_t tree_workspace_create(int64_t n_max, const TreeParams *p, TreeWork
               dalloc((unsigned char **)&ws->spos, N * v4) && dalloc((unsigned char **)&ws->xm, N * v4) &&
               dalloc(&ws->nfirst, NC) && dalloc(&ws->ncount, NC) &&
               dalloc(&ws->ngeo, NC) && dalloc(&ws->nlink, NC) && dalloc(&ws->mom64, 10 * NC) &&
-              dalloc(&ws->morder, NC) && dalloc(&ws->mbucket, 3 * kMomBuckets + 1) &&
+              dalloc(&ws->morder, NC) && dalloc(&ws->mbucket, 3 * kMomBuckets + 1) && dalloc(&ws->marrived, NC) &&
               dalloc((unsigned char **)&ws->mom_a, NC * v4) && dalloc((unsigned char **)&ws->mom_b, NC * v4) &&
               dalloc((unsigned char **)&ws->mom_c, NC * v2) && dalloc(&ws->dstatus, 1) &&
               dalloc(&ws->stats, kStatCount) && dalloc(&ws->gstat, (size_t)ws->groups_max) &&
@@ -302,6 +302,7 @@ tree_status_t tree_workspace_create(int64_t n_max, const TreeParams *p, TreeWork
     }
     const DevCtl ctl{kWaitCycles, -1};
     if (cudaMemset(ws->dstatus, 0, sizeof(int32_t)) != cudaSuccess ||
+        cudaMemset(ws->marrived, 0, NC * sizeof(uint32_t)) != cudaSuccess ||
         cudaMemset(ws->stats, 0, kStatCount * sizeof(unsigned long long)) != cudaSuccess ||
         cudaMemcpy(ws->dctl, &ctl, sizeof(ctl), cudaMemcpyHostToDevice) != cudaSuccess) {
         free_all(ws);

@@ -44,6 +44,13 @@ constexpr int kTilesPer = 12;
 constexpr int kTileChunk = 16;
 constexpr uint32_t kTilesFull = 0xffffffffu;     // group whose tiles found no slot
 
+// Moments up to kClimbMaxN particles climb the tree in one launch, up to
+// kClimbPlainN without sorting the leaves by their particle counts first
+// (Plummer spheres, all moments: N = 1031 182 us level by level, 69 climbing;
+// 131072 272, 131 plain, 151 sorted; 262144 285, 187 plain, 157 sorted; 2^20
+// 355, 268 sorted; beyond, the level-by-level form's full warps gain on it).
+constexpr int64_t kClimbMaxN = (int64_t)1 << 20, kClimbPlainN = (int64_t)1 << 17;
+
 // lookback status words: 2-bit flag + 30-bit value
 constexpr uint32_t kFlagAgg = 1u << 30;
 constexpr uint32_t kFlagInc = 2u << 30;
@@ -170,6 +177,7 @@ struct TreeWorkspace {
     double *mom64 = nullptr;           // [10][node_cap]: M, Rx, Ry, Rz, Qxx, Qyy, Qzz, Qxy, Qxz, Qyz
     uint32_t *morder = nullptr;        // nodes in moment-bucket order [node_cap]
     uint32_t *mbucket = nullptr;       // moment buckets: counts, offsets (+ total), cursors
+    uint32_t *marrived = nullptr;      // moments: finished children of every cell (zero between passes)
     void *mom_a = nullptr;             // Vec4: (Rx, Ry, Rz, M)
     void *mom_b = nullptr;             // Vec4: (Qxx, Qyy, Qzz, Qxy); FP32 copies hold -Q
     void *mom_c = nullptr;             // Vec2: (Qxz, Qyz); FP32 copies hold -Q

@@ -95,9 +95,10 @@ struct MomSums {
     double M = 0, sx = 0, sy = 0, sz = 0, txx = 0, tyy = 0, tzz = 0, txy = 0, txz = 0, tyz = 0;
     double qxx = 0, qyy = 0, qzz = 0, qxy = 0, qxz = 0, qyz = 0;  // sum of the sources' own Q
     __device__ __forceinline__ void add(double m, double ux, double uy, double uz) {
+        // every rounding explicit: the kernels that sum cells round alike
         M += m;
-        const double mx = m * ux, my = m * uy, mz = m * uz;
-        sx += mx; sy += my; sz += mz;
+        const double mx = __dmul_rn(m, ux), my = __dmul_rn(m, uy), mz = __dmul_rn(m, uz);
+        sx = __dadd_rn(sx, mx); sy = __dadd_rn(sy, my); sz = __dadd_rn(sz, mz);
         txx = fma(mx, ux, txx); tyy = fma(my, uy, tyy); tzz = fma(mz, uz, tzz);
         txy = fma(mx, uy, txy); txz = fma(mx, uz, txz); tyz = fma(my, uz, tyz);
     }
@@ -112,12 +113,14 @@ __device__ __forceinline__ void mom_store(const MomSums &a, double cx, double cy
     double Rx = cx, Ry = cy, Rz = cz, qxx = 0, qyy = 0, qzz = 0, qxy = 0, qxz = 0, qyz = 0;
     if (a.M != 0.0) {
         const double iM = 1.0 / a.M;
-        Rx = cx + a.sx * iM; Ry = cy + a.sy * iM; Rz = cz + a.sz * iM;
-        const double txx = a.txx - a.sx * a.sx * iM, tyy = a.tyy - a.sy * a.sy * iM, tzz = a.tzz - a.sz * a.sz * iM;
-        const double txy = a.txy - a.sx * a.sy * iM, txz = a.txz - a.sx * a.sz * iM, tyz = a.tyz - a.sy * a.sz * iM;
+        Rx = fma(a.sx, iM, cx); Ry = fma(a.sy, iM, cy); Rz = fma(a.sz, iM, cz);
+        const double nx = -a.sx, ny = -a.sy, nz = -a.sz;
+        const double txx = fma(__dmul_rn(nx, a.sx), iM, a.txx), tyy = fma(__dmul_rn(ny, a.sy), iM, a.tyy);
+        const double tzz = fma(__dmul_rn(nz, a.sz), iM, a.tzz), txy = fma(__dmul_rn(nx, a.sy), iM, a.txy);
+        const double txz = fma(__dmul_rn(nx, a.sz), iM, a.txz), tyz = fma(__dmul_rn(ny, a.sz), iM, a.tyz);
         const double tr = txx + tyy + tzz;
-        qxx = a.qxx + (3.0 * txx - tr); qyy = a.qyy + (3.0 * tyy - tr); qzz = a.qzz + (3.0 * tzz - tr);
-        qxy = a.qxy + 3.0 * txy; qxz = a.qxz + 3.0 * txz; qyz = a.qyz + 3.0 * tyz;
+        qxx = a.qxx + fma(3.0, txx, -tr); qyy = a.qyy + fma(3.0, tyy, -tr); qzz = a.qzz + fma(3.0, tzz, -tr);
+        qxy = fma(3.0, txy, a.qxy); qxz = fma(3.0, txz, a.qxz); qyz = fma(3.0, tyz, a.qyz);
     }
     mom64[node] = a.M; mom64[cap + node] = Rx; mom64[2 * cap + node] = Ry; mom64[3 * cap + node] = Rz;
     mom64[4 * cap + node] = qxx; mom64[5 * cap + node] = qyy; mom64[6 * cap + node] = qzz;
@@ -149,9 +152,97 @@ __device__ __forceinline__ void mom_centre(uint4 g, uint32_t node, const DevBox 
         cz = (double)__fmaf_rn((float)g.z + half, unit, (float)bx->lo[2]);
     } else {
         const double half = 0.5 * (double)(1u << (kBits - lvl)), unit = bx->unit;
-        cx = bx->lo[0] + ((double)g.x + half) * unit;
-        cy = bx->lo[1] + ((double)g.y + half) * unit;
-        cz = bx->lo[2] + ((double)g.z + half) * unit;
+        cx = fma((double)g.x + half, unit, bx->lo[0]);
+        cy = fma((double)g.y + half, unit, bx->lo[1]);
+        cz = fma((double)g.z + half, unit, bx->lo[2]);
+    }
+}
+
+// Sums over the particles [first, end) of a leaf.  Four loads are in flight at
+// a time; the sums keep the particles' order.
+template <typename Real>
+__device__ __forceinline__ void mom_leaf(MomSums &a, const typename Vec4<Real>::T *__restrict__ spos, uint32_t first,
+                                         uint32_t end, double cx, double cy, double cz) {
+    for (uint32_t j = first; j < end; j += 4) {
+        typename Vec4<Real>::T p[4];
+#pragma unroll
+        for (int k = 0; k < 4; ++k)
+            if (j + k < end) p[k] = spos[j + k];
+#pragma unroll
+        for (int k = 0; k < 4; ++k)
+            if (j + k < end) a.add((double)p[k].w, (double)p[k].x - cx, (double)p[k].y - cy, (double)p[k].z - cz);
+    }
+}
+
+// The whole moment tree in one launch: a thread takes a leaf, and whoever
+// finishes the last child of a cell goes on with that cell, up to the root
+// (one arrival counter per cell, back at zero when the cell's children are
+// done, so the next pass finds it clear).  Nobody waits for anybody.  The
+// same sums in the same order as level by level (k_moments_level), which is
+// 21 launches of latency for a small system; here the latency is that of one
+// path of about ten cells, so what a cell needs is loaded before it is
+// needed: its own record with its child's sums, four children at a time (76
+// -> 69 us at N = 1031, 110 -> 104 at 30011).  What is left is FP64 latency
+// (ncu: 60 % of a warp's time in fixed-latency waits), about 8 us a cell.
+// Sixteen lanes per cell, one sum each, two cells of a warp at a time, took
+// longer (89 and 144 us).  BUCKETS: leaves in bucket order.
+template <typename Real, bool BUCKETS>
+__global__ void __launch_bounds__(64) k_moments_climb(
+    const uint32_t *__restrict__ ctr, const uint32_t *__restrict__ off, const uint32_t *__restrict__ order,
+    const uint4 *__restrict__ ngeo, const uint2 *__restrict__ nlink, const uint32_t *__restrict__ nparent,
+    uint32_t *__restrict__ arrived, const typename Vec4<Real>::T *__restrict__ spos, DevBox *__restrict__ box,
+    const uint32_t *__restrict__ nfirst, const int64_t *__restrict__ seg_off, int64_t nseg, double *mom64, int64_t cap,
+    typename Vec4<Real>::T *__restrict__ mom_a, typename Vec4<Real>::T *__restrict__ mom_b,
+    typename Vec2<Real>::T *__restrict__ mom_c) {
+    if (aborted(ctr, kStageAfter)) return;
+    const uint32_t end = BUCKETS ? off[kMomLeafBuckets] : ctr[kCtrLevelStart + kLevels];
+    for (uint32_t t = blockIdx.x * blockDim.x + threadIdx.x; t < end; t += gridDim.x * blockDim.x) {
+        uint32_t node = BUCKETS ? order[t] : t;
+        uint4 g = ngeo[node];
+        if (!BUCKETS && !((g.w >> 8) & 1u)) continue;
+        uint2 lk = nlink[node];
+        uint32_t par = nparent[node];
+        double cx, cy, cz;
+        mom_centre<Real>(g, node, box, nfirst, seg_off, nseg, cx, cy, cz);
+        MomSums a;
+        mom_leaf<Real>(a, spos, lk.x, lk.x + lk.y, cx, cy, cz);
+        lk = nlink[par];
+        g = ngeo[par];
+        mom_store<Real>(a, cx, cy, cz, node, mom64, cap, mom_a, mom_b, mom_c);
+        double M = a.M;
+        bool whole = true;  // this thread finished its cell
+        while (node >= (uint32_t)nseg) {
+            node = par;
+            __threadfence();  // this child's moments before its arrival
+            whole = atomicAdd(arrived + node, 1u) + 1u == lk.y;
+            if (!whole) break;
+            __threadfence();  // the other children's arrivals before their moments
+            arrived[node] = 0;
+            par = nparent[node];
+            mom_centre<Real>(g, node, box, nfirst, seg_off, nseg, cx, cy, cz);
+            MomSums b;
+            const uint32_t k1 = lk.x + lk.y;
+            for (uint32_t k0 = lk.x; k0 < k1; k0 += 4) {
+                double r[4][10];
+#pragma unroll
+                for (int j = 0; j < 4; ++j)
+#pragma unroll
+                    for (int c = 0; c < 10; ++c)
+                        if (k0 + j < k1) r[j][c] = __ldcg(mom64 + c * cap + k0 + j);
+#pragma unroll
+                for (int j = 0; j < 4; ++j)
+                    if (k0 + j < k1) {
+                        b.add(r[j][0], r[j][1] - cx, r[j][2] - cy, r[j][3] - cz);
+                        b.qxx += r[j][4]; b.qyy += r[j][5]; b.qzz += r[j][6];
+                        b.qxy += r[j][7]; b.qxz += r[j][8]; b.qyz += r[j][9];
+                    }
+            }
+            lk = nlink[par];
+            g = ngeo[par];
+            mom_store<Real>(b, cx, cy, cz, node, mom64, cap, mom_a, mom_b, mom_c);
+            M = b.M;
+        }
+        if (sizeof(Real) == 4 && whole) box[node].r5fit = pc_r5_fits(box[node].k, (float)M) ? 1 : 0;
     }
 }
 
@@ -171,10 +262,7 @@ __global__ void __launch_bounds__(256) k_moments_leaves(
         double cx, cy, cz;
         mom_centre<Real>(g, node, box, nfirst, seg_off, nseg, cx, cy, cz);
         MomSums a;
-        for (uint32_t j = lk.x; j < lk.x + lk.y; ++j) {
-            const typename Vec4<Real>::T p = spos[j];
-            a.add((double)p.w, (double)p.x - cx, (double)p.y - cy, (double)p.z - cz);
-        }
+        mom_leaf<Real>(a, spos, lk.x, lk.x + lk.y, cx, cy, cz);
         mom_store<Real>(a, cx, cy, cz, node, mom64, cap, mom_a, mom_b, mom_c);
     }
 }
@@ -220,12 +308,27 @@ static cudaError_t moments_impl(TreeWorkspace *ws, cudaStream_t s) {
     using V4 = typename Vec4<Real>::T;
     using V2 = typename Vec2<Real>::T;
     uint32_t *cnt = ws->mbucket, *off = ws->mbucket + kMomBuckets, *cursor = ws->mbucket + 2 * kMomBuckets + 1;
+    const int64_t cap = ws->node_cap;
+    const bool climb = ws->n <= kClimbMaxN, buckets = !climb || ws->n > kClimbPlainN;
+    if (climb && !buckets) {
+        k_moments_climb<Real, false><<<grid_for(cap, 64, 152 * 16), 64, 0, s>>>(
+            ws->ctr, off, ws->morder, ws->ngeo, ws->nlink, ws->nparent, ws->marrived, (const V4 *)ws->spos, ws->box,
+            ws->nfirst, ws->seg_off, ws->nseg, ws->mom64, cap, (V4 *)ws->mom_a, (V4 *)ws->mom_b, (V2 *)ws->mom_c);
+        ws->launches += 1;
+        return cudaGetLastError();
+    }
     cudaError_t e = cudaMemsetAsync(ws->mbucket, 0, (3 * kMomBuckets + 1) * sizeof(uint32_t), s);
     if (e != cudaSuccess) return e;
-    const int64_t cap = ws->node_cap;
     k_mom_hist<<<grid_for(cap, 256, 152 * 8), 256, 0, s>>>(ws->ctr, ws->ngeo, ws->nlink, cnt);
     k_mom_scatter<<<grid_for(cap, 256, 152 * 8), 256, 0, s>>>(ws->ctr, ws->ngeo, ws->nlink, cnt, off,
                                                                              cursor, ws->morder);
+    if (climb) {
+        k_moments_climb<Real, true><<<grid_for(cap, 64, 152 * 16), 64, 0, s>>>(
+            ws->ctr, off, ws->morder, ws->ngeo, ws->nlink, ws->nparent, ws->marrived, (const V4 *)ws->spos, ws->box,
+            ws->nfirst, ws->seg_off, ws->nseg, ws->mom64, cap, (V4 *)ws->mom_a, (V4 *)ws->mom_b, (V2 *)ws->mom_c);
+        ws->launches += 3;
+        return cudaGetLastError();
+    }
     k_moments_leaves<Real><<<grid_for(cap, 256, 152 * 8), 256, 0, s>>>(
         off, ws->morder, ws->ngeo, ws->nlink, (const V4 *)ws->spos, ws->box, ws->nfirst, ws->seg_off, ws->nseg,
         ws->mom64, cap, (V4 *)ws->mom_a, (V4 *)ws->mom_b, (V2 *)ws->mom_c);
