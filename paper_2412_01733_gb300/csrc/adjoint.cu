@@ -25,18 +25,19 @@
 // the lane and added to global FP64 accumulators with one atomic per
 // quantity per source per group; the target-side sums rotate through the
 // lanes with the targets.
-#include <cfloat>
+#include <type_traits>
 
-#include "common.cuh"
+#include "pairs.cuh"
 
 namespace treegb {
 
 constexpr int kAdjWarps = 4;
-constexpr int kAdjMaxTargets = 64;
+constexpr int kAdjMaxParts = 8;   // warps sharing a group's lists, at most
 
 struct AdjArgs {
     int64_t n;
     int64_t ngroups;
+    int32_t parts;         // warps per group: part p takes every parts-th tile of the lists
     const uint32_t *gfirst;
     const void *spos;      // Vec4 (x, y, z, m), key order
     const void *cot;       // Vec4 (abar, phibar), key order
@@ -45,234 +46,269 @@ struct AdjArgs {
     const int64_t *list_off;  // [2][ngroups + 1]
     const int32_t *pc_list, *pp_list;
     double G, eps2;
-    double *xt;            // [3][n] target-side xbar (plain stores), key order
-    double *xg;            // [3][n] source-side xbar (atomics), key order
-    double *mg;            // [n]    source-side mbar (atomics), key order
+    double *xg;            // [3][n] xbar (atomics), key order
+    double *mg;            // [n]    mbar (atomics), key order
     double *ccot;          // [10][cap] cell cotangents: Mbar, Rbar(3), Qbar(6)
     int64_t cap;
 };
 
-template <typename Real> struct AdjVec;
-template <> struct AdjVec<float> { using V4 = float4; using V2 = float2; };
-template <> struct AdjVec<double> { using V4 = double4a; using V2 = double2a; };
-
-template <typename Real> __device__ __forceinline__ Real rs_(Real x);
-template <> __device__ __forceinline__ float rs_<float>(float x) { return rsqrtf(x); }
-template <> __device__ __forceinline__ double rs_<double>(double x) { return rsqrt(x); }
-
-// 1/r of a pair.  Softened FP32 (SOFT, taken only when eps^2 is a normal FP32
-// number): r^2 >= eps^2 is never subnormal, so the PTX reciprocal square root
-// with subnormal inputs flushed serves, as in the walk's pair terms.
-// Otherwise the guarded form: a pair at r^2 = 0 contributes nothing.
-template <typename Real, bool SOFT>
-__device__ __forceinline__ Real inv_r(Real r2) {
-    if constexpr (SOFT && sizeof(Real) == 4) {
-        float y;
-        asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(r2));
-        return y;
-    } else {
-        return r2 > Real(0) ? rs_<Real>(r2) : Real(0);
+// One quantity of the targets a lane meets at a time: two in FP32 (packed
+// instructions), one in FP64.
+template <typename Real> struct Pack;
+template <> struct Pack<float> {
+    using V = float2;
+    static constexpr int kW = 2;
+    static __device__ __forceinline__ V dup(float a) { return make_float2(a, a); }
+    static __device__ __forceinline__ V add(V a, V b) { return __fadd2_rn(a, b); }
+    static __device__ __forceinline__ V mul(V a, V b) { return __fmul2_rn(a, b); }
+    static __device__ __forceinline__ V fma(V a, V b, V c) { return __ffma2_rn(a, b, c); }
+    static __device__ __forceinline__ V pick(bool ox, bool oy, V a) { return make_float2(ox ? 0.f : a.x, oy ? 0.f : a.y); }
+    static __device__ __forceinline__ float total(V a) { return a.x + a.y; }
+    template <bool SOFT> static __device__ __forceinline__ V rsqrt(V a) { return rsqrt_pair<SOFT>(a); }
+    static __device__ __forceinline__ V shfl(V a, int src) {
+        return make_float2(__shfl_sync(0xffffffffu, a.x, src), __shfl_sync(0xffffffffu, a.y, src));
     }
-}
+};
+template <> struct Pack<double> {
+    using V = double;
+    static constexpr int kW = 1;
+    static __device__ __forceinline__ V dup(double a) { return a; }
+    static __device__ __forceinline__ V add(V a, V b) { return a + b; }
+    static __device__ __forceinline__ V mul(V a, V b) { return a * b; }
+    static __device__ __forceinline__ V fma(V a, V b, V c) { return ::fma(a, b, c); }
+    static __device__ __forceinline__ V pick(bool ox, bool, V a) { return ox ? 0.0 : a; }
+    static __device__ __forceinline__ double total(V a) { return a; }
+    // r^2 = 0 contributes nothing, in the softened case too (eps^2 may underflow)
+    template <bool SOFT> static __device__ __forceinline__ V rsqrt(V a) { return a > 0.0 ? ::rsqrt(a) : 0.0; }
+    static __device__ __forceinline__ V shfl(V a, int src) { return __shfl_sync(0xffffffffu, a, src); }
+};
 
-// Derivatives of abar.a_PC + pb phi_PC for one (target, cell) pair.
-// y = target - R.  Outputs: gy (d/dy), mb (d/dM), qb (d/dQ stored components).
+// What a lane knows of its source (a cell, or a particle with no quadrupole).
+template <typename Real>
+struct AdjSource {
+    typename Pack<Real>::V x, y, z, nm, q[6];  // position, -M, -Q (xx yy zz xy xz yz)
+};
+
+// Adds the derivatives of f = abar.a + phibar phi of (target, source) pairs to
+// the source's sums and to the targets'.  With u = R - x, b = abar, p = phibar:
+//   e = -(u.b)/r^2, k = -5/2 e - p/2, h = -(b/r^5 + k u/r^5)... in the signs that
+// need no subtraction; -b, -p, -p/2 and -x are staged, -M and -Q held:
+//   df/du = C u + D (-b) + 2 c (-Q u) - r^-5 Q b,
+//     c = -k/r^5,  D = -M/r^3 - 5/2 (u.Q u)/r^7,
+//     C = M/r^3 (3e + p) + 5/r^7 [(Q u).b - (u.Q u)(k - e)];
+//   df/dM = -(u.(-b))/r^3 - p/r;   df/dQ_ij = -(u_i h_j + u_j h_i) (once on the
+//     diagonal), h = b/r^5 (signs as staged) + c u.
+// acc: 0, 1 the two parts of df/dM; 2-4 df/du; 5-10 -df/dQ.  85 operations for
+// a cell with quadrupole, 29 without.  own: the pair leaves the source itself
+// out (ox, oy: which of the lane's targets it is).
 template <typename Real, bool QUAD, bool SOFT>
-__device__ __forceinline__ void pc_vjp(Real yx, Real yy, Real yz, Real bx, Real by, Real bz, Real pb, Real Mc,
-                                       const Real (&q)[6], Real eps2, Real &gx, Real &gy, Real &gz, Real &mb,
-                                       Real (&qb)[6]) {
-    const Real r2 = yx * yx + yy * yy + yz * yz + eps2;
-    const Real i1 = inv_r<Real, SOFT>(r2);
-    const Real i2 = i1 * i1;
-    const Real i3 = i1 * i2, i5 = i3 * i2, i7 = i5 * i2, i9 = i7 * i2;
-    const Real yb = yx * bx + yy * by + yz * bz;
-    gx = -Mc * (bx * i3 - Real(3) * yx * yb * i5) + Mc * pb * yx * i3;
-    gy = -Mc * (by * i3 - Real(3) * yy * yb * i5) + Mc * pb * yy * i3;
-    gz = -Mc * (bz * i3 - Real(3) * yz * yb * i5) + Mc * pb * yz * i3;
-    mb = -yb * i3 - pb * i1;
+__device__ __forceinline__ void pair_vjp(const AdjSource<Real> &S, typename Pack<Real>::V nx, typename Pack<Real>::V ny,
+                                         typename Pack<Real>::V nz, typename Pack<Real>::V bx,
+                                         typename Pack<Real>::V by, typename Pack<Real>::V bz,
+                                         typename Pack<Real>::V np, typename Pack<Real>::V eps2, bool own, bool ox,
+                                         bool oy, typename Pack<Real>::V (&acc)[11], typename Pack<Real>::V (&t)[3]) {
+    using P = Pack<Real>;
+    using V = typename P::V;
+    const V ux = P::add(S.x, nx), uy = P::add(S.y, ny), uz = P::add(S.z, nz);
+    const V r2 = P::fma(ux, ux, P::fma(uy, uy, P::fma(uz, uz, eps2)));
+    V i1 = P::template rsqrt<SOFT>(r2);
+    if (own) i1 = P::pick(ox, oy, i1);
+    const V i2 = P::mul(i1, i1);
+    const V i3 = P::mul(i1, i2);
+    const V ub = P::fma(ux, bx, P::fma(uy, by, P::mul(uz, bz)));  // u.(-b)
+    const V e = P::mul(ub, i2);
+    const V nmi3 = P::mul(S.nm, i3);
+    const V s = P::fma(P::dup(Real(-3)), e, np);  // -(3e + p)
+    V C = P::mul(nmi3, s), D = nmi3;
+    acc[0] = P::fma(np, i1, acc[0]);
+    acc[1] = P::fma(ub, i3, acc[1]);
+    V gx, gy, gz;
     if (QUAD) {
-        const Real Qx = q[0] * yx + q[3] * yy + q[4] * yz;
-        const Real Qy = q[3] * yx + q[1] * yy + q[5] * yz;
-        const Real Qz = q[4] * yx + q[5] * yy + q[2] * yz;
-        const Real yQy = yx * Qx + yy * Qy + yz * Qz;
-        const Real Qb = Qx * bx + Qy * by + Qz * bz;
-        const Real Qbx = q[0] * bx + q[3] * by + q[4] * bz;
-        const Real Qby = q[3] * bx + q[1] * by + q[5] * bz;
-        const Real Qbz = q[4] * bx + q[5] * by + q[2] * bz;
-        const Real c1 = Real(17.5) * yQy * yb * i9 - Real(5) * Qb * i7 + Real(2.5) * pb * yQy * i7;
-        const Real c2 = -Real(5) * yb * i7 - pb * i5;
-        const Real c3 = -Real(2.5) * yQy * i7;
-        gx += Qbx * i5 + c2 * Qx + c3 * bx + c1 * yx;
-        gy += Qby * i5 + c2 * Qy + c3 * by + c1 * yy;
-        gz += Qbz * i5 + c2 * Qz + c3 * bz + c1 * yz;
-        const Real ca = i5, cb = -Real(2.5) * i7 * yb - Real(0.5) * pb * i5;
-        qb[0] = ca * yx * bx + cb * yx * yx;
-        qb[1] = ca * yy * by + cb * yy * yy;
-        qb[2] = ca * yz * bz + cb * yz * yz;
-        qb[3] = ca * (yx * by + yy * bx) + cb * Real(2) * yx * yy;
-        qb[4] = ca * (yx * bz + yz * bx) + cb * Real(2) * yx * yz;
-        qb[5] = ca * (yy * bz + yz * by) + cb * Real(2) * yy * yz;
+        const V ni2 = P::mul(i2, P::dup(Real(-1)));
+        const V ni5 = P::mul(i3, ni2);
+        const V k5 = P::mul(ni5, P::mul(ni2, P::dup(Real(5))));  // 5 / r^7
+        const V wx = P::fma(S.q[0], ux, P::fma(S.q[3], uy, P::mul(S.q[4], uz)));
+        const V wy = P::fma(S.q[3], ux, P::fma(S.q[1], uy, P::mul(S.q[5], uz)));
+        const V wz = P::fma(S.q[4], ux, P::fma(S.q[5], uy, P::mul(S.q[2], uz)));
+        const V vx = P::fma(S.q[0], bx, P::fma(S.q[3], by, P::mul(S.q[4], bz)));
+        const V vy = P::fma(S.q[3], bx, P::fma(S.q[1], by, P::mul(S.q[5], bz)));
+        const V vz = P::fma(S.q[4], bx, P::fma(S.q[5], by, P::mul(S.q[2], bz)));
+        const V uw = P::fma(ux, wx, P::fma(uy, wy, P::mul(uz, wz)));
+        const V wb = P::fma(bx, wx, P::fma(by, wy, P::mul(bz, wz)));
+        const V hp = P::mul(np, P::dup(Real(0.5)));               // -p/2
+        const V k = P::fma(P::dup(Real(-2.5)), e, hp);
+        const V d = P::fma(P::dup(Real(-3.5)), e, hp);
+        const V uwk = P::mul(uw, k5);
+        C = P::add(C, P::fma(uwk, d, P::mul(k5, wb)));
+        D = P::fma(P::dup(Real(0.5)), uwk, D);
+        const V c = P::mul(ni5, k), c2 = P::add(c, c);
+        gx = P::fma(C, ux, P::fma(D, bx, P::fma(c2, wx, P::mul(ni5, vx))));
+        gy = P::fma(C, uy, P::fma(D, by, P::fma(c2, wy, P::mul(ni5, vy))));
+        gz = P::fma(C, uz, P::fma(D, bz, P::fma(c2, wz, P::mul(ni5, vz))));
+        const V hx = P::fma(ni5, bx, P::mul(c, ux)), hy = P::fma(ni5, by, P::mul(c, uy)),
+                hz = P::fma(ni5, bz, P::mul(c, uz));
+        acc[5] = P::fma(ux, hx, acc[5]);
+        acc[6] = P::fma(uy, hy, acc[6]);
+        acc[7] = P::fma(uz, hz, acc[7]);
+        acc[8] = P::fma(ux, hy, P::fma(uy, hx, acc[8]));
+        acc[9] = P::fma(ux, hz, P::fma(uz, hx, acc[9]));
+        acc[10] = P::fma(uy, hz, P::fma(uz, hy, acc[10]));
     } else {
-#pragma unroll
-        for (int k = 0; k < 6; ++k) qb[k] = Real(0);
+        gx = P::fma(C, ux, P::mul(D, bx));
+        gy = P::fma(C, uy, P::mul(D, by));
+        gz = P::fma(C, uz, P::mul(D, bz));
     }
+    acc[2] = P::add(acc[2], gx); acc[3] = P::add(acc[3], gy); acc[4] = P::add(acc[4], gz);
+    t[0] = P::add(t[0], gx); t[1] = P::add(t[1], gy); t[2] = P::add(t[2], gz);
 }
 
-// PP pair: d = source - target.  g as in the header; dm = d/dm_j (without G).
-template <typename Real, bool SOFT>
-__device__ __forceinline__ void pp_vjp(Real dx, Real dy, Real dz, Real bx, Real by, Real bz, Real pb, Real mj,
-                                       Real eps2, Real &gx, Real &gy, Real &gz, Real &dm) {
-    const Real r2 = dx * dx + dy * dy + dz * dz + eps2;
-    const Real i1 = inv_r<Real, SOFT>(r2);
-    const Real i3 = i1 * i1 * i1, i5 = i3 * i1 * i1;
-    const Real db = dx * bx + dy * by + dz * bz;
-    gx = mj * (bx * i3 - Real(3) * dx * db * i5 + pb * dx * i3);
-    gy = mj * (by * i3 - Real(3) * dy * db * i5 + pb * dy * i3);
-    gz = mj * (bz * i3 - Real(3) * dz * db * i5 + pb * dz * i3);
-    dm = db * i3 - pb * i1;
-}
-
+// A warp (one of A.parts sharing the group) walks its share of the group's
+// stored lists, 32 sources at a time, one source per lane.  Bound by the FMA
+// pipe; in FP32 a lane meets two targets at a time in packed instructions:
+// targets j and j + 16 of a half of the group travel as a pair through
+// sixteen lanes, the warp's two halves holding one copy of the targets' sums
+// each.  (One pair at a time: Plummer sphere, N = 262144, 5.3 ms; now 2.9.)
+// Up to kAdjMaxParts warps share a group where there are few groups: N =
+// 65536 1.9 -> 0.85 ms.
 template <typename Real, bool QUAD, bool SOFT>
 __global__ void __launch_bounds__(kAdjWarps * 32) k_force_vjp(const AdjArgs A) {
-    using V4 = typename AdjVec<Real>::V4;
-    using V2 = typename AdjVec<Real>::V2;
-    __shared__ V4 s_tp[kAdjWarps][kAdjMaxTargets];   // target position + mass
-    __shared__ V4 s_tc[kAdjWarps][kAdjMaxTargets];   // target cotangent
+    using P = Pack<Real>;
+    using V = typename P::V;
+    using V4 = typename Vec4<Real>::T;
+    using V2 = typename Vec2<Real>::T;
+    constexpr int W = P::kW, L = 32 / W;  // targets met at a time, and steps to meet a half
+    // per warp and half: -x, -y, -z, -bx, -by, -bz, -p of the targets, packed
+    __shared__ V s_t[kAdjWarps][2][7][L];
     __shared__ uint32_t s_buf[kAdjWarps][32 + 32 * kMaxLeafSmall];
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    const int next = (lane + 1) & 31;
-    const int64_t g = (int64_t)blockIdx.x * kAdjWarps + w;
+    const int next = (lane & ~(L - 1)) | ((lane + 1) & (L - 1));
+    const int64_t item = (int64_t)blockIdx.x * kAdjWarps + w;
+    const int64_t g = item / A.parts;
+    const int part = (int)(item - g * A.parts);
     if (g >= A.ngroups) return;
     const V4 *spos = reinterpret_cast<const V4 *>(A.spos);
     const V4 *cot = reinterpret_cast<const V4 *>(A.cot);
     const V4 *momA = reinterpret_cast<const V4 *>(A.mom_a);
     const V4 *momB = reinterpret_cast<const V4 *>(A.mom_b);
     const V2 *momC = reinterpret_cast<const V2 *>(A.mom_c);
-    const Real eps2 = (Real)A.eps2;
+    const V eps2 = P::dup((Real)A.eps2);
     const uint32_t s0 = A.gfirst[g];
     const int cnt = (int)(A.gfirst[g + 1] - s0);
-    for (int t = lane; t < cnt; t += 32) {
-        s_tp[w][t] = spos[s0 + t];
-        s_tc[w][t] = cot[s0 + t];
+    const int halves = cnt > 32 ? 2 : 1;
+    for (int t = lane; t < 32 * halves; t += 32) {
+        // places past the group's end: its first particle without a cotangent, which adds nothing
+        const V4 p = spos[s0 + (t < cnt ? t : 0)];
+        V4 b{};
+        if (t < cnt) b = cot[s0 + t];
+        const int at = W * (t & (L - 1)) + ((t & 31) >= L ? 1 : 0);  // target j + 16 is the second of pair j
+        Real *st = reinterpret_cast<Real *>(&s_t[w][t >> 5][0][0]);
+        const Real v[7] = {-p.x, -p.y, -p.z, -b.x, -b.y, -b.z, -b.w};
+#pragma unroll
+        for (int c = 0; c < 7; ++c) st[c * 32 + at] = v[c];
     }
     __syncwarp();
     double xt[2][3] = {{0, 0, 0}, {0, 0, 0}};
+    const Real px0 = spos[s0].x, py0 = spos[s0].y, pz0 = spos[s0].z;
 
-    // Every pair of a tile is evaluated once.  Lane l holds source l (a cell
-    // or a particle) and, at step k, meets target (l + k) mod 32 of the
-    // current half of the group: the source-side sums stay in the lane, the
-    // target-side partial sums travel with their target (one shuffle per step
-    // passes each to the lane that meets it next; after 32 steps a final
-    // shuffle brings target l's total to lane l).
+    // All pairs of the lanes' sources with the group's targets: the source-side
+    // sums stay in the lane, the targets' partial sums travel with them (one
+    // shuffle per step passes each on to the lane that meets it next).
+    auto meet = [&](const AdjSource<Real> &S, auto quad, bool own, uint32_t sj, V(&acc)[11]) {
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            if (h >= halves) break;
+            V t[3] = {P::dup(Real(0)), P::dup(Real(0)), P::dup(Real(0))};
+            const V(*st)[L] = s_t[w][h];
+            const uint32_t first = s0 + 32u * (uint32_t)h;
+#pragma unroll 1
+            for (int k = 0; k < L; ++k) {
+                if (k > 0) {
+#pragma unroll
+                    for (int c = 0; c < 3; ++c) t[c] = P::shfl(t[c], next);
+                }
+                const int j = (lane + k) & (L - 1);
+                pair_vjp<Real, decltype(quad)::value, SOFT>(S, st[0][j], st[1][j], st[2][j], st[3][j], st[4][j],
+                                                            st[5][j], st[6][j], eps2, own, first + j == sj,
+                                                            first + j + L == sj, acc, t);
+            }
+#pragma unroll
+            for (int c = 0; c < 3; ++c) {
+                t[c] = P::shfl(t[c], next);
+                if constexpr (W == 2) {
+                    // both halves of the warp hold a share of pair (lane & 15)
+                    t[c] = P::add(t[c], P::shfl(t[c], lane ^ 16));
+                    xt[h][c] += (double)(lane < 16 ? t[c].x : t[c].y);
+                } else {
+                    xt[h][c] += t[c];
+                }
+            }
+        }
+    };
 
     // ---- far cells ----
     const int64_t pc0 = A.list_off[g], pc1 = A.list_off[g + 1];
-    for (int64_t base = pc0; base < pc1; base += 32) {
+    for (int64_t base = pc0 + 32 * part; base < pc1; base += 32 * A.parts) {
         const int nt = (int)min((int64_t)32, pc1 - base);
         uint32_t cid = 0;
-        V4 ca{};
-        Real cq[6] = {0, 0, 0, 0, 0, 0};
+        AdjSource<Real> S;
+        S.x = P::dup(px0); S.y = P::dup(py0); S.z = P::dup(pz0); S.nm = P::dup(Real(0));
+#pragma unroll
+        for (int q = 0; q < 6; ++q) S.q[q] = P::dup(Real(0));
         if (lane < nt) {
             cid = (uint32_t)A.pc_list[base + lane];
-            ca = momA[cid];
+            const V4 a = momA[cid];
+            S.x = P::dup(a.x); S.y = P::dup(a.y); S.z = P::dup(a.z); S.nm = P::dup(-a.w);
             if (QUAD) {
                 const V4 b = momB[cid];
-                const V2 cc = momC[cid];
-                const Real qs = sizeof(Real) == 4 ? Real(-1) : Real(1);  // FP32 walk copies hold -Q
-                cq[0] = qs * b.x; cq[1] = qs * b.y; cq[2] = qs * b.z;
-                cq[3] = qs * b.w; cq[4] = qs * cc.x; cq[5] = qs * cc.y;
+                const V2 c = momC[cid];
+                const Real qs = sizeof(Real) == 4 ? Real(1) : Real(-1);  // the FP32 walk copies hold -Q
+                S.q[0] = P::dup(qs * b.x); S.q[1] = P::dup(qs * b.y); S.q[2] = P::dup(qs * b.z);
+                S.q[3] = P::dup(qs * b.w); S.q[4] = P::dup(qs * c.x); S.q[5] = P::dup(qs * c.y);
             }
         }
         // the group's (at most 64) targets are summed in the working precision;
         // the per-group totals go to the FP64 accumulators
-        Real acc[10] = {0, 0, 0, 0, 0, 0, 0, 0, 0, 0};
+        V acc[11];
 #pragma unroll
-        for (int h = 0; h < 2; ++h) {
-            if (32 * h >= cnt) break;
-            const int ch = min(32, cnt - 32 * h);
-            Real tx = 0, ty = 0, tz = 0;
-            for (int k = 0; k < 32; ++k) {
-                if (k > 0) {
-                    tx = __shfl_sync(0xffffffffu, tx, next);
-                    ty = __shfl_sync(0xffffffffu, ty, next);
-                    tz = __shfl_sync(0xffffffffu, tz, next);
-                }
-                const int t = (lane + k) & 31;
-                if (lane < nt && t < ch) {
-                    const V4 p = s_tp[w][32 * h + t];
-                    const V4 b = s_tc[w][32 * h + t];
-                    Real gx, gy, gz, mb, qb[6];
-                    pc_vjp<Real, QUAD, SOFT>(p.x - ca.x, p.y - ca.y, p.z - ca.z, b.x, b.y, b.z, b.w, ca.w, cq, eps2, gx,
-                                       gy, gz, mb, qb);
-                    tx += gx; ty += gy; tz += gz;
-                    acc[0] += mb;
-                    acc[1] -= gx; acc[2] -= gy; acc[3] -= gz;
-#pragma unroll
-                    for (int q = 0; q < 6; ++q) acc[4 + q] += qb[q];
-                }
-            }
-            tx = __shfl_sync(0xffffffffu, tx, next);
-            ty = __shfl_sync(0xffffffffu, ty, next);
-            tz = __shfl_sync(0xffffffffu, tz, next);
-            if (lane < ch) { xt[h][0] += (double)tx; xt[h][1] += (double)ty; xt[h][2] += (double)tz; }
-        }
+        for (int q = 0; q < 11; ++q) acc[q] = P::dup(Real(0));
+        meet(S, std::bool_constant<QUAD>{}, false, 0u, acc);
         if (lane < nt) {
+            const Real mb = P::total(acc[0]) - P::total(acc[1]);
+            if (mb != Real(0)) atomicAdd(A.ccot + cid, A.G * (double)mb);
 #pragma unroll
-            for (int q = 0; q < (QUAD ? 10 : 4); ++q)
-                if (acc[q] != Real(0)) atomicAdd(A.ccot + (int64_t)q * A.cap + cid, A.G * (double)acc[q]);
+            for (int q = 2; q < (QUAD ? 11 : 5); ++q) {
+                const Real v = P::total(acc[q]);
+                if (v != Real(0)) atomicAdd(A.ccot + (int64_t)(q - 1) * A.cap + cid, (q < 5 ? A.G : -A.G) * (double)v);
+            }
         }
     }
 
     // ---- near leaves: expand particles into the buffer, tiles of 32 ----
     const int64_t pp0 = A.list_off[A.ngroups + 1 + g], pp1 = A.list_off[A.ngroups + 1 + g + 1];
-    auto pp_tile = [&](const uint32_t *src, int nt) {
-        uint32_t sj = 0;
-        V4 sa{};
+    auto pp_tile = [&](uint32_t sj, int nt) {
+        AdjSource<Real> S;
+        S.x = P::dup(px0); S.y = P::dup(py0); S.z = P::dup(pz0); S.nm = P::dup(Real(0));
         if (lane < nt) {
-            sj = src[lane];
-            sa = spos[sj];
+            const V4 a = spos[sj];
+            S.x = P::dup(a.x); S.y = P::dup(a.y); S.z = P::dup(a.z); S.nm = P::dup(-a.w);
         }
-        __syncwarp();
-        Real gxs = 0, gys = 0, gzs = 0, dms = 0;
+        const bool own = __any_sync(0xffffffffu, lane < nt && sj - s0 < (uint32_t)cnt);
+        V acc[11];
 #pragma unroll
-        for (int h = 0; h < 2; ++h) {
-            if (32 * h >= cnt) break;
-            const int ch = min(32, cnt - 32 * h);
-            Real tx = 0, ty = 0, tz = 0;
-            for (int k = 0; k < 32; ++k) {
-                if (k > 0) {
-                    tx = __shfl_sync(0xffffffffu, tx, next);
-                    ty = __shfl_sync(0xffffffffu, ty, next);
-                    tz = __shfl_sync(0xffffffffu, tz, next);
-                }
-                const int t = (lane + k) & 31;
-                // the self pair is excluded by index
-                if (lane < nt && t < ch && s0 + (uint32_t)(32 * h + t) != sj) {
-                    const V4 p = s_tp[w][32 * h + t];
-                    const V4 b = s_tc[w][32 * h + t];
-                    Real gx, gy, gz, dm;
-                    pp_vjp<Real, SOFT>(sa.x - p.x, sa.y - p.y, sa.z - p.z, b.x, b.y, b.z, b.w, sa.w, eps2, gx, gy, gz,
-                                 dm);
-                    tx -= gx; ty -= gy; tz -= gz;
-                    gxs += gx; gys += gy; gzs += gz; dms += dm;
-                }
-            }
-            tx = __shfl_sync(0xffffffffu, tx, next);
-            ty = __shfl_sync(0xffffffffu, ty, next);
-            tz = __shfl_sync(0xffffffffu, tz, next);
-            if (lane < ch) { xt[h][0] += (double)tx; xt[h][1] += (double)ty; xt[h][2] += (double)tz; }
-        }
+        for (int q = 0; q < 5; ++q) acc[q] = P::dup(Real(0));
+        // the self pair is excluded by index
+        if (own) meet(S, std::false_type{}, true, lane < nt ? sj : 0xffffffffu, acc);
+        else meet(S, std::false_type{}, false, 0u, acc);
         if (lane < nt) {
-            atomicAdd(A.xg + sj, A.G * (double)gxs);
-            atomicAdd(A.xg + A.n + sj, A.G * (double)gys);
-            atomicAdd(A.xg + 2 * A.n + sj, A.G * (double)gzs);
-            atomicAdd(A.mg + sj, A.G * (double)dms);
+            atomicAdd(A.xg + sj, A.G * (double)P::total(acc[2]));
+            atomicAdd(A.xg + A.n + sj, A.G * (double)P::total(acc[3]));
+            atomicAdd(A.xg + 2 * A.n + sj, A.G * (double)P::total(acc[4]));
+            atomicAdd(A.mg + sj, A.G * (double)(P::total(acc[0]) - P::total(acc[1])));
         }
-        __syncwarp();
     };
     uint32_t *buf = s_buf[w];
     int nb = 0;
-    for (int64_t base = pp0; base < pp1; base += 32) {
+    for (int64_t base = pp0 + 32 * part; base < pp1; base += 32 * A.parts) {
         const int nl = (int)min((int64_t)32, pp1 - base);
         uint2 lk = make_uint2(0, 0);
         if (lane < nl) lk = A.nlink[(uint32_t)A.pp_list[base + lane]];
@@ -293,17 +329,11 @@ __global__ void __launch_bounds__(kAdjWarps * 32) k_force_vjp(const AdjArgs A) {
             const int b = __ffs(bm) - 1;
             bm &= bm - 1;
             const uint32_t f = __shfl_sync(0xffffffffu, lk.x, b), c = __shfl_sync(0xffffffffu, lk.y, b);
-            for (uint32_t o = 0; o < c; o += 32) {
-                const int k = (int)min(32u, c - o);
-                __shared__ uint32_t s_rng[kAdjWarps][32];
-                if (lane < k) s_rng[w][lane] = f + o + lane;
-                __syncwarp();
-                pp_tile(s_rng[w], k);
-            }
+            for (uint32_t o = 0; o < c; o += 32) pp_tile(f + o + (uint32_t)lane, (int)min(32u, c - o));
         }
         int done = 0;
         while (nb - done >= 32) {
-            pp_tile(buf + done, 32);
+            pp_tile(buf[done + lane], 32);
             done += 32;
         }
         const int r = nb - done;
@@ -313,14 +343,13 @@ __global__ void __launch_bounds__(kAdjWarps * 32) k_force_vjp(const AdjArgs A) {
         __syncwarp();
         nb = r;
     }
-    if (nb > 0) pp_tile(buf, nb);
+    if (nb > 0) pp_tile(lane < nb ? buf[lane] : 0u, nb);
 
-    for (int tt = 0; tt < 2; ++tt) {
-        const int t = lane + 32 * tt;
+    for (int h = 0; h < halves; ++h) {
+        const int t = lane + 32 * h;
         if (t < cnt) {
-            A.xt[s0 + t] = A.G * xt[tt][0];
-            A.xt[A.n + s0 + t] = A.G * xt[tt][1];
-            A.xt[2 * A.n + s0 + t] = A.G * xt[tt][2];
+#pragma unroll
+            for (int c = 0; c < 3; ++c) atomicAdd(A.xg + c * A.n + s0 + t, -A.G * xt[h][c]);
         }
     }
 }
@@ -329,12 +358,12 @@ __global__ void __launch_bounds__(kAdjWarps * 32) k_force_vjp(const AdjArgs A) {
 template <typename Real>
 __global__ void __launch_bounds__(256) k_cot_gather(const Real *__restrict__ abar, const Real *__restrict__ phibar,
                                                     const uint32_t *__restrict__ perm, int64_t n,
-                                                    typename AdjVec<Real>::V4 *__restrict__ cot,
+                                                    typename Vec4<Real>::T *__restrict__ cot,
                                                     const uint32_t *__restrict__ ctr) {
     if (aborted(ctr, kStageAfter)) return;
     for (int64_t s = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; s < n; s += (int64_t)gridDim.x * blockDim.x) {
         const uint32_t i = perm[s];
-        typename AdjVec<Real>::V4 c;
+        typename Vec4<Real>::T c;
         c.x = abar[i]; c.y = abar[n + i]; c.z = abar[2 * n + i];
         c.w = phibar ? phibar[i] : Real(0);
         cot[s] = c;
@@ -346,7 +375,7 @@ template <typename Real>
 __global__ void __launch_bounds__(256) k_cot_push(int L, const uint32_t *__restrict__ ctr,
                                                   const uint4 *__restrict__ ngeo, const uint2 *__restrict__ nlink,
                                                   const double *__restrict__ mom64, int64_t cap,
-                                                  const typename AdjVec<Real>::V4 *__restrict__ spos,
+                                                  const typename Vec4<Real>::T *__restrict__ spos,
                                                   double *__restrict__ ccot, double *__restrict__ xg,
                                                   double *__restrict__ mg, int64_t n) {
     if (aborted(ctr, kStageAfter)) return;
@@ -374,7 +403,7 @@ __global__ void __launch_bounds__(256) k_cot_push(int L, const uint32_t *__restr
         for (uint32_t k = lk.x; k < lk.x + lk.y; ++k) {
             double mk, dx, dy, dz;
             if (leaf) {
-                const typename AdjVec<Real>::V4 p = spos[k];
+                const typename Vec4<Real>::T p = spos[k];
                 mk = (double)p.w;
                 dx = (double)p.x - Rx; dy = (double)p.y - Ry; dz = (double)p.z - Rz;
             } else {
@@ -406,19 +435,19 @@ __global__ void __launch_bounds__(256) k_cot_push(int L, const uint32_t *__restr
     }
 }
 
-// xbar[i] += xt + xg, mbar[i] += mg (key order -> caller order)
+// xbar[i] += xg, mbar[i] += mg (key order -> caller order)
 template <typename Real>
-__global__ void __launch_bounds__(256) k_grad_scatter(const double *__restrict__ xt, const double *__restrict__ xg,
-                                                      const double *__restrict__ mg, const uint32_t *__restrict__ perm,
+__global__ void __launch_bounds__(256) k_grad_scatter(const double *__restrict__ xg, const double *__restrict__ mg,
+                                                      const uint32_t *__restrict__ perm,
                                                       int64_t n, Real *__restrict__ xbar, Real *__restrict__ mbar,
                                                       const uint32_t *__restrict__ ctr) {
     if (aborted(ctr, kStageAfter)) return;
     for (int64_t s = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; s < n; s += (int64_t)gridDim.x * blockDim.x) {
         const uint32_t i = perm[s];
         if (xbar) {
-            xbar[i] += (Real)(xt[s] + xg[s]);
-            xbar[n + i] += (Real)(xt[n + s] + xg[n + s]);
-            xbar[2 * n + i] += (Real)(xt[2 * n + s] + xg[2 * n + s]);
+            xbar[i] += (Real)xg[s];
+            xbar[n + i] += (Real)xg[n + s];
+            xbar[2 * n + i] += (Real)xg[2 * n + s];
         }
         if (mbar) mbar[i] += (Real)mg[s];
     }
@@ -434,7 +463,7 @@ static cudaError_t adjoint_impl(TreeWorkspace *ws, const void *abar, const void 
     if ((e = cudaMemsetAsync(ws->adj_ccot, 0, 10 * cap * sizeof(double), s)) != cudaSuccess) return e;
     const int nb = grid_for(n, 256, 152 * 8);
     k_cot_gather<Real><<<nb, 256, 0, s>>>((const Real *)abar, (const Real *)phibar, ws->idx, n,
-                                          (typename AdjVec<Real>::V4 *)ws->adj_cot, ws->ctr);
+                                          (typename Vec4<Real>::T *)ws->adj_cot, ws->ctr);
     AdjArgs A;
     A.n = n;
     A.ngroups = ws->list_groups;
@@ -447,30 +476,29 @@ static cudaError_t adjoint_impl(TreeWorkspace *ws, const void *abar, const void 
     A.pc_list = ws->pc_list; A.pp_list = ws->pp_list;
     A.G = ws->p.G;
     A.eps2 = ws->p.eps * ws->p.eps;
-    A.xt = ws->adj_xt; A.xg = ws->adj_xg; A.mg = ws->adj_mg; A.ccot = ws->adj_ccot;
+    A.xg = ws->adj_xg; A.mg = ws->adj_mg; A.ccot = ws->adj_ccot;
     A.cap = cap;
-    const unsigned gb = (unsigned)((A.ngroups + kAdjWarps - 1) / kAdjWarps);
+    // enough warps for several rounds of the chip also when there are few groups
+    const int64_t want = 152 * 64;
+    A.parts = A.ngroups > 0 ? (int)((want + A.ngroups - 1) / A.ngroups) : 1;
+    if (A.parts > kAdjMaxParts) A.parts = kAdjMaxParts;
+    const unsigned gb = (unsigned)((A.ngroups * A.parts + kAdjWarps - 1) / kAdjWarps);
     if (A.ngroups > 0) {
-        const bool quad = ws->p.order == 2;
-        bool done = false;
-        if constexpr (sizeof(Real) == 4) {
-            if ((float)(ws->p.eps * ws->p.eps) >= FLT_MIN) {  // softened FP32 pairs (inv_r)
-                if (quad) k_force_vjp<Real, true, true><<<gb, kAdjWarps * 32, 0, s>>>(A);
-                else k_force_vjp<Real, false, true><<<gb, kAdjWarps * 32, 0, s>>>(A);
-                done = true;
-            }
-        }
-        if (!done) {
-            if (quad) k_force_vjp<Real, true, false><<<gb, kAdjWarps * 32, 0, s>>>(A);
+        const bool quad = ws->p.order == 2, soft = sizeof(Real) == 8 || walk_soft_f32(ws->p.eps);
+        if (quad) {
+            if (soft) k_force_vjp<Real, true, true><<<gb, kAdjWarps * 32, 0, s>>>(A);
+            else k_force_vjp<Real, true, false><<<gb, kAdjWarps * 32, 0, s>>>(A);
+        } else {
+            if (soft) k_force_vjp<Real, false, true><<<gb, kAdjWarps * 32, 0, s>>>(A);
             else k_force_vjp<Real, false, false><<<gb, kAdjWarps * 32, 0, s>>>(A);
         }
     }
     const int nbn = grid_for(ws->node_cap, 256, 152 * 8);
     for (int L = 0; L < kLevels; ++L)
         k_cot_push<Real><<<nbn, 256, 0, s>>>(L, ws->ctr, ws->ngeo, ws->nlink, ws->mom64, cap,
-                                             (const typename AdjVec<Real>::V4 *)ws->spos, ws->adj_ccot, ws->adj_xg,
+                                             (const typename Vec4<Real>::T *)ws->spos, ws->adj_ccot, ws->adj_xg,
                                              ws->adj_mg, n);
-    k_grad_scatter<Real><<<nb, 256, 0, s>>>(ws->adj_xt, ws->adj_xg, ws->adj_mg, ws->idx, n, (Real *)xbar,
+    k_grad_scatter<Real><<<nb, 256, 0, s>>>(ws->adj_xg, ws->adj_mg, ws->idx, n, (Real *)xbar,
                                             (Real *)mbar, ws->ctr);
     ws->launches += 3 + kLevels;
     return cudaGetLastError();

@@ -74,7 +74,7 @@ void free_all(TreeWorkspace *ws) {
                     ws->mom64, ws->mom_a, ws->mom_b, ws->mom_c, ws->dstatus, ws->stats, ws->gstat,
                     ws->list_cnt, ws->pc_list, ws->pp_list, ws->direct_part, ws->dmac, ws->gorder,
                     ws->gkey, ws->gbucket, ws->gfirst, ws->plev, ws->ccount, ws->coff, ws->gscan_status,
-                    ws->adj_cot, ws->adj_xt, ws->adj_xg, ws->adj_mg, ws->adj_ccot, ws->pleaf, ws->nparent,
+                    ws->adj_cot, ws->adj_xg, ws->adj_mg, ws->adj_ccot, ws->pleaf, ws->nparent,
                     ws->seg_off, ws->seg_cstart, ws->seg_bchunk, ws->seg_bfirst, ws->seg_part,
                     ws->seg_digit_off, ws->cmask, ws->morder, ws->mbucket, ws->xm, ws->hs_x, ws->hs_v,
                     ws->hs_m, ws->hs_a, ws->hs_phi, ws->hs_diag, ws->dctl, ws->tile_hdr, ws->tile_idx,
@@ -572,13 +572,13 @@ tree_status_t tree_forces(TreeWorkspace *ws, void *a, void *phi, int32_t flags, 
 
 static tree_status_t adjoint_ready(TreeWorkspace *ws) {
     if (!ws->has_moments || ws->list_groups < 0) return TREE_ERR_STATE;
-    if (!ws->adj_xt) {
-        const size_t N = (size_t)ws->n_max, NC = (size_t)ws->node_cap;
-        const size_t v4 = ws->p.precision == TREE_F64 ? sizeof(double4a) : sizeof(float4);
-        if (!(dalloc((unsigned char **)&ws->adj_cot, N * v4) && dalloc(&ws->adj_xt, 3 * N) &&
-              dalloc(&ws->adj_xg, 3 * N) && dalloc(&ws->adj_mg, N) && dalloc(&ws->adj_ccot, 10 * NC))) {
-            return TREE_ERR_ALLOC;
-        }
+    const size_t N = (size_t)ws->n_max, NC = (size_t)ws->node_cap;
+    const size_t v4 = ws->p.precision == TREE_F64 ? sizeof(double4a) : sizeof(float4);
+    if (!((ws->adj_cot || dalloc((unsigned char **)&ws->adj_cot, N * v4)) &&
+          (ws->adj_xg || dalloc(&ws->adj_xg, 3 * N)) && (ws->adj_mg || dalloc(&ws->adj_mg, N)) &&
+          (ws->adj_ccot || dalloc(&ws->adj_ccot, 10 * NC)))) {
+        cudaGetLastError();
+        return TREE_ERR_ALLOC;
     }
     return TREE_OK;
 }

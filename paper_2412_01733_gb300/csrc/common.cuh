@@ -215,7 +215,7 @@ struct TreeWorkspace {
     int64_t list_groups_host = 0;      // group count used by the last list emission
     // adjoint scratch (allocated on first use)
     void *adj_cot = nullptr;           // Vec4 (abar, phibar) in key order
-    double *adj_xt = nullptr, *adj_xg = nullptr, *adj_mg = nullptr, *adj_ccot = nullptr;
+    double *adj_xg = nullptr, *adj_mg = nullptr, *adj_ccot = nullptr;
     // direct-sum scratch
     double *direct_part = nullptr;
     size_t direct_part_bytes = 0;
