@@ -11,14 +11,12 @@
 //   PC pair (cell C, y = r_i - R): derivative of the cell expansion with
 //     respect to y (xbar_i += ybar, Rbar_C -= ybar), M and the six stored
 //     quadrupole components.
-//   Cell cotangents travel down the moment tree: with d = R_child - R_parent
-//     (or r_j - R for the members of a leaf), Qf the symmetric matrix of the
-//     stored-component cotangent (off-diagonals halved) and
-//     f(d) = 3 d.Qf.d - |d|^2 tr Qf:
-//       Mbar_child += Mbar + d.Rbar / M + f(d),
-//       Rbar_child += (M_child / M) Rbar + M_child (6 Qf d - 2 tr(Qf) d),
-//       Qbar_child += Qbar  (the children's quadrupoles enter Q linearly);
-//     a massless cell passes only Mbar.
+//   Cell cotangents reach the particles of the cell: with d = r_j - R, Qf the
+//     symmetric matrix of the stored-component cotangent (off-diagonals
+//     halved) and f(d) = 3 d.Qf.d - |d|^2 tr Qf:
+//       mbar_j += Mbar + d.Rbar / M + f(d),
+//       xbar_j += m_j (Rbar / M + 6 Qf d - 2 tr(Qf) d);
+//     a massless cell passes only Mbar (k_cot_paths).
 // One warp per group walks the group's stored lists, 32 sources (cells or
 // particles) at a time, one source per lane.  Each (target, source) pair is
 // evaluated once: the source-side cotangents (cell or particle) are summed in
@@ -370,86 +368,99 @@ __global__ void __launch_bounds__(256) k_cot_gather(const Real *__restrict__ aba
     }
 }
 
-// Level L of the top-down cotangent push (see the header comment).
-template <typename Real>
-__global__ void __launch_bounds__(256) k_cot_push(int L, const uint32_t *__restrict__ ctr,
-                                                  const uint4 *__restrict__ ngeo, const uint2 *__restrict__ nlink,
-                                                  const double *__restrict__ mom64, int64_t cap,
-                                                  const typename Vec4<Real>::T *__restrict__ spos,
-                                                  double *__restrict__ ccot, double *__restrict__ xg,
-                                                  double *__restrict__ mg, int64_t n) {
+// Cell cotangents back to the particles.  What a cell's cotangents give a
+// particle at r is a quadratic polynomial, with d = r - R:
+//   P(d) = Mbar + d.Rbar / M + 3 d.Qf.d - |d|^2 tr Qf,
+// P itself to mbar and m grad P to xbar (the chain of the moment tree, cell by
+// cell, composes to just that, the moments being exact sums over the cell's
+// particles).  A massless cell passes only Mbar on, so what is above one acts
+// through its value at that cell's R.  So a leaf adds up the polynomials of
+// its ancestors, shifted to its own R, in one launch without order (top-down,
+// level by level, this was 22 launches and 0.83 ms at N = 262144), and leaves
+// the sum in its own row: a; gx, gy, gz; hxx, hyy, hzz, hxy, hxz, hyz with
+// P = a + g.d + d.h.d (h symmetric).
+__global__ void __launch_bounds__(128) k_cot_paths(const uint32_t *__restrict__ ctr, const uint4 *__restrict__ ngeo,
+                                                   const uint32_t *__restrict__ nparent,
+                                                   const double *__restrict__ mom64, int64_t cap, int64_t nseg,
+                                                   double *ccot) {
     if (aborted(ctr, kStageAfter)) return;
-    const uint32_t start = ctr[kCtrLevelStart + L], end = ctr[kCtrLevelStart + L + 1];
-    for (uint32_t node = start + blockIdx.x * blockDim.x + threadIdx.x; node < end;
-         node += gridDim.x * blockDim.x) {
-        double cb[10];
-        bool nz = false;
+    const uint32_t nn = ctr[kCtrLevelStart + kLevels];
+    for (uint32_t leaf = blockIdx.x * blockDim.x + threadIdx.x; leaf < nn; leaf += gridDim.x * blockDim.x) {
+        if (!((ngeo[leaf].w >> 8) & 1u)) continue;
+        const double *R = mom64 + cap;
+        double px = R[leaf], py = R[cap + leaf], pz = R[2 * cap + leaf];  // where the sum is centred
+        double a = 0, gx = 0, gy = 0, gz = 0, hxx = 0, hyy = 0, hzz = 0, hxy = 0, hxz = 0, hyz = 0;
+        bool value = false;  // below a massless cell: only the value at its R counts
+        for (uint32_t c = leaf;;) {
+            const uint32_t up = nparent[c];
+            double q[10];
+            bool any = false;
 #pragma unroll
-        for (int k = 0; k < 10; ++k) {
-            cb[k] = ccot[(int64_t)k * cap + node];
-            nz |= cb[k] != 0.0;
+            for (int k = 0; k < 10; ++k) {
+                q[k] = ccot[(int64_t)k * cap + c];
+                any |= q[k] != 0.0;
+            }
+            const double M = mom64[c];
+            if (any) {
+                a += q[0];
+                if (M != 0.0) {
+                    const double iM = 1.0 / M;
+                    const double bx = q[1] * iM, by = q[2] * iM, bz = q[3] * iM;
+                    const double tr = q[4] + q[5] + q[6];
+                    const double sxx = 3.0 * q[4] - tr, syy = 3.0 * q[5] - tr, szz = 3.0 * q[6] - tr;
+                    const double sxy = 1.5 * q[7], sxz = 1.5 * q[8], syz = 1.5 * q[9];
+                    const double dx = px - R[c], dy = py - R[cap + c], dz = pz - R[2 * cap + c];
+                    const double fx = sxx * dx + sxy * dy + sxz * dz, fy = sxy * dx + syy * dy + syz * dz,
+                                 fz = sxz * dx + syz * dy + szz * dz;
+                    a += dx * (bx + fx) + dy * (by + fy) + dz * (bz + fz);
+                    if (!value) {
+                        gx += bx + 2.0 * fx; gy += by + 2.0 * fy; gz += bz + 2.0 * fz;
+                        hxx += sxx; hyy += syy; hzz += szz;
+                        hxy += sxy; hxz += sxz; hyz += syz;
+                    }
+                }
+            }
+            if (M == 0.0) {
+                value = true;
+                px = R[c]; py = R[cap + c]; pz = R[2 * cap + c];
+            }
+            if (c < (uint32_t)nseg) break;
+            c = up;
         }
-        if (!nz) continue;
-        const uint4 geo = ngeo[node];
-        const uint2 lk = nlink[node];
-        const bool leaf = (geo.w >> 8) & 1u;
-        const double M = mom64[node];
-        const double Rx = mom64[cap + node], Ry = mom64[2 * cap + node], Rz = mom64[3 * cap + node];
-        const double fxx = cb[4], fyy = cb[5], fzz = cb[6];
-        const double fxy = 0.5 * cb[7], fxz = 0.5 * cb[8], fyz = 0.5 * cb[9];
-        const double tr = fxx + fyy + fzz;
-        const bool massive = M != 0.0;
-        const double iM = massive ? 1.0 / M : 0.0;
-        for (uint32_t k = lk.x; k < lk.x + lk.y; ++k) {
-            double mk, dx, dy, dz;
-            if (leaf) {
-                const typename Vec4<Real>::T p = spos[k];
-                mk = (double)p.w;
-                dx = (double)p.x - Rx; dy = (double)p.y - Ry; dz = (double)p.z - Rz;
-            } else {
-                mk = mom64[k];
-                dx = mom64[cap + k] - Rx; dy = mom64[2 * cap + k] - Ry; dz = mom64[3 * cap + k] - Rz;
-            }
-            double dM = cb[0], gx = 0, gy = 0, gz = 0;
-            if (massive) {
-                const double Fx = fxx * dx + fxy * dy + fxz * dz;
-                const double Fy = fxy * dx + fyy * dy + fyz * dz;
-                const double Fz = fxz * dx + fyz * dy + fzz * dz;
-                const double d2 = dx * dx + dy * dy + dz * dz;
-                dM += (dx * cb[1] + dy * cb[2] + dz * cb[3]) * iM + 3.0 * (dx * Fx + dy * Fy + dz * Fz) - d2 * tr;
-                const double wgt = mk * iM;
-                gx = wgt * cb[1] + mk * (6.0 * Fx - 2.0 * tr * dx);
-                gy = wgt * cb[2] + mk * (6.0 * Fy - 2.0 * tr * dy);
-                gz = wgt * cb[3] + mk * (6.0 * Fz - 2.0 * tr * dz);
-            }
-            if (leaf) {
-                mg[k] += dM;
-                xg[k] += gx; xg[n + k] += gy; xg[2 * n + k] += gz;
-            } else {
-                ccot[k] += dM;
-                ccot[cap + k] += gx; ccot[2 * cap + k] += gy; ccot[3 * cap + k] += gz;
-                if (massive)
-                    for (int q = 0; q < 6; ++q) ccot[(int64_t)(4 + q) * cap + k] += cb[4 + q];
-            }
-        }
+        const double out[10] = {a, gx, gy, gz, hxx, hyy, hzz, hxy, hxz, hyz};
+#pragma unroll
+        for (int k = 0; k < 10; ++k) ccot[(int64_t)k * cap + leaf] = out[k];
     }
 }
 
-// xbar[i] += xg, mbar[i] += mg (key order -> caller order)
+// xbar[i] += xg + m grad P, mbar[i] += mg + P (key order -> caller order), P of
+// the particle's leaf.
 template <typename Real>
 __global__ void __launch_bounds__(256) k_grad_scatter(const double *__restrict__ xg, const double *__restrict__ mg,
-                                                      const uint32_t *__restrict__ perm,
-                                                      int64_t n, Real *__restrict__ xbar, Real *__restrict__ mbar,
+                                                      const double *__restrict__ ccot,
+                                                      const double *__restrict__ mom64, int64_t cap,
+                                                      const uint32_t *__restrict__ pleaf,
+                                                      const typename Vec4<Real>::T *__restrict__ spos,
+                                                      const uint32_t *__restrict__ perm, int64_t n,
+                                                      Real *__restrict__ xbar, Real *__restrict__ mbar,
                                                       const uint32_t *__restrict__ ctr) {
     if (aborted(ctr, kStageAfter)) return;
     for (int64_t s = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; s < n; s += (int64_t)gridDim.x * blockDim.x) {
-        const uint32_t i = perm[s];
+        const uint32_t i = perm[s], c = pleaf[s];
+        const typename Vec4<Real>::T p = spos[s];
+        double q[10];
+#pragma unroll
+        for (int k = 0; k < 10; ++k) q[k] = ccot[(int64_t)k * cap + c];
+        const double dx = (double)p.x - mom64[cap + c], dy = (double)p.y - mom64[2 * cap + c],
+                     dz = (double)p.z - mom64[3 * cap + c], m = (double)p.w;
+        const double fx = q[4] * dx + q[7] * dy + q[8] * dz, fy = q[7] * dx + q[5] * dy + q[9] * dz,
+                     fz = q[8] * dx + q[9] * dy + q[6] * dz;
         if (xbar) {
-            xbar[i] += (Real)xg[s];
-            xbar[n + i] += (Real)xg[n + s];
-            xbar[2 * n + i] += (Real)xg[2 * n + s];
+            xbar[i] += (Real)(xg[s] + m * (q[1] + 2.0 * fx));
+            xbar[n + i] += (Real)(xg[n + s] + m * (q[2] + 2.0 * fy));
+            xbar[2 * n + i] += (Real)(xg[2 * n + s] + m * (q[3] + 2.0 * fz));
         }
-        if (mbar) mbar[i] += (Real)mg[s];
+        if (mbar) mbar[i] += (Real)(mg[s] + q[0] + dx * (q[1] + fx) + dy * (q[2] + fy) + dz * (q[3] + fz));
     }
 }
 
@@ -493,14 +504,12 @@ static cudaError_t adjoint_impl(TreeWorkspace *ws, const void *abar, const void 
             else k_force_vjp<Real, false, false><<<gb, kAdjWarps * 32, 0, s>>>(A);
         }
     }
-    const int nbn = grid_for(ws->node_cap, 256, 152 * 8);
-    for (int L = 0; L < kLevels; ++L)
-        k_cot_push<Real><<<nbn, 256, 0, s>>>(L, ws->ctr, ws->ngeo, ws->nlink, ws->mom64, cap,
-                                             (const typename Vec4<Real>::T *)ws->spos, ws->adj_ccot, ws->adj_xg,
-                                             ws->adj_mg, n);
-    k_grad_scatter<Real><<<nb, 256, 0, s>>>(ws->adj_xg, ws->adj_mg, ws->idx, n, (Real *)xbar,
+    k_cot_paths<<<grid_for(cap, 128, 152 * 16), 128, 0, s>>>(ws->ctr, ws->ngeo, ws->nparent, ws->mom64, cap, ws->nseg,
+                                                              ws->adj_ccot);
+    k_grad_scatter<Real><<<nb, 256, 0, s>>>(ws->adj_xg, ws->adj_mg, ws->adj_ccot, ws->mom64, cap, ws->pleaf,
+                                            (const typename Vec4<Real>::T *)ws->spos, ws->idx, n, (Real *)xbar,
                                             (Real *)mbar, ws->ctr);
-    ws->launches += 3 + kLevels;
+    ws->launches += 4;
     return cudaGetLastError();
 }
 
