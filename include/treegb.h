@@ -375,7 +375,10 @@ tree_status_t tree_direct_forces_noalloc(const void *x, const void *m, int64_t n
  * (default 2e9 cycles, about 1 s); 0 keeps it.  withhold_pass and
  * withhold_tile >= 0 make that tile of that sort pass (0..9) skip publishing
  * its look-back words, so the tiles after it run into the limit: a test of
- * the timeout path that needs no fault; -1 for both turns it off.
+ * the timeout path that needs no fault; -1 for both turns it off.  (While
+ * it is on, builds of up to 65536 particles sort in those passes too, which
+ * they otherwise do in one launch without waits; a step captured before keeps
+ * the form it was captured in.)
  * Synchronises the device.  Errors: TREE_ERR_ARG. */
 tree_status_t tree_set_waits(TreeWorkspace *ws, int64_t wait_cycles, int32_t withhold_pass, int64_t withhold_tile);
 

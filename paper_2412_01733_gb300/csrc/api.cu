@@ -440,6 +440,21 @@ tree_status_t tree_get_params(const TreeWorkspace *ws, TreeParams *p) {
     return TREE_OK;
 }
 
+// Clears the counters and look-back words that the build's kernels start from.
+static cudaError_t clear_build(TreeWorkspace *ws, int64_t n, cudaStream_t s) {
+    cudaError_t e = cudaMemsetAsync(ws->ctr, 0, kCtrCount * sizeof(uint32_t), s);
+    if (e == cudaSuccess && !small_sort(ws, n)) {
+        const size_t word = sizeof(uint32_t), tiles = (size_t)((n + kSortTile - 1) / kSortTile);
+        e = cudaMemsetAsync(ws->hist, 0, kSortPasses * kRadix * word, s);
+        if (e == cudaSuccess)
+            e = cudaMemset2DAsync(ws->sort_status, (size_t)ws->sort_tiles_max * kRadix * word, 0, tiles * kRadix * word,
+                                  (size_t)(kSortPasses + ws->seg_passes), s);
+    }
+    if (e == cudaSuccess && !flat_octree(ws, n))
+        e = cudaMemsetAsync(ws->level_status, 0, (size_t)kLevels * ws->level_tiles_max * sizeof(uint32_t), s);
+    return e;
+}
+
 tree_status_t tree_build(TreeWorkspace *ws, const void *x, int64_t n, int32_t dtype, void *stream) {
     if (!ws) return TREE_ERR_ARG;
     tree_status_t stn = check_n(ws, n);
@@ -452,13 +467,7 @@ tree_status_t tree_build(TreeWorkspace *ws, const void *x, int64_t n, int32_t dt
     ws->has_moments = false;
     ws->list_groups = -1;
     if (n == 0) { ws->built = true; return TREE_OK; }
-    const int64_t tiles = (n + kSortTile - 1) / kSortTile;
-    TRY_CUDA(cudaMemsetAsync(ws->ctr, 0, kCtrCount * sizeof(uint32_t), s));
-    TRY_CUDA(cudaMemsetAsync(ws->hist, 0, kSortPasses * kRadix * sizeof(uint32_t), s));
-    for (int p = 0; p < kSortPasses + ws->seg_passes; ++p)
-        TRY_CUDA(cudaMemsetAsync(ws->sort_status + (size_t)p * ws->sort_tiles_max * kRadix, 0,
-                                 (size_t)tiles * kRadix * sizeof(uint32_t), s));
-    TRY_CUDA(cudaMemsetAsync(ws->level_status, 0, (size_t)kLevels * ws->level_tiles_max * sizeof(uint32_t), s));
+    TRY_CUDA(clear_build(ws, n, s));
     {
         PhaseScope ph(ws, TREE_PHASE_BOX, s);
         TRY_CUDA(launch_box(ws, x, n, s));
@@ -646,13 +655,7 @@ static tree_status_t leapfrog_begin(TreeWorkspace *ws, void *x, void *v, const v
     ws->built = false;
     ws->has_moments = false;
     ws->list_groups = -1;
-    const int64_t tiles = (n + kSortTile - 1) / kSortTile;
-    TRY_CUDA(cudaMemsetAsync(ws->ctr, 0, kCtrCount * sizeof(uint32_t), s));
-    TRY_CUDA(cudaMemsetAsync(ws->hist, 0, kSortPasses * kRadix * sizeof(uint32_t), s));
-    for (int p = 0; p < kSortPasses + ws->seg_passes; ++p)
-        TRY_CUDA(cudaMemsetAsync(ws->sort_status + (size_t)p * ws->sort_tiles_max * kRadix, 0,
-                                 (size_t)tiles * kRadix * sizeof(uint32_t), s));
-    TRY_CUDA(cudaMemsetAsync(ws->level_status, 0, (size_t)kLevels * ws->level_tiles_max * sizeof(uint32_t), s));
+    TRY_CUDA(clear_build(ws, n, s));
     // Eqs. 2-3 fused with the box of the new positions
     PhaseScope ph(ws, TREE_PHASE_BOX, s);
     TRY_CUDA(launch_kick_drift_box(ws, x, v, a, m, tau, n, s));
@@ -1102,6 +1105,7 @@ tree_status_t tree_set_waits(TreeWorkspace *ws, int64_t wait_cycles, int32_t wit
     if (wait_cycles > 0) ctl.wait_cycles = wait_cycles;
     ctl.withhold = withhold_pass < 0 ? -1 : (((long long)withhold_pass << 32) | (long long)withhold_tile);
     TRY_CUDA(cudaMemcpy(ws->dctl, &ctl, sizeof(ctl), cudaMemcpyHostToDevice));
+    ws->withhold = withhold_pass >= 0;
     return TREE_OK;
 }
 

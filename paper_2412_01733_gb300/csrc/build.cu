@@ -56,25 +56,6 @@ __global__ void __launch_bounds__(256) k_box_partial(const Real *__restrict__ x,
     }
 }
 
-// lo = min, ext = max_d (hi_d - lo_d) in FP64, L = 2^k the smallest power of
-// two strictly greater than ext (k = 0 when ext = 0): with ext = f 2^e,
-// f in [0.5, 1), that power is 2^e.
-__device__ void box_from_minmax(double (&lo)[3], double (&hi)[3], DevBox *box) {
-    double ext = 0.0;
-    for (int d = 0; d < 3; ++d) {
-        if (!(lo[d] <= hi[d])) { lo[d] = 0.0; hi[d] = 0.0; }  // no finite value on this axis
-        double e = __dsub_rn(hi[d], lo[d]);
-        if (e > ext) ext = e;
-    }
-    int k = 0;
-    if (ext > 0.0) frexp(ext, &k);
-    for (int d = 0; d < 3; ++d) box->lo[d] = lo[d];
-    box->k = k;
-    box->r5fit = 0;  // decided after the moments
-    box->scale = ldexp(1.0, kBits - k);
-    box->unit = ldexp(1.0, k - kBits);
-}
-
 // One block: each thread folds a strided share of the partials, then the
 // block folds the threads (min and max are exact in any order).
 __global__ void __launch_bounds__(256) k_box_final(const double *__restrict__ part, int nblocks, DevBox *box) {
@@ -106,7 +87,9 @@ __global__ void __launch_bounds__(256) k_box_final(const double *__restrict__ pa
     }
 }
 
-cudaError_t launch_box_final(TreeWorkspace *ws, int nblocks, cudaStream_t s) {
+cudaError_t launch_box_final(TreeWorkspace *ws, int nblocks, int64_t n, cudaStream_t s) {
+    ws->box_parts = nblocks;
+    if (small_sort(ws, n)) return cudaGetLastError();  // k_small_keys folds the partials
     k_box_final<<<1, 256, 0, s>>>(ws->part, nblocks, ws->box);
     ws->launches += 1;
     return cudaGetLastError();
@@ -222,7 +205,7 @@ static cudaError_t box_impl(TreeWorkspace *ws, const Real *x, int64_t n, cudaStr
     const int nb = wave_grid(k_box_partial<Real>, n, 256, kMaxBlocksReduce);
     k_box_partial<Real><<<nb, 256, 0, s>>>(x, n, ws->part, ws->dstatus);
     ws->launches += 1;
-    return launch_box_final(ws, nb, s);
+    return launch_box_final(ws, nb, n, s);
 }
 
 cudaError_t launch_box(TreeWorkspace *ws, const void *x, int64_t n, cudaStream_t s) {
@@ -239,22 +222,6 @@ cudaError_t launch_box(TreeWorkspace *ws, const void *x, int64_t n, cudaStream_t
 // eight 8-bit digits of every key for the radix sort (warp-aggregated
 // shared-memory atomics).
 // SEG: every particle is quantised in the box of its own segment.
-
-// The floor and both clamps are one saturating round-down conversion
-// (cvt.rmi.u32.f64 clamps out-of-range values, negatives to 0) and an integer
-// min; a NaN lands in some in-range cell (the box pass has already raised
-// TREE_DEV_NONFINITE for it).
-__device__ __forceinline__ uint32_t quantize(double x, double lo, double sc) {
-    return min(__double2uint_rd(__dmul_rn(__dsub_rn(x, lo), sc)), (1u << kBits) - 1u);
-}
-// FP32 coordinates: x sc and lo sc are exact in FP64 (a float, or the box
-// corner, times a power of two stays far inside the FP64 range), so one fused
-// multiply-add, x sc - lo sc, rounds (x - lo) sc exactly as the FP64
-// subtraction followed by the exact scaling does: the same q_d with a third
-// of the FP64 instructions (the FP64 pipe runs at 1/64 of the FP32 rate here).
-__device__ __forceinline__ uint32_t quantize(float x, double lo, double sc) {
-    return min(__double2uint_rd(fma((double)x, sc, -(lo * sc))), (1u << kBits) - 1u);
-}
 
 template <typename Real, bool SEG>
 __global__ void __launch_bounds__(256) k_keys(const Real *__restrict__ x, int64_t n,
@@ -472,11 +439,13 @@ static cudaError_t keys_impl(TreeWorkspace *ws, const Real *x, int64_t n, cudaSt
 }
 
 cudaError_t launch_keys(TreeWorkspace *ws, const void *x, int64_t n, cudaStream_t s) {
+    if (small_sort(ws, n)) return launch_small_keys(ws, x, n, s);
     if (ws->p.precision == TREE_F64) return keys_impl(ws, (const double *)x, n, s);
     return keys_impl(ws, (const float *)x, n, s);
 }
 
 cudaError_t launch_sort(TreeWorkspace *ws, int64_t n, cudaStream_t s) {
+    if (small_sort(ws, n)) return launch_small_sort(ws, n, s);
     const int64_t tiles = (n + kSortTile - 1) / kSortTile;
     const size_t smem = sizeof(SortSmem);
     static bool attr_done[64] = {};

@@ -2,6 +2,7 @@
 #pragma once
 
 #include <cuda_runtime.h>
+#include <float.h>
 #include <math.h>
 #include <stdint.h>
 
@@ -24,6 +25,7 @@ constexpr int kSegPassesMax = 2;   // extra passes over the segment index (ensem
 constexpr int kMaxSegments = 65536;
 constexpr int kBoxChunk = 8192;    // particles per partial box of a segmented reduction
 constexpr int kRadix = 256;
+constexpr int64_t kSmallSortMax = 65536;  // particles sorted by one cluster (sort_small.cu)
 constexpr int kLevelThreads = 256;  // octree level block (nodes per tile)
 constexpr int kMaxBlocksReduce = 1024;  // partial-result slots of the reductions
 constexpr int kMaxLeafSmall = 16;   // leaves up to this size are expanded in the walk buffer
@@ -137,6 +139,8 @@ struct TreeWorkspace {
     uint32_t *level_status = nullptr;  // [22][level_tiles]
     uint32_t *ctr = nullptr;           // kCtrCount words
     // box
+    int box_parts = 0;                 // partial boxes of the last box reduction
+    bool withhold = false;             // tree_set_waits has a sort tile withhold its words (test injection)
     double *part = nullptr;            // reduction partials [kMaxBlocksReduce][8]
     treegb::DevBox *box = nullptr;     // one per segment
     // segments (independent systems sharing one build; nseg = 1: a single system of any n)
@@ -464,6 +468,41 @@ __device__ __forceinline__ void octant_bounds(const uint64_t *__restrict__ skey,
     b[8] = first + count;
 }
 
+// lo = min, ext = max_d (hi_d - lo_d) in FP64, L = 2^k the smallest power of
+// two strictly greater than ext (k = 0 when ext = 0): with ext = f 2^e,
+// f in [0.5, 1), that power is 2^e.
+__device__ inline void box_from_minmax(double (&lo)[3], double (&hi)[3], DevBox *box) {
+    double ext = 0.0;
+    for (int d = 0; d < 3; ++d) {
+        if (!(lo[d] <= hi[d])) { lo[d] = 0.0; hi[d] = 0.0; }  // no finite value on this axis
+        double e = __dsub_rn(hi[d], lo[d]);
+        if (e > ext) ext = e;
+    }
+    int k = 0;
+    if (ext > 0.0) frexp(ext, &k);
+    for (int d = 0; d < 3; ++d) box->lo[d] = lo[d];
+    box->k = k;
+    box->r5fit = 0;  // decided after the moments
+    box->scale = ldexp(1.0, kBits - k);
+    box->unit = ldexp(1.0, k - kBits);
+}
+
+// The floor and both clamps are one saturating round-down conversion
+// (cvt.rmi.u32.f64 clamps out-of-range values, negatives to 0) and an integer
+// min; a NaN lands in some in-range cell (the box pass has already raised
+// TREE_DEV_NONFINITE for it).
+__device__ __forceinline__ uint32_t quantize(double x, double lo, double sc) {
+    return min(__double2uint_rd(__dmul_rn(__dsub_rn(x, lo), sc)), (1u << kBits) - 1u);
+}
+// FP32 coordinates: x sc and lo sc are exact in FP64 (a float, or the box
+// corner, times a power of two stays far inside the FP64 range), so one fused
+// multiply-add, x sc - lo sc, rounds (x - lo) sc exactly as the FP64
+// subtraction followed by the exact scaling does: the same q_d with a third
+// of the FP64 instructions (the FP64 pipe runs at 1/64 of the FP32 rate here).
+__device__ __forceinline__ uint32_t quantize(float x, double lo, double sc) {
+    return min(__double2uint_rd(fma((double)x, sc, -(lo * sc))), (1u << kBits) - 1u);
+}
+
 inline int grid_for(int64_t n, int threads, int max_blocks) {
     int64_t b = (n + threads - 1) / threads;
     if (b < 1) b = 1;
@@ -494,12 +533,20 @@ inline int wave_grid(Kernel k, int64_t n, int threads, int max_blocks, size_t sm
 namespace treegb {
 // build.cu
 cudaError_t launch_box(TreeWorkspace *ws, const void *x, int64_t n, cudaStream_t s);
-cudaError_t launch_box_final(TreeWorkspace *ws, int nblocks, cudaStream_t s);
+cudaError_t launch_box_final(TreeWorkspace *ws, int nblocks, int64_t n, cudaStream_t s);
 cudaError_t launch_box_segments(TreeWorkspace *ws, void *x, void *v, const void *a, const void *m, double tau,
                                 int64_t n, bool kick, cudaStream_t s);
 cudaError_t launch_keys(TreeWorkspace *ws, const void *x, int64_t n, cudaStream_t s);
 cudaError_t launch_sort(TreeWorkspace *ws, int64_t n, cudaStream_t s);
 cudaError_t launch_octree(TreeWorkspace *ws, int64_t n, cudaStream_t s);
+// sort_small.cu
+cudaError_t launch_small_keys(TreeWorkspace *ws, const void *x, int64_t n, cudaStream_t s);
+cudaError_t launch_small_sort(TreeWorkspace *ws, int64_t n, cudaStream_t s);
+// Whether keys and sort take the one-cluster form: one small system, and no
+// onesweep tile to withhold.
+inline bool small_sort(const TreeWorkspace *ws, int64_t n) {
+    return ws->nseg == 1 && n <= kSmallSortMax && !ws->withhold;
+}
 // octree_flat.cu
 int64_t flat_octree_max();
 cudaError_t launch_octree_flat(TreeWorkspace *ws, int64_t n, cudaStream_t s);

@@ -171,8 +171,10 @@ cudaError_t launch_groups(TreeWorkspace *ws, int64_t n, cudaStream_t s) {
     const int gs = ws->p.group_size;
     const int64_t nchunks = ws->nseg > 1 ? ws->seg_nchunks : (n + gs - 1) / gs;
     const int64_t tiles = (nchunks + kGScanTile - 1) / kGScanTile;
-    cudaError_t e = cudaMemsetAsync(ws->gscan_status, 0, (size_t)tiles * sizeof(uint32_t), s);
-    if (e != cudaSuccess) return e;
+    if (tiles > 1) {  // (a single tile looks at nobody's word)
+        const cudaError_t e = cudaMemsetAsync(ws->gscan_status, 0, (size_t)tiles * sizeof(uint32_t), s);
+        if (e != cudaSuccess) return e;
+    }
     if (!flat_octree(ws, n)) {
         k_leaf_levels<<<grid_for(ws->node_cap, 256, 152 * 8), 256, 0, s>>>(ws->ctr, ws->ngeo, ws->nlink, ws->plev,
                                                                             ws->pleaf);

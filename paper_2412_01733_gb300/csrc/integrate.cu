@@ -83,7 +83,7 @@ cudaError_t launch_kick_drift_box(TreeWorkspace *ws, void *x, void *v, const voi
                                                    ws->dstatus);
     }
     ws->launches += 1;
-    return launch_box_final(ws, nb, s);
+    return launch_box_final(ws, nb, n, s);
 }
 
 // ============================================================== diagnostics (FP64)
