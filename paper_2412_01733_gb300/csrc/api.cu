@@ -455,6 +455,31 @@ static cudaError_t clear_build(TreeWorkspace *ws, int64_t n, cudaStream_t s) {
     return e;
 }
 
+// Keys, sort and octree of positions whose box (or its partials) is known.
+static tree_status_t sort_and_octree(TreeWorkspace *ws, const void *x, int64_t n, cudaStream_t s) {
+    {
+        PhaseScope ph(ws, TREE_PHASE_KEYS, s);
+        TRY_CUDA(launch_keys(ws, x, n, s));
+    }
+    {
+        PhaseScope ph(ws, TREE_PHASE_SORT, s);
+        TRY_CUDA(launch_sort(ws, n, s));
+    }
+    PhaseScope ph(ws, TREE_PHASE_OCTREE, s);
+    TRY_CUDA(launch_octree(ws, n, s));
+    return TREE_OK;
+}
+
+// Everything of a build but the walk groups.
+static tree_status_t build_octree(TreeWorkspace *ws, const void *x, int64_t n, cudaStream_t s) {
+    TRY_CUDA(clear_build(ws, n, s));
+    {
+        PhaseScope ph(ws, TREE_PHASE_BOX, s);
+        TRY_CUDA(launch_box(ws, x, n, s));
+    }
+    return sort_and_octree(ws, x, n, s);
+}
+
 tree_status_t tree_build(TreeWorkspace *ws, const void *x, int64_t n, int32_t dtype, void *stream) {
     if (!ws) return TREE_ERR_ARG;
     tree_status_t stn = check_n(ws, n);
@@ -467,24 +492,10 @@ tree_status_t tree_build(TreeWorkspace *ws, const void *x, int64_t n, int32_t dt
     ws->has_moments = false;
     ws->list_groups = -1;
     if (n == 0) { ws->built = true; return TREE_OK; }
-    TRY_CUDA(clear_build(ws, n, s));
-    {
-        PhaseScope ph(ws, TREE_PHASE_BOX, s);
-        TRY_CUDA(launch_box(ws, x, n, s));
-    }
-    {
-        PhaseScope ph(ws, TREE_PHASE_KEYS, s);
-        TRY_CUDA(launch_keys(ws, x, n, s));
-    }
-    {
-        PhaseScope ph(ws, TREE_PHASE_SORT, s);
-        TRY_CUDA(launch_sort(ws, n, s));
-    }
-    {
-        PhaseScope ph(ws, TREE_PHASE_OCTREE, s);
-        TRY_CUDA(launch_octree(ws, n, s));
-        TRY_CUDA(launch_groups(ws, n, s));
-    }
+    tree_status_t st = build_octree(ws, x, n, s);
+    if (st != TREE_OK) return st;
+    PhaseScope ph(ws, TREE_PHASE_OCTREE, s);
+    TRY_CUDA(launch_groups(ws, n, s));
     ws->built = true;
     return TREE_OK;
 }
@@ -511,14 +522,15 @@ static tree_status_t walk(TreeWorkspace *ws, int mode, WalkOut out, cudaStream_t
     tree_status_t st = upload_mac(ws, s);
     if (st != TREE_OK) return st;
     PhaseScope ph(ws, mode == kWalkForce ? TREE_PHASE_WALK : TREE_PHASE_LISTS, s);
-    // (the split walk has no straggler to put first)
-    const bool split = mode == kWalkForce && walk_splits(ws);
-    out.ordered = walk_widest_first(ws) && !split;
+    if (mode == kWalkForce && walk_splits(ws)) {
+        // (the split walk has no straggler to put first)
+        TRY_CUDA(launch_walk_split(ws, kWalkTiles, out, s));
+        TRY_CUDA(launch_walk_split(ws, kWalkFold, out, s));
+        return TREE_OK;
+    }
+    out.ordered = walk_widest_first(ws);
     if (out.ordered) TRY_CUDA(launch_group_order(ws, s));
-    if (split) {
-        if (ws->p.precision == TREE_F64) TRY_CUDA(launch_walk_split_f64(ws, out, s));
-        else TRY_CUDA(launch_walk_split_f32(ws, out, s));
-    } else if (ws->p.precision == TREE_F64) TRY_CUDA(launch_walk_f64(ws, mode, out, s));
+    if (ws->p.precision == TREE_F64) TRY_CUDA(launch_walk_f64(ws, mode, out, s));
     else TRY_CUDA(launch_walk_f32(ws, mode, out, s));
     return TREE_OK;
 }
@@ -627,24 +639,83 @@ tree_status_t tree_energy_vjp(TreeWorkspace *ws, const void *m, const void *phi,
     return TREE_OK;
 }
 
-tree_status_t tree_accel(TreeWorkspace *ws, const void *x, const void *m, int64_t n, void *a, void *phi,
-                         void *stream) {
-    if (!ws) return TREE_ERR_ARG;
-    if (n > 0 && (!x || !m || !a)) return TREE_ERR_ARG;
-    tree_status_t st = tree_build(ws, x, n, ws->p.precision, stream);
-    if (st != TREE_OK) return st;
-    st = tree_moments(ws, x, m, stream);
-    if (st != TREE_OK) return st;
-    return tree_forces(ws, a, phi, 0, stream);
-}
-
-// The side stream and events a leapfrog step forks its walk groups onto
-// (created outside any stream capture).
+// The side stream and events that one force evaluation forks part of its work
+// onto (created outside any stream capture).
 static tree_status_t ensure_side_stream(TreeWorkspace *ws) {
     if (!ws->side_stream) TRY_CUDA(cudaStreamCreateWithFlags(&ws->side_stream, cudaStreamNonBlocking));
     if (!ws->ev_fork) TRY_CUDA(cudaEventCreateWithFlags(&ws->ev_fork, cudaEventDisableTiming));
     if (!ws->ev_join) TRY_CUDA(cudaEventCreateWithFlags(&ws->ev_join, cudaEventDisableTiming));
     return TREE_OK;
+}
+
+// The walk groups' launches count as timed although no phase's events enclose them.
+static cudaError_t launch_groups_timed(TreeWorkspace *ws, int64_t n, cudaStream_t s) {
+    const int64_t l0 = ws->launches;
+    const cudaError_t e = launch_groups(ws, n, s);
+    if (ws->timing) ws->timed_launches += ws->launches - l0;
+    return e;
+}
+
+// From the octree to the forces: walk groups, gather, moments and walk.  x and
+// m: the caller's arrays, or NULL to gather from the packed copy of the
+// kick-drift pass.
+//
+// The walk groups need the octree only, and the gather and the moments do not
+// need the groups, so one of the two runs on the side stream beside the other
+// and is joined before whatever needs both.  A split walk's traversal reads
+// cells and groups but neither particles nor moments: there the gather and the
+// moments (FP64 latency) go aside and the groups and the traversal (dependent
+// loads) go on, up to the evaluation of the tiles (force at N = 1031 186 ->
+// 152 us, step at 30011 453 -> 369).  Otherwise the groups go aside.  The phase events of what
+// runs aside are on the side stream.
+static tree_status_t finish_forces(TreeWorkspace *ws, const void *x, const void *m, const WalkOut &out, int64_t n,
+                                   cudaStream_t s) {
+    tree_status_t st = upload_mac(ws, s);
+    if (st != TREE_OK) return st;
+    st = ensure_side_stream(ws);
+    if (st != TREE_OK) return st;
+    const bool split = walk_splits(ws);
+    const cudaStream_t side = ws->side_stream, sg = split ? s : side, sm = split ? side : s;
+    TRY_CUDA(cudaEventRecord(ws->ev_fork, s));
+    TRY_CUDA(cudaStreamWaitEvent(side, ws->ev_fork, 0));
+    if (!split) TRY_CUDA(launch_groups_timed(ws, n, sg));
+    {
+        PhaseScope ph(ws, TREE_PHASE_GATHER, sm);
+        TRY_CUDA(x ? launch_gather(ws, x, m, n, sm) : launch_gather_packed(ws, n, sm));
+    }
+    {
+        PhaseScope ph(ws, TREE_PHASE_MOMENTS, sm);
+        TRY_CUDA(launch_moments(ws, sm));
+    }
+    TRY_CUDA(cudaEventRecord(ws->ev_join, side));
+    if (split) {
+        TRY_CUDA(launch_groups_timed(ws, n, sg));
+        PhaseScope ph(ws, TREE_PHASE_WALK, s);
+        TRY_CUDA(launch_walk_split(ws, kWalkTiles, out, s));
+        TRY_CUDA(cudaStreamWaitEvent(s, ws->ev_join, 0));
+        ws->built = ws->has_moments = true;
+        TRY_CUDA(launch_walk_split(ws, kWalkFold, out, s));
+        return TREE_OK;
+    }
+    TRY_CUDA(cudaStreamWaitEvent(s, ws->ev_join, 0));
+    ws->built = ws->has_moments = true;
+    return walk(ws, kWalkForce, out, s);
+}
+
+tree_status_t tree_accel(TreeWorkspace *ws, const void *x, const void *m, int64_t n, void *a, void *phi,
+                         void *stream) {
+    if (!ws) return TREE_ERR_ARG;
+    if (n > 0 && (!x || !m || !a)) return TREE_ERR_ARG;
+    tree_status_t st = check_n(ws, n);
+    if (st != TREE_OK) return st;
+    cudaStream_t s = as_stream(stream);
+    ws->n = n;
+    ws->built = ws->has_moments = n == 0;
+    ws->list_groups = -1;
+    if (n == 0) return TREE_OK;
+    st = build_octree(ws, x, n, s);
+    if (st != TREE_OK) return st;
+    return finish_forces(ws, x, m, WalkOut{a, phi, nullptr, 0.0}, n, s);
 }
 
 // First part of a step: the first kick and the drift (Eqs. 2-3), fused with
@@ -667,42 +738,12 @@ static tree_status_t leapfrog_begin(TreeWorkspace *ws, void *x, void *v, const v
 static tree_status_t leapfrog_finish(TreeWorkspace *ws, const void *x, void *v, void *a, void *phi, double tau,
                                      int64_t n, cudaStream_t s, void *v_mirror = nullptr,
                                      void *phi_mirror = nullptr) {
-    {
-        PhaseScope ph(ws, TREE_PHASE_KEYS, s);
-        TRY_CUDA(launch_keys(ws, x, n, s));
-    }
-    {
-        PhaseScope ph(ws, TREE_PHASE_SORT, s);
-        TRY_CUDA(launch_sort(ws, n, s));
-    }
-    {
-        // The walk groups need the octree only, and the gather and the moments
-        // do not need the groups: the groups run on the side stream meanwhile
-        // (their kernels wait on dependent loads, the moments on the FP64 pipe)
-        // and are joined before the walk.  The phase's events, on s, time the
-        // octree; its launch count includes the groups.
-        PhaseScope ph(ws, TREE_PHASE_OCTREE, s);
-        TRY_CUDA(launch_octree(ws, n, s));
-        TRY_CUDA(cudaEventRecord(ws->ev_fork, s));
-        TRY_CUDA(cudaStreamWaitEvent(ws->side_stream, ws->ev_fork, 0));
-        TRY_CUDA(launch_groups(ws, n, ws->side_stream));
-        TRY_CUDA(cudaEventRecord(ws->ev_join, ws->side_stream));
-    }
-    ws->built = true;
-    {
-        PhaseScope ph(ws, TREE_PHASE_GATHER, s);
-        TRY_CUDA(launch_gather_packed(ws, n, s));
-    }
-    {
-        PhaseScope ph(ws, TREE_PHASE_MOMENTS, s);
-        TRY_CUDA(launch_moments(ws, s));
-    }
-    ws->has_moments = true;
-    TRY_CUDA(cudaStreamWaitEvent(s, ws->ev_join, 0));
+    tree_status_t st = sort_and_octree(ws, x, n, s);
+    if (st != TREE_OK) return st;
     WalkOut out{a, phi, v, 0.5 * tau};
     out.v_mirror = v_mirror;
     out.phi_mirror = phi_mirror;
-    return walk(ws, kWalkForce, out, s);
+    return finish_forces(ws, nullptr, nullptr, out, n, s);
 }
 
 tree_status_t leapfrog_step(TreeWorkspace *ws, void *x, void *v, const void *m, void *a, void *phi, double tau,

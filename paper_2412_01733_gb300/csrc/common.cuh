@@ -163,7 +163,7 @@ struct TreeWorkspace {
     double *hs_diag = nullptr;
     cudaStream_t copy_stream = nullptr;  // copies back that overlap the rest of the step
     cudaEvent_t ev_drift = nullptr, ev_xback = nullptr;
-    cudaStream_t side_stream = nullptr;  // a leapfrog step's walk groups, beside its gather and moments
+    cudaStream_t side_stream = nullptr;  // part of a force evaluation beside the rest (finish_forces)
     cudaEvent_t ev_fork = nullptr, ev_join = nullptr;
     // one captured leapfrog step (leapfrog_graph_capture)
     cudaStream_t cap_stream = nullptr;
@@ -577,9 +577,14 @@ struct WalkOut {
 };
 cudaError_t launch_walk_f32(TreeWorkspace *ws, int mode, const WalkOut &out, cudaStream_t s);
 cudaError_t launch_walk_f64(TreeWorkspace *ws, int mode, const WalkOut &out, cudaStream_t s);
-// walk_split_f32.cu / walk_split_f64.cu
-cudaError_t launch_walk_split_f32(TreeWorkspace *ws, const WalkOut &out, cudaStream_t s);
-cudaError_t launch_walk_split_f64(TreeWorkspace *ws, const WalkOut &out, cudaStream_t s);
+// walk_split_f32.cu / walk_split_f64.cu: the traversal (kWalkTiles), or the
+// evaluation and the fold (kWalkFold), of the split walk
+cudaError_t launch_walk_split_f32(TreeWorkspace *ws, WalkMode part, const WalkOut &out, cudaStream_t s);
+cudaError_t launch_walk_split_f64(TreeWorkspace *ws, WalkMode part, const WalkOut &out, cudaStream_t s);
+inline cudaError_t launch_walk_split(TreeWorkspace *ws, WalkMode part, const WalkOut &out, cudaStream_t s) {
+    return ws->p.precision == TREE_F64 ? launch_walk_split_f64(ws, part, out, s)
+                                       : launch_walk_split_f32(ws, part, out, s);
+}
 // adjoint.cu
 cudaError_t launch_adjoint(TreeWorkspace *ws, const void *abar, const void *phibar, void *xbar, void *mbar,
                            cudaStream_t s);

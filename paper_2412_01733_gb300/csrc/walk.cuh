@@ -932,15 +932,16 @@ cudaError_t walk_run(TreeWorkspace *ws, const WalkArgs &a, cudaStream_t s) {
     return cudaGetLastError();
 }
 
-// The split walk: traversal into tile slots, evaluation of the slots, fold.
+// The split walk's traversal into tile slots (kWalkTiles; the precision and the
+// pair terms play no part in it), or the evaluation of the slots and the fold.
 template <typename Real, int TPL, bool QUAD, bool KAHAN, bool SOFT>
-cudaError_t walk_split(TreeWorkspace *ws, const WalkArgs &a, cudaStream_t s) {
-    cudaError_t e = walk_run<Real, TPL, false, false, true, kWalkTiles>(ws, a, s);
-    if (e != cudaSuccess || ws->n <= 0) return e;
+cudaError_t walk_split(TreeWorkspace *ws, WalkMode part, const WalkArgs &a, cudaStream_t s) {
+    if (ws->n <= 0) return cudaSuccess;
+    if (part == kWalkTiles) return walk_run<Real, TPL, false, false, true, kWalkTiles>(ws, a, s);
     auto k = k_eval_tiles<Real, TPL, QUAD, SOFT>;
     k<<<wave_grid(k, (int64_t)ws->tile_cap * 32, kWalkWarps * 32, 1 << 20), kWalkWarps * 32, 0, s>>>(a);
     ws->launches += 1;
-    e = cudaGetLastError();
+    const cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     return walk_run<Real, TPL, QUAD, KAHAN, SOFT, kWalkFold>(ws, a, s);
 }
