@@ -153,13 +153,32 @@ __device__ __forceinline__ void pc_term(Real px, Real py, Real pz, const typenam
     }
 }
 
-__device__ __forceinline__ uint32_t warp_incl_scan(uint32_t v, int lane) {
+// Inclusive prefix of v < 2^B over the (full) warp and the warp's total.  A
+// warp that is alone on its scheduler (BALLOTS: the split walk's traversal)
+// waits less for B independent ballots than for five dependent shuffles; among
+// many warps the shuffles cost less issue (large walk: ballots +0.5 %).
+template <int B, bool BALLOTS>
+__device__ __forceinline__ uint32_t warp_prefix(uint32_t v, int lane, uint32_t &total) {
+    if constexpr (BALLOTS) {
+        uint32_t ex = 0, tot = 0;
+        const uint32_t lt = lanemask_lt();
 #pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        uint32_t y = __shfl_up_sync(0xffffffffu, v, o);
-        if (lane >= o) v += y;
+        for (int b = 0; b < B; ++b) {
+            const uint32_t m = __ballot_sync(0xffffffffu, (v >> b) & 1u);
+            ex += (uint32_t)__popc(m & lt) << b;
+            tot += (uint32_t)__popc(m) << b;
+        }
+        total = tot;
+        return ex + v;
+    } else {
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            uint32_t y = __shfl_up_sync(0xffffffffu, v, o);
+            if (lane >= o) v += y;
+        }
+        total = __shfl_sync(0xffffffffu, v, 31);
+        return v;
     }
-    return v;
 }
 
 // --- evaluation of one tile (whole warp) -----------------------------------
@@ -434,6 +453,8 @@ __global__ void __launch_bounds__(kWalkWarps * 32, walk_blocks(MODE, TPL, sizeof
     constexpr bool kR5 = sizeof(Real) == 4 && QUAD && TPL == 1;
     // tiles are filled and consumed (evaluated or emitted)
     constexpr bool kTiles = MODE == kWalkForce || MODE == kWalkFold || MODE == kWalkTiles;
+    // few warps, each with its scheduler to itself: shorter chains of instructions before fewer of them
+    constexpr bool kAlone = MODE == kWalkTiles;
 
     // persistent warps: each takes the next group slot until all are done
     const uint32_t ngroups = A.ctr[kCtrGroups];
@@ -509,23 +530,45 @@ __global__ void __launch_bounds__(kWalkWarps * 32, walk_blocks(MODE, TPL, sizeof
     uint32_t ntile = 0, tbase = 0, tnext = 0;
     bool full = false;  // out of slots: kWalkFold walks this group itself
     if (MODE == kWalkTiles && lane == 0) tnext = atomicAdd(A.ctr + kCtrTiles, (uint32_t)kTileChunk);
+    // room for the next tile's chunk; false when the slots have run out
+    auto open_chunk = [&]() {
+        const uint32_t base = __shfl_sync(0xffffffffu, tnext, 0);
+        if (base > A.tile_cap - kTileChunk) { full = true; return; }
+        if (lane == 0) {
+            if (ntile == 0) A.ghead[g] = base;
+            else A.tile_next[tbase / kTileChunk] = base;
+        }
+        tbase = base;
+    };
     auto emit_tile = [&](uint32_t src, int ns, uint32_t far) {
         if (full) return;
-        if ((ntile & (kTileChunk - 1)) == 0) {
-            const uint32_t base = __shfl_sync(0xffffffffu, tnext, 0);
-            if (base > A.tile_cap - kTileChunk) { full = true; return; }
-            if (lane == 0) {
-                if (ntile == 0) A.ghead[g] = base;
-                else A.tile_next[tbase / kTileChunk] = base;
-            }
-            tbase = base;
-        }
-        const uint32_t slot = tbase + (ntile & (kTileChunk - 1));
-        if ((ntile & (kTileChunk - 1)) == kTileChunk / 2 && lane == 0)
-            tnext = atomicAdd(A.ctr + kCtrTiles, (uint32_t)kTileChunk);
+        const uint32_t k = ntile & (kTileChunk - 1);
+        if (k == 0) open_chunk();
+        if (full) return;
+        if (k == kTileChunk / 2 && lane == 0) tnext = atomicAdd(A.ctr + kCtrTiles, (uint32_t)kTileChunk);
+        const uint32_t slot = tbase + k;
         if (lane == 0) A.tile_hdr[slot] = make_uint2((uint32_t)g, (uint32_t)ns | (far << 8));
         A.tile_idx[(size_t)slot * 32 + lane] = lane < ns ? src : 0u;
         ++ntile;
+    };
+    // `count` full tiles from a buffer: as many at a time as their chunk holds
+    auto emit_tiles = [&](const uint32_t *buf, int count, uint32_t far) {
+        while (count > 0 && !full) {
+            const uint32_t k = ntile & (kTileChunk - 1);
+            if (k == 0) open_chunk();
+            if (full) return;
+            const int m = min(count, (int)(kTileChunk - k));
+            if (k <= kTileChunk / 2 && k + m > kTileChunk / 2 && lane == 0)
+                tnext = atomicAdd(A.ctr + kCtrTiles, (uint32_t)kTileChunk);
+            const uint32_t slot = tbase + k;
+            if (lane < m) A.tile_hdr[slot + lane] = make_uint2((uint32_t)g, 32u | (far << 8));
+            uint32_t *dst = A.tile_idx + (size_t)slot * 32 + lane;
+#pragma unroll 4
+            for (int t = 0; t < m; ++t) dst[32 * t] = buf[32 * t + lane];
+            buf += 32 * m;
+            ntile += (uint32_t)m;
+            count -= m;
+        }
     };
     auto pc_tile = [&](const uint32_t *buf, int ns) {
         if (MODE == kWalkTiles) emit_tile(lane < ns ? buf[lane] : 0u, ns, 1u);
@@ -607,9 +650,9 @@ __global__ void __launch_bounds__(kWalkWarps * 32, walk_blocks(MODE, TPL, sizeof
             e = stack[top - 1 - lane];
             sz = (e >> 29) + 1u;
         }
-        const uint32_t incl0 = warp_incl_scan(sz, lane);
+        uint32_t avail;
+        const uint32_t incl0 = warp_prefix<4, kAlone>(sz, lane, avail);
         const uint32_t excl0 = incl0 - sz;
-        const uint32_t avail = __shfl_sync(0xffffffffu, incl0, 31);
         const uint32_t take = avail < 32u ? avail : 32u;
         const bool contrib = lane < nr && excl0 < take;
         const int nfull = __popc(__ballot_sync(0xffffffffu, lane < nr && incl0 <= take));
@@ -661,11 +704,18 @@ __global__ void __launch_bounds__(kWalkWarps * 32, walk_blocks(MODE, TPL, sizeof
         const uint32_t am = __ballot_sync(0xffffffffu, allfar);
         if (am) {
             const uint32_t cc = allfar ? lk.y : 0u;
-            const uint32_t incl = warp_incl_scan(cc, lane);
-            const uint32_t tot = __shfl_sync(0xffffffffu, incl, 31);
+            uint32_t tot;
+            const uint32_t incl = warp_prefix<4, kAlone>(cc, lane, tot);
             if (kTiles) {
-                if (allfar)
-                    for (uint32_t c = 0; c < cc; ++c) pcbuf[npc + (incl - cc) + c] = lk.x + c;
+                uint32_t *dst = pcbuf + npc + (incl - cc);
+                if constexpr (kAlone) {
+#pragma unroll
+                    for (uint32_t c = 0; c < 8; ++c)
+                        if (c < cc) dst[c] = lk.x + c;
+                } else {
+                    if (allfar)
+                        for (uint32_t c = 0; c < cc; ++c) dst[c] = lk.x + c;
+                }
                 npc += (int)tot;
             } else if (MODE == kWalkEmit) {
                 if (allfar)
@@ -698,12 +748,19 @@ __global__ void __launch_bounds__(kWalkWarps * 32, walk_blocks(MODE, TPL, sizeof
             const uint32_t lc = nleaf ? lk.y : 0u;
             const bool big = lc > (uint32_t)kMaxLeafSmall;
             const uint32_t sc = big ? 0u : lc;
-            const uint32_t incl2 = warp_incl_scan(sc, lane);
-            const uint32_t tot2 = __shfl_sync(0xffffffffu, incl2, 31);
+            uint32_t tot2;
+            const uint32_t incl2 = warp_prefix<5, kAlone>(sc, lane, tot2);
             n_pp += __reduce_add_sync(0xffffffffu, lc);
             if (kTiles) {
-                if (nleaf && !big)
-                    for (uint32_t c = 0; c < lc; ++c) ppbuf[npp + (incl2 - lc) + c] = lk.x + c;
+                uint32_t *dst = ppbuf + npp + (incl2 - sc);
+                if constexpr (kAlone) {
+#pragma unroll
+                    for (uint32_t c = 0; c < (uint32_t)kMaxLeafSmall; ++c)
+                        if (c < sc) dst[c] = lk.x + c;
+                } else {
+                    if (nleaf && !big)
+                        for (uint32_t c = 0; c < lc; ++c) dst[c] = lk.x + c;
+                }
                 npp += (int)tot2;
                 __syncwarp();
                 uint32_t bm = __ballot_sync(0xffffffffu, big);
@@ -719,20 +776,24 @@ __global__ void __launch_bounds__(kWalkWarps * 32, walk_blocks(MODE, TPL, sizeof
         if (kTiles) {
             if (npc >= 32) {
                 __syncwarp();
-                const int ntile = npc >> 5;
-                for (int t = 0; t < ntile; ++t) pc_tile(pcbuf + 32 * t, 32);
+                const int nfull = npc >> 5;
+                if (MODE == kWalkTiles) emit_tiles(pcbuf, nfull, 1u);
+                else
+                    for (int t = 0; t < nfull; ++t) pc_tile(pcbuf + 32 * t, 32);
                 const int r = npc & 31;
-                uint32_t t = lane < r ? pcbuf[32 * ntile + lane] : 0;
+                uint32_t t = lane < r ? pcbuf[32 * nfull + lane] : 0;
                 __syncwarp();
                 if (lane < r) pcbuf[lane] = t;
                 __syncwarp();
                 npc = r;
             }
             if (npp >= 32) {
-                const int ntile = npp >> 5;
-                for (int t = 0; t < ntile; ++t) pp_tile(ppbuf[32 * t + lane], 32);
+                const int nfull = npp >> 5;
+                if (MODE == kWalkTiles) emit_tiles(ppbuf, nfull, 0u);
+                else
+                    for (int t = 0; t < nfull; ++t) pp_tile(ppbuf[32 * t + lane], 32);
                 const int r = npp & 31;
-                uint32_t t = lane < r ? ppbuf[32 * ntile + lane] : 0;
+                uint32_t t = lane < r ? ppbuf[32 * nfull + lane] : 0;
                 __syncwarp();
                 if (lane < r) ppbuf[lane] = t;
                 __syncwarp();
