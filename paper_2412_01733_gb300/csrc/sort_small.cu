@@ -5,11 +5,12 @@
 // 1031, 99 at 30011.  Here one cluster of up to eight blocks keeps everything
 // in its shared memory and sorts in one launch: a stable LSD radix sort by
 // 8-bit digits, positions split evenly over the blocks, digit counts read and
-// keys sent through distributed shared memory.  Only the top five digits (40
-// bits, 13 octree levels) are sorted that way; the few keys that agree in
-// them are put in order by insertion, since LSD passes leave such a run in
-// the order of its particles' indices.  A run of more than kRunMax of them
-// out of order sends the cluster through all eight digits instead.  Box, keys
+// keys sent through distributed shared memory.  Only the top five or six
+// digits (40 or 48 bits, 13 or 16 octree levels) are sorted that way; the few
+// keys that agree in them are put in order by insertion, since LSD passes
+// leave such a run in the order of its particles' indices.  A run of more than
+// kRunMax of them sends the cluster through all eight digits instead (a galaxy
+// of 65536 has such runs in the top five digits: 127 us against 86).  Box, keys
 // and sort: N = 1031 96 -> 47 us, 30011 129 -> 69, 65536 136 -> 104 (the
 // ranking of eight keys a thread on eight SMs; beyond, the chip is needed).
 #include <cooperative_groups.h>
@@ -24,8 +25,8 @@ constexpr int kSmThreads = 1024, kSmWarps = kSmThreads / 32;
 constexpr int kSmItems = 8;                           // keys per thread at most
 constexpr int kSmBlock = kSmThreads * kSmItems;       // positions per block at most
 constexpr int kSmCluster = 8;
-constexpr int kTopPass = 3;                           // first of the digits sorted in the first place
 constexpr int kRunMax = 32;
+constexpr int64_t kTop5Max = 16384;                   // top five digits first up to this size, six above
 static_assert((int64_t)kSmBlock * kSmCluster == kSmallSortMax && kSmallSortMax <= 65536, "indices are 16 bits here");
 
 struct SmallSmem {
@@ -86,7 +87,7 @@ __global__ void __launch_bounds__(256) k_small_keys(const Real *__restrict__ x, 
 
 // Block r of the cluster holds positions [r Q, min(n, (r + 1) Q)), Q <= kSmBlock.
 __global__ void __launch_bounds__(kSmThreads, 1) k_small_sort(const uint64_t *__restrict__ kin, uint64_t *kout,
-                                                              uint32_t *vout, uint32_t n, uint32_t Q) {
+                                                              uint32_t *vout, uint32_t n, uint32_t Q, int top) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     SmallSmem &S = *reinterpret_cast<SmallSmem *>(smem_raw);
     cg::cluster_group cl = cg::this_cluster();
@@ -100,7 +101,7 @@ __global__ void __launch_bounds__(kSmThreads, 1) k_small_sort(const uint64_t *__
     const int nit = (int)(per / 32u);
     if (tid == 0) S.flag = 0;
     bool done = false;
-    for (int first = kTopPass; !done; first = 0) {
+    for (int first = top; !done; first = 0) {
         for (int pass = first; pass < kSortPasses; ++pass) {
             const int shift = 8 * pass;
             uint64_t k[kSmItems];
@@ -188,7 +189,7 @@ __global__ void __launch_bounds__(kSmThreads, 1) k_small_sort(const uint64_t *__
         done = first == 0;
         if (!done) {
             // runs that agree in the sorted digits (the output is this cluster's: seen after the sync)
-            constexpr int kLow = 8 * kTopPass;
+            const int kLow = 8 * top;
             for (uint32_t j = tid; j < cnt; j += kSmThreads) {
                 const uint32_t i = b0 + j;
                 const uint64_t h = __ldcg(kout + i) >> kLow;
@@ -244,7 +245,8 @@ cudaError_t launch_small_sort(TreeWorkspace *ws, int64_t n, cudaStream_t s) {
     at.val.clusterDim.y = at.val.clusterDim.z = 1;
     cfg.attrs = &at;
     cfg.numAttrs = 1;
-    e = cudaLaunchKernelEx(&cfg, k_small_sort, (const uint64_t *)ws->key_alt, ws->key, ws->idx, (uint32_t)n, Q);
+    e = cudaLaunchKernelEx(&cfg, k_small_sort, (const uint64_t *)ws->key_alt, ws->key, ws->idx, (uint32_t)n, Q,
+                           n <= kTop5Max ? 3 : 2);
     ws->launches += 1;
     return e;
 }
