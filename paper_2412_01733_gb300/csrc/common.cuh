@@ -40,17 +40,17 @@ constexpr int64_t kWalkOrderMaxN = (int64_t)1 << 22;
 // Split walk (walk.cuh): workspaces of at most this many particles (FP32,
 // FP64; the measured lines are in walk.cuh) keep tile slots for it, kTilesPer
 // for each particle, handed out kTileChunk at a time.  12 a particle serve
-// theta >= 0.43 at N = 65536 (660 B a slot in FP32).
-constexpr int64_t kSplitMaxN32 = (int64_t)1 << 16, kSplitMaxN64 = (int64_t)1 << 17;
+// theta >= 0.45 at N = 131072 (660 B a slot in FP32).
+constexpr int64_t kSplitMaxN32 = (int64_t)1 << 17, kSplitMaxN64 = (int64_t)1 << 17;
 constexpr int kTilesPer = 12;
 constexpr int kTileChunk = 16;
 constexpr uint32_t kTilesFull = 0xffffffffu;     // group whose tiles found no slot
 
 // Moments up to kClimbMaxN particles climb the tree in one launch, up to
 // kClimbPlainN without sorting the leaves by their particle counts first
-// (Plummer spheres, all moments: N = 1031 182 us level by level, 69 climbing;
-// 131072 272, 131 plain, 151 sorted; 262144 285, 187 plain, 157 sorted; 2^20
-// 355, 268 sorted; beyond, the level-by-level form's full warps gain on it).
+// (Plummer spheres, all moments, level by level -> climbing: N = 1031 182 ->
+// 53 us, 30011 241 -> 83, 131072 272 -> 88 plain; 2^20 355 -> 220 sorted;
+// beyond, the level-by-level form's full warps gain on it).
 constexpr int64_t kClimbMaxN = (int64_t)1 << 20, kClimbPlainN = (int64_t)1 << 17;
 
 // lookback status words: 2-bit flag + 30-bit value

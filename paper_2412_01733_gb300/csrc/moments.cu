@@ -174,18 +174,90 @@ __device__ __forceinline__ void mom_leaf(MomSums &a, const typename Vec4<Real>::
     }
 }
 
-// The whole moment tree in one launch: a thread takes a leaf, and whoever
+// Moments of internal cell `nd` by a half-warp (c = lane & 15), one of the
+// sixteen sums per lane:
+//   c = 0: M;  1..3: S;  4..9: T (xx yy zz xy xz yz);  10..15: sum of the
+//   children's Q (same order).
+// Every sum is acc = fma(m ua, ub, acc) with ones in the places of missing
+// factors, which rounds as MomSums::add does, so the results are those of one
+// thread doing all sixteen.  All 32 lanes call it together; has: this half
+// has a cell.
+template <typename Real>
+__device__ __forceinline__ void mom_cell_half(uint32_t nd, bool has, int lane, const uint4 *__restrict__ ngeo,
+                                              const uint2 *__restrict__ nlink, DevBox *__restrict__ box,
+                                              const uint32_t *__restrict__ nfirst, const int64_t *__restrict__ seg_off,
+                                              int64_t nseg, double *mom64, int64_t cap, Real *__restrict__ mom_a,
+                                              Real *__restrict__ mom_b, Real *__restrict__ mom_c) {
+    const int c = lane & 15, hb = lane & 16;
+    const uint2 lk = nlink[nd];
+    const uint4 g = ngeo[nd];
+    // axes (0 x, 1 y, 2 z) of this lane's factors; 3: one
+    const int aa = c == 0 ? 3 : c <= 3 ? c - 1 : c <= 6 ? c - 4 : c <= 8 ? 0 : c == 9 ? 1 : 3;
+    const int ab = c <= 3 ? 3 : c <= 6 ? c - 4 : c == 7 ? 1 : c <= 9 ? 2 : 3;
+    // rows of mom64 this lane's factors come from
+    const double *rm = mom64, *ra = mom64 + (c >= 10 ? c - 6 : 1 + (aa & 3)) * cap, *rb = mom64 + (1 + (ab & 3)) * cap;
+    const bool lm = c < 10, la = aa < 3 || c >= 10, lb = ab < 3;
+    const int nch = has ? (int)lk.y : 0;
+    double vm[8], va[8], vb[8];
+#pragma unroll
+    for (int k = 0; k < 8; ++k) {
+        vm[k] = va[k] = vb[k] = 1.0;
+        if (k < nch) {
+            if (lm) vm[k] = __ldcg(rm + lk.x + k);
+            if (la) va[k] = __ldcg(ra + lk.x + k);
+            if (lb) vb[k] = __ldcg(rb + lk.x + k);
+        }
+    }
+    double cx, cy, cz;
+    mom_centre<Real>(g, nd, box, nfirst, seg_off, nseg, cx, cy, cz);
+    const double ca = aa == 0 ? cx : aa == 1 ? cy : cz, cb = ab == 0 ? cx : ab == 1 ? cy : cz;
+    double acc = 0.0;
+#pragma unroll
+    for (int k = 0; k < 8; ++k) {
+        if (k < nch) {
+            const double ua = aa < 3 ? va[k] - ca : va[k], ub = ab < 3 ? vb[k] - cb : vb[k];
+            acc = fma(__dmul_rn(vm[k], ua), ub, acc);
+        }
+    }
+    const double M = __shfl_sync(0xffffffffu, acc, hb);
+    const double sx = __shfl_sync(0xffffffffu, acc, hb + 1), sy = __shfl_sync(0xffffffffu, acc, hb + 2),
+                 sz = __shfl_sync(0xffffffffu, acc, hb + 3);
+    const double iM = M != 0.0 ? 1.0 / M : 0.0;
+    // T about the centre of mass, in the lanes of T
+    const double sa = aa == 0 ? sx : aa == 1 ? sy : sz, sb = ab == 0 ? sx : ab == 1 ? sy : sz;
+    const double T = fma(__dmul_rn(-sa, sb), iM, acc);
+    const double txx = __shfl_sync(0xffffffffu, T, hb + 4), tyy = __shfl_sync(0xffffffffu, T, hb + 5),
+                 tzz = __shfl_sync(0xffffffffu, T, hb + 6);
+    const double Tc = __shfl_sync(0xffffffffu, T, hb + (c >= 10 ? c - 6 : c));  // Q lane <- its T lane
+    double out = acc;  // M
+    if (c >= 1 && c <= 3) out = M != 0.0 ? fma(acc, iM, ca) : ca;
+    if (c >= 10) {
+        const double tr = txx + tyy + tzz;
+        out = M == 0.0 ? 0.0 : c <= 12 ? acc + fma(3.0, Tc, -tr) : fma(3.0, Tc, acc);
+    }
+    if (has && (c <= 3 || c >= 10)) {
+        mom64[(c <= 3 ? c : c - 6) * cap + nd] = out;
+        const double qs = sizeof(Real) == 4 ? -1.0 : 1.0;  // the FP32 walk copies hold -Q
+        if (c <= 3) mom_a[4 * (size_t)nd + (c == 0 ? 3 : c - 1)] = (Real)out;
+        else if (c <= 13) mom_b[4 * (size_t)nd + (c - 10)] = (Real)(qs * out);
+        else mom_c[2 * (size_t)nd + (c - 14)] = (Real)(qs * out);
+        if (sizeof(Real) == 4 && c == 0 && nd < (uint32_t)nseg) box[nd].r5fit = pc_r5_fits(box[nd].k, (float)M) ? 1 : 0;
+    }
+}
+
+// The whole moment tree in one launch: a lane takes a leaf, and whoever
 // finishes the last child of a cell goes on with that cell, up to the root
 // (one arrival counter per cell, back at zero when the cell's children are
 // done, so the next pass finds it clear).  Nobody waits for anybody.  The
 // same sums in the same order as level by level (k_moments_level), which is
 // 21 launches of latency for a small system; here the latency is that of one
-// path of about ten cells, so what a cell needs is loaded before it is
-// needed: its own record with its child's sums, four children at a time (76
-// -> 69 us at N = 1031, 110 -> 104 at 30011).  What is left is FP64 latency
-// (ncu: 60 % of a warp's time in fixed-latency waits), about 8 us a cell.
-// Sixteen lanes per cell, one sum each, two cells of a warp at a time, took
-// longer (89 and 144 us).  BUCKETS: leaves in bucket order.
+// path of about ten cells, and most of it is FP64 latency (ncu: 60 % of a
+// warp's time in fixed-latency waits).  So what a cell needs is loaded before
+// it is needed, and while a warp has one or two cells left (the upper part of
+// every path) sixteen lanes share each; with more cells to a warp, a lane
+// does its own (sixteen lanes for all of them took longer, 144 us against 104
+// at N = 30011, the cells of a warp then following one another).  BUCKETS:
+// leaves in bucket order.
 template <typename Real, bool BUCKETS>
 __global__ void __launch_bounds__(64) k_moments_climb(
     const uint32_t *__restrict__ ctr, const uint32_t *__restrict__ off, const uint32_t *__restrict__ order,
@@ -195,54 +267,78 @@ __global__ void __launch_bounds__(64) k_moments_climb(
     typename Vec4<Real>::T *__restrict__ mom_a, typename Vec4<Real>::T *__restrict__ mom_b,
     typename Vec2<Real>::T *__restrict__ mom_c) {
     if (aborted(ctr, kStageAfter)) return;
+    const int lane = threadIdx.x & 31;
     const uint32_t end = BUCKETS ? off[kMomLeafBuckets] : ctr[kCtrLevelStart + kLevels];
-    for (uint32_t t = blockIdx.x * blockDim.x + threadIdx.x; t < end; t += gridDim.x * blockDim.x) {
-        uint32_t node = BUCKETS ? order[t] : t;
-        uint4 g = ngeo[node];
-        if (!BUCKETS && !((g.w >> 8) & 1u)) continue;
-        uint2 lk = nlink[node];
-        uint32_t par = nparent[node];
+    const uint32_t stride = gridDim.x * blockDim.x;
+    for (uint32_t t0 = blockIdx.x * blockDim.x + (threadIdx.x & ~31u); t0 < end; t0 += stride) {
+        const uint32_t t = t0 + lane;
+        bool active = t < end;  // this lane has finished cell `node`
+        // node's parent, and the parent's children
+        uint32_t node = 0, par = 0;
+        uint2 lk = make_uint2(0, 0);
         double cx, cy, cz;
-        mom_centre<Real>(g, node, box, nfirst, seg_off, nseg, cx, cy, cz);
-        MomSums a;
-        mom_leaf<Real>(a, spos, lk.x, lk.x + lk.y, cx, cy, cz);
-        lk = nlink[par];
-        g = ngeo[par];
-        mom_store<Real>(a, cx, cy, cz, node, mom64, cap, mom_a, mom_b, mom_c);
-        double M = a.M;
-        bool whole = true;  // this thread finished its cell
-        while (node >= (uint32_t)nseg) {
-            node = par;
-            __threadfence();  // this child's moments before its arrival
-            whole = atomicAdd(arrived + node, 1u) + 1u == lk.y;
-            if (!whole) break;
-            __threadfence();  // the other children's arrivals before their moments
-            arrived[node] = 0;
-            par = nparent[node];
-            mom_centre<Real>(g, node, box, nfirst, seg_off, nseg, cx, cy, cz);
-            MomSums b;
-            const uint32_t k1 = lk.x + lk.y;
-            for (uint32_t k0 = lk.x; k0 < k1; k0 += 4) {
-                double r[4][10];
-#pragma unroll
-                for (int j = 0; j < 4; ++j)
-#pragma unroll
-                    for (int c = 0; c < 10; ++c)
-                        if (k0 + j < k1) r[j][c] = __ldcg(mom64 + c * cap + k0 + j);
-#pragma unroll
-                for (int j = 0; j < 4; ++j)
-                    if (k0 + j < k1) {
-                        b.add(r[j][0], r[j][1] - cx, r[j][2] - cy, r[j][3] - cz);
-                        b.qxx += r[j][4]; b.qyy += r[j][5]; b.qzz += r[j][6];
-                        b.qxy += r[j][7]; b.qxz += r[j][8]; b.qyz += r[j][9];
-                    }
+        if (active) {
+            node = BUCKETS ? order[t] : t;
+            const uint4 g = ngeo[node];
+            active = BUCKETS || ((g.w >> 8) & 1u);
+            if (active) {
+                lk = nlink[node];
+                par = nparent[node];
+                mom_centre<Real>(g, node, box, nfirst, seg_off, nseg, cx, cy, cz);
+                MomSums a;
+                mom_leaf<Real>(a, spos, lk.x, lk.x + lk.y, cx, cy, cz);
+                lk = nlink[par];
+                mom_store<Real>(a, cx, cy, cz, node, mom64, cap, mom_a, mom_b, mom_c);
+                if (sizeof(Real) == 4 && node < (uint32_t)nseg)
+                    box[node].r5fit = pc_r5_fits(box[node].k, (float)a.M) ? 1 : 0;
             }
-            lk = nlink[par];
-            g = ngeo[par];
-            mom_store<Real>(b, cx, cy, cz, node, mom64, cap, mom_a, mom_b, mom_c);
-            M = b.M;
         }
-        if (sizeof(Real) == 4 && whole) box[node].r5fit = pc_r5_fits(box[node].k, (float)M) ? 1 : 0;
+        for (;;) {
+            __threadfence();  // the finished cells' moments before their arrivals
+            __syncwarp();
+            bool ready = false;
+            if (active && node >= (uint32_t)nseg) ready = atomicAdd(arrived + par, 1u) + 1u == lk.y;
+            const uint32_t todo = __ballot_sync(0xffffffffu, ready);
+            if (!todo) break;
+            __threadfence();  // the other children's arrivals before their moments
+            active = ready;
+            if (ready) {
+                node = par;
+                arrived[node] = 0;
+                par = nparent[node];
+            }
+            if (__popc(todo) <= 2) {
+                const int l0 = __ffs(todo) - 1, l1 = 31 - __clz(todo);
+                const uint32_t nd = __shfl_sync(0xffffffffu, node, lane < 16 ? l0 : l1);
+                if (ready) lk = nlink[par];
+                mom_cell_half<Real>(nd, lane < 16 || l1 != l0, lane, ngeo, nlink, box, nfirst, seg_off, nseg, mom64,
+                                    cap, reinterpret_cast<Real *>(mom_a), reinterpret_cast<Real *>(mom_b),
+                                    reinterpret_cast<Real *>(mom_c));
+            } else if (ready) {
+                mom_centre<Real>(ngeo[node], node, box, nfirst, seg_off, nseg, cx, cy, cz);
+                MomSums b;
+                const uint32_t k1 = lk.x + lk.y;
+                for (uint32_t k0 = lk.x; k0 < k1; k0 += 4) {
+                    double r[4][10];
+#pragma unroll
+                    for (int j = 0; j < 4; ++j)
+#pragma unroll
+                        for (int c = 0; c < 10; ++c)
+                            if (k0 + j < k1) r[j][c] = __ldcg(mom64 + c * cap + k0 + j);
+#pragma unroll
+                    for (int j = 0; j < 4; ++j)
+                        if (k0 + j < k1) {
+                            b.add(r[j][0], r[j][1] - cx, r[j][2] - cy, r[j][3] - cz);
+                            b.qxx += r[j][4]; b.qyy += r[j][5]; b.qzz += r[j][6];
+                            b.qxy += r[j][7]; b.qxz += r[j][8]; b.qyz += r[j][9];
+                        }
+                }
+                lk = nlink[par];
+                mom_store<Real>(b, cx, cy, cz, node, mom64, cap, mom_a, mom_b, mom_c);
+                if (sizeof(Real) == 4 && node < (uint32_t)nseg)
+                    box[node].r5fit = pc_r5_fits(box[node].k, (float)b.M) ? 1 : 0;
+            }
+        }
     }
 }
 

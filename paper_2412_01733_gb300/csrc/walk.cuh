@@ -11,11 +11,12 @@
 // the partial sums are folded, group by group, in the order of the tiles
 // (kWalkFold).  Each tile's partial sums and the order of the folds are those
 // of the one-warp walk, so the results are the same bits, alone or in an
-// ensemble.  Walk of a Plummer sphere, theta = 0.7 (one-warp -> split): FP32
-// N = 1031 62 -> 39 us, 16384 334 -> 172, 65536 495 -> 415, but 100003 560 ->
-// 592 (1.25 KB of slot traffic per tile, and the traversal no longer hides
-// behind the arithmetic); FP64 N = 16384 12.8 -> 2.7 ms, 65536 21.6 -> 13.1,
-// 131072 32.6 -> 28.7.  walk_splits() draws the lines there.
+// ensemble.  Force on a Plummer sphere, theta = 0.7 (one-warp -> split, the
+// moments then beside the traversal): FP32 N = 16384 455 -> 221 us, 65536 742
+// -> 528, 131072 987 -> 917, but 262144 1585 -> 1649 (1.25 KB of slot traffic
+// per tile, and the traversal no longer hides behind the arithmetic); FP64
+// walk alone N = 16384 12.8 -> 2.7 ms, 65536 21.6 -> 13.1, 131072 32.6 ->
+// 28.7.  walk_splits() draws the lines there.
 //
 // Traversal (per warp, depth first, stack in shared memory):
 //   the stack holds ranges of sibling nodes (children are contiguous in the
