@@ -43,10 +43,10 @@ struct AdjArgs {
     const void *mom_a, *mom_b, *mom_c;
     const int64_t *list_off;  // [2][ngroups + 1]
     const int32_t *pc_list, *pp_list;
-    double G, eps2;
-    double *xg;            // [3][n] xbar (atomics), key order
-    double *mg;            // [n]    mbar (atomics), key order
-    double *ccot;          // [10][cap] cell cotangents: Mbar, Rbar(3), Qbar(6)
+    double eps2;
+    double *xg;            // [3][n] xbar / G (atomics), key order
+    double *mg;            // [n]    mbar / G (atomics), key order
+    double *ccot;          // [10][cap] cell cotangents / G: Mbar, Rbar(3), Qbar(6)
     int64_t cap;
 };
 
@@ -165,11 +165,13 @@ __device__ __forceinline__ void pair_vjp(const AdjSource<Real> &S, typename Pack
 // pipe; in FP32 a lane meets two targets at a time in packed instructions:
 // targets j and j + 16 of a half of the group travel as a pair through
 // sixteen lanes, the warp's two halves holding one copy of the targets' sums
-// each.  (One pair at a time: Plummer sphere, N = 262144, 5.3 ms; now 2.9.)
-// Up to kAdjMaxParts warps share a group where there are few groups: N =
-// 65536 1.9 -> 0.85 ms.
+// each.  Plummer sphere, N = 262144: 5.3 ms with one pair at a time, 2.9 in
+// twos, 2.7 with two steps in flight and G left to the scatter (the FP64 pipe
+// was 40 % busy with the totals); five blocks per SM (96 registers, spills)
+// +3 %.  Up to kAdjMaxParts warps share a group where there are few groups:
+// N = 65536 1.9 -> 0.63 ms.
 template <typename Real, bool QUAD, bool SOFT>
-__global__ void __launch_bounds__(kAdjWarps * 32) k_force_vjp(const AdjArgs A) {
+__global__ void __launch_bounds__(kAdjWarps * 32, 4) k_force_vjp(const AdjArgs A) {
     using P = Pack<Real>;
     using V = typename P::V;
     using V4 = typename Vec4<Real>::T;
@@ -218,7 +220,7 @@ __global__ void __launch_bounds__(kAdjWarps * 32) k_force_vjp(const AdjArgs A) {
             V t[3] = {P::dup(Real(0)), P::dup(Real(0)), P::dup(Real(0))};
             const V(*st)[L] = s_t[w][h];
             const uint32_t first = s0 + 32u * (uint32_t)h;
-#pragma unroll 1
+#pragma unroll W
             for (int k = 0; k < L; ++k) {
                 if (k > 0) {
 #pragma unroll
@@ -265,18 +267,18 @@ __global__ void __launch_bounds__(kAdjWarps * 32) k_force_vjp(const AdjArgs A) {
             }
         }
         // the group's (at most 64) targets are summed in the working precision;
-        // the per-group totals go to the FP64 accumulators
+        // the per-group totals go to the FP64 accumulators (G comes with the scatter)
         V acc[11];
 #pragma unroll
         for (int q = 0; q < 11; ++q) acc[q] = P::dup(Real(0));
         meet(S, std::bool_constant<QUAD>{}, false, 0u, acc);
         if (lane < nt) {
             const Real mb = P::total(acc[0]) - P::total(acc[1]);
-            if (mb != Real(0)) atomicAdd(A.ccot + cid, A.G * (double)mb);
+            if (mb != Real(0)) atomicAdd(A.ccot + cid, (double)mb);
 #pragma unroll
             for (int q = 2; q < (QUAD ? 11 : 5); ++q) {
                 const Real v = P::total(acc[q]);
-                if (v != Real(0)) atomicAdd(A.ccot + (int64_t)(q - 1) * A.cap + cid, (q < 5 ? A.G : -A.G) * (double)v);
+                if (v != Real(0)) atomicAdd(A.ccot + (int64_t)(q - 1) * A.cap + cid, (double)(q < 5 ? v : -v));
             }
         }
     }
@@ -298,10 +300,10 @@ __global__ void __launch_bounds__(kAdjWarps * 32) k_force_vjp(const AdjArgs A) {
         if (own) meet(S, std::false_type{}, true, lane < nt ? sj : 0xffffffffu, acc);
         else meet(S, std::false_type{}, false, 0u, acc);
         if (lane < nt) {
-            atomicAdd(A.xg + sj, A.G * (double)P::total(acc[2]));
-            atomicAdd(A.xg + A.n + sj, A.G * (double)P::total(acc[3]));
-            atomicAdd(A.xg + 2 * A.n + sj, A.G * (double)P::total(acc[4]));
-            atomicAdd(A.mg + sj, A.G * (double)(P::total(acc[0]) - P::total(acc[1])));
+            atomicAdd(A.xg + sj, (double)P::total(acc[2]));
+            atomicAdd(A.xg + A.n + sj, (double)P::total(acc[3]));
+            atomicAdd(A.xg + 2 * A.n + sj, (double)P::total(acc[4]));
+            atomicAdd(A.mg + sj, (double)(P::total(acc[0]) - P::total(acc[1])));
         }
     };
     uint32_t *buf = s_buf[w];
@@ -347,7 +349,7 @@ __global__ void __launch_bounds__(kAdjWarps * 32) k_force_vjp(const AdjArgs A) {
         const int t = lane + 32 * h;
         if (t < cnt) {
 #pragma unroll
-            for (int c = 0; c < 3; ++c) atomicAdd(A.xg + c * A.n + s0 + t, -A.G * xt[h][c]);
+            for (int c = 0; c < 3; ++c) atomicAdd(A.xg + c * A.n + s0 + t, -xt[h][c]);
         }
     }
 }
@@ -433,7 +435,7 @@ __global__ void __launch_bounds__(128) k_cot_paths(const uint32_t *__restrict__ 
     }
 }
 
-// xbar[i] += xg + m grad P, mbar[i] += mg + P (key order -> caller order), P of
+// xbar[i] += G (xg + m grad P), mbar[i] += G (mg + P) (key order -> caller order), P of
 // the particle's leaf.
 template <typename Real>
 __global__ void __launch_bounds__(256) k_grad_scatter(const double *__restrict__ xg, const double *__restrict__ mg,
@@ -441,7 +443,7 @@ __global__ void __launch_bounds__(256) k_grad_scatter(const double *__restrict__
                                                       const double *__restrict__ mom64, int64_t cap,
                                                       const uint32_t *__restrict__ pleaf,
                                                       const typename Vec4<Real>::T *__restrict__ spos,
-                                                      const uint32_t *__restrict__ perm, int64_t n,
+                                                      const uint32_t *__restrict__ perm, int64_t n, double G,
                                                       Real *__restrict__ xbar, Real *__restrict__ mbar,
                                                       const uint32_t *__restrict__ ctr) {
     if (aborted(ctr, kStageAfter)) return;
@@ -456,11 +458,11 @@ __global__ void __launch_bounds__(256) k_grad_scatter(const double *__restrict__
         const double fx = q[4] * dx + q[7] * dy + q[8] * dz, fy = q[7] * dx + q[5] * dy + q[9] * dz,
                      fz = q[8] * dx + q[9] * dy + q[6] * dz;
         if (xbar) {
-            xbar[i] += (Real)(xg[s] + m * (q[1] + 2.0 * fx));
-            xbar[n + i] += (Real)(xg[n + s] + m * (q[2] + 2.0 * fy));
-            xbar[2 * n + i] += (Real)(xg[2 * n + s] + m * (q[3] + 2.0 * fz));
+            xbar[i] += (Real)(G * (xg[s] + m * (q[1] + 2.0 * fx)));
+            xbar[n + i] += (Real)(G * (xg[n + s] + m * (q[2] + 2.0 * fy)));
+            xbar[2 * n + i] += (Real)(G * (xg[2 * n + s] + m * (q[3] + 2.0 * fz)));
         }
-        if (mbar) mbar[i] += (Real)(mg[s] + q[0] + dx * (q[1] + fx) + dy * (q[2] + fy) + dz * (q[3] + fz));
+        if (mbar) mbar[i] += (Real)(G * (mg[s] + q[0] + dx * (q[1] + fx) + dy * (q[2] + fy) + dz * (q[3] + fz)));
     }
 }
 
@@ -485,7 +487,6 @@ static cudaError_t adjoint_impl(TreeWorkspace *ws, const void *abar, const void 
     A.mom_a = ws->mom_a; A.mom_b = ws->mom_b; A.mom_c = ws->mom_c;
     A.list_off = ws->list_cnt;
     A.pc_list = ws->pc_list; A.pp_list = ws->pp_list;
-    A.G = ws->p.G;
     A.eps2 = ws->p.eps * ws->p.eps;
     A.xg = ws->adj_xg; A.mg = ws->adj_mg; A.ccot = ws->adj_ccot;
     A.cap = cap;
@@ -507,7 +508,7 @@ static cudaError_t adjoint_impl(TreeWorkspace *ws, const void *abar, const void 
     k_cot_paths<<<grid_for(cap, 128, 152 * 16), 128, 0, s>>>(ws->ctr, ws->ngeo, ws->nparent, ws->mom64, cap, ws->nseg,
                                                               ws->adj_ccot);
     k_grad_scatter<Real><<<nb, 256, 0, s>>>(ws->adj_xg, ws->adj_mg, ws->adj_ccot, ws->mom64, cap, ws->pleaf,
-                                            (const typename Vec4<Real>::T *)ws->spos, ws->idx, n, (Real *)xbar,
+                                            (const typename Vec4<Real>::T *)ws->spos, ws->idx, n, ws->p.G, (Real *)xbar,
                                             (Real *)mbar, ws->ctr);
     ws->launches += 4;
     return cudaGetLastError();
