@@ -529,30 +529,30 @@ static tree_status_t walk(TreeWorkspace *ws, int mode, WalkOut out, cudaStream_t
         return TREE_OK;
     }
     out.ordered = walk_widest_first(ws);
-    if (out.ordered) TRY_CUDA(launch_group_order(ws, s));
+    // (the walk that stores the lists follows the one that counted them: same order)
+    if (out.ordered && mode != kWalkEmit) TRY_CUDA(launch_group_order(ws, s));
     if (ws->p.precision == TREE_F64) TRY_CUDA(launch_walk_f64(ws, mode, out, s));
     else TRY_CUDA(launch_walk_f32(ws, mode, out, s));
     return TREE_OK;
 }
 
 static tree_status_t build_lists(TreeWorkspace *ws, cudaStream_t s) {
-    uint32_t ngd = 0;
-    TRY_CUDA(cudaMemcpyAsync(&ngd, ws->ctr + kCtrGroups, sizeof(uint32_t), cudaMemcpyDeviceToHost, s));
-    TRY_CUDA(cudaStreamSynchronize(s));
-    const int64_t ng = ngd;
-    ws->list_groups_host = ng;
+    if (!ws->list_cnt && !dalloc(&ws->list_cnt, (size_t)(2 * (ws->groups_max + 1)))) return TREE_ERR_ALLOC;
     WalkOut none{nullptr, nullptr, nullptr, 0.0};
     tree_status_t st = walk(ws, kWalkCount, none, s);
     if (st != TREE_OK) return st;
-    if (!ws->list_cnt && !dalloc(&ws->list_cnt, (size_t)(2 * (ws->groups_max + 1)))) return TREE_ERR_ALLOC;
+    // the statistics slots hold the sizes until the host has read them
+    int64_t *sizes = reinterpret_cast<int64_t *>(ws->stats);
+    static_assert(kStatCount >= 3, "room for the list sizes");
     {
         PhaseScope ph(ws, TREE_PHASE_LISTS, s);
-        TRY_CUDA(launch_scan_lists(ws, ng, s));
+        TRY_CUDA(launch_scan_lists(ws, sizes, s));
     }
-    int64_t tot[2];
-    TRY_CUDA(cudaMemcpyAsync(&tot[0], ws->list_cnt + ng, sizeof(int64_t), cudaMemcpyDeviceToHost, s));
-    TRY_CUDA(cudaMemcpyAsync(&tot[1], ws->list_cnt + (ng + 1) + ng, sizeof(int64_t), cudaMemcpyDeviceToHost, s));
+    int64_t sz[3];
+    TRY_CUDA(cudaMemcpyAsync(sz, sizes, sizeof(sz), cudaMemcpyDeviceToHost, s));
     TRY_CUDA(cudaStreamSynchronize(s));
+    const int64_t ng = sz[0], *tot = sz + 1;
+    ws->list_groups_host = ng;
     if (tot[0] > ws->list_pc_cap) {
         if (ws->pc_list) cudaFree(ws->pc_list);
         ws->pc_list = nullptr;

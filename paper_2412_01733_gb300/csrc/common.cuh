@@ -608,7 +608,7 @@ cudaError_t launch_direct_range(TreeWorkspace *ws, const void *x, const void *m,
 cudaError_t launch_widen(TreeWorkspace *ws, const float *in, int64_t count, double *out, cudaStream_t s);
 cudaError_t launch_rel_err(TreeWorkspace *ws, const void *a, int64_t n, int dtype, const int64_t *tgt,
                            const double *ref, int64_t nt, double *err, cudaStream_t s);
-cudaError_t launch_scan_lists(TreeWorkspace *ws, int64_t ngroups, cudaStream_t s);
+cudaError_t launch_scan_lists(TreeWorkspace *ws, int64_t *sizes, cudaStream_t s);
 cudaError_t launch_gstat_reduce(TreeWorkspace *ws, int64_t ngroups, cudaStream_t s);
 cudaError_t launch_group_order(TreeWorkspace *ws, cudaStream_t s);
 cudaError_t launch_export_gstat(TreeWorkspace *ws, int64_t ngroups, uint32_t *out, cudaStream_t s);

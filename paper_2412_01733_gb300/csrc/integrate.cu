@@ -696,13 +696,14 @@ __global__ void __launch_bounds__(256) k_gstat_reduce(const uint4 *__restrict__ 
 }
 
 // Exclusive scans of the per-group list lengths (x: PC cells, w: PP leaves)
-// into list_off[0..ng] and list_off[ng+1 .. 2ng+1].  Single block: the list
+// into list_off[0..ng] and list_off[ng+1 .. 2ng+1]; sizes: ng and both totals.  Single block: the list
 // path is a test/adjoint path, not the force hot path.
-__global__ void __launch_bounds__(1024) k_list_scan(const uint4 *__restrict__ gstat, int64_t ng,
-                                                    int64_t *__restrict__ off) {
+__global__ void __launch_bounds__(1024) k_list_scan(const uint4 *__restrict__ gstat, const uint32_t *__restrict__ ctr,
+                                                    int64_t *__restrict__ off, int64_t *__restrict__ sizes) {
     __shared__ unsigned long long wt[2][32];
     __shared__ unsigned long long carry[2];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int64_t ng = ctr[kCtrGroups];
     if (tid < 2) carry[tid] = 0;
     __syncthreads();
     for (int64_t b = 0; b < ng; b += 1024) {
@@ -737,7 +738,8 @@ __global__ void __launch_bounds__(1024) k_list_scan(const uint4 *__restrict__ gs
         if (tid < 2) carry[tid] += wt[tid][31];
         __syncthreads();
     }
-    if (tid < 2) off[tid * (ng + 1) + ng] = (int64_t)carry[tid];
+    if (tid < 2) off[tid * (ng + 1) + ng] = sizes[1 + tid] = (int64_t)carry[tid];
+    if (tid == 0) sizes[0] = ng;
 }
 
 __global__ void k_export_gstat(const uint4 *__restrict__ gstat, int64_t ng, uint32_t *__restrict__ out) {
@@ -754,8 +756,8 @@ cudaError_t launch_export_gstat(TreeWorkspace *ws, int64_t ngroups, uint32_t *ou
     return cudaGetLastError();
 }
 
-cudaError_t launch_scan_lists(TreeWorkspace *ws, int64_t ngroups, cudaStream_t s) {
-    k_list_scan<<<1, 1024, 0, s>>>(ws->gstat, ngroups, ws->list_cnt);
+cudaError_t launch_scan_lists(TreeWorkspace *ws, int64_t *sizes, cudaStream_t s) {
+    k_list_scan<<<1, 1024, 0, s>>>(ws->gstat, ws->ctr, ws->list_cnt, sizes);
     ws->launches += 1;
     return cudaGetLastError();
 }

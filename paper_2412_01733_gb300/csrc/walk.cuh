@@ -455,7 +455,8 @@ __global__ void __launch_bounds__(kWalkWarps * 32, walk_blocks(MODE, TPL, sizeof
     // tiles are filled and consumed (evaluated or emitted)
     constexpr bool kTiles = MODE == kWalkForce || MODE == kWalkFold || MODE == kWalkTiles;
     // few warps, each with its scheduler to itself: shorter chains of instructions before fewer of them
-    constexpr bool kAlone = MODE == kWalkTiles;
+    // (the list walks serve gradients, at sizes where that holds too)
+    constexpr bool kAlone = MODE == kWalkTiles || MODE == kWalkCount || MODE == kWalkEmit;
 
     // persistent warps: each takes the next group slot until all are done
     const uint32_t ngroups = A.ctr[kCtrGroups];
@@ -719,8 +720,10 @@ __global__ void __launch_bounds__(kWalkWarps * 32, walk_blocks(MODE, TPL, sizeof
                 }
                 npc += (int)tot;
             } else if (MODE == kWalkEmit) {
-                if (allfar)
-                    for (uint32_t c = 0; c < cc; ++c) A.pc_list[pc_base + n_pc + (incl - cc) + c] = (int32_t)(lk.x + c);
+                int32_t *dst = A.pc_list + pc_base + n_pc + (incl - cc);
+#pragma unroll
+                for (uint32_t c = 0; c < 8; ++c)
+                    if (c < cc) dst[c] = (int32_t)(lk.x + c);
             }
             n_pc += tot;
         }
