@@ -76,7 +76,7 @@ struct DevBox {
     double scale;   // 2^(21-k)
     double unit;    // 2^(k-21): grid spacing
     int32_t k;
-    int32_t r5fit;  // set after the moments: the FP32 walk's r^-5 far-cell form fits (pc_r5_fits)
+    int32_t r5fit;  // set after the moments: the walk's r^-5 far-cell form fits (pc_r5_fits)
 };
 
 // Offsets into the counter block (uint32), cleared at the start of a build.
@@ -338,6 +338,14 @@ __device__ __forceinline__ bool pc_r5_fits(int k, float m_root) {
     if (k > 24) return false;
     const float span = 1.7320508f * ldexpf(1.0f, max(k, -40));
     return m_root * span * span * span <= 1e37f;
+}
+
+// The same for the FP64 walk: k <= 200 keeps r^-5 a normal FP64 number, the
+// mass bound keeps M r^2 u <= 1e300.
+__device__ __forceinline__ bool pc_r5_fits(int k, double m_root) {
+    if (k > 200) return false;
+    const double span = 1.7320508075688774 * ldexp(1.0, max(k, -300));
+    return fabs(m_root) * span * span * span <= 1e300;
 }
 
 __device__ __forceinline__ bool aborted(const uint32_t *ctr, uint32_t stage) {

@@ -241,7 +241,7 @@ __device__ __forceinline__ void mom_cell_half(uint32_t nd, bool has, int lane, c
         if (c <= 3) mom_a[4 * (size_t)nd + (c == 0 ? 3 : c - 1)] = (Real)out;
         else if (c <= 13) mom_b[4 * (size_t)nd + (c - 10)] = (Real)(qs * out);
         else mom_c[2 * (size_t)nd + (c - 14)] = (Real)(qs * out);
-        if (sizeof(Real) == 4 && c == 0 && nd < (uint32_t)nseg) box[nd].r5fit = pc_r5_fits(box[nd].k, (float)M) ? 1 : 0;
+        if (c == 0 && nd < (uint32_t)nseg) box[nd].r5fit = pc_r5_fits(box[nd].k, (Real)M) ? 1 : 0;
     }
 }
 
@@ -289,8 +289,7 @@ __global__ void __launch_bounds__(64) k_moments_climb(
                 mom_leaf<Real>(a, spos, lk.x, lk.x + lk.y, cx, cy, cz);
                 lk = nlink[par];
                 mom_store<Real>(a, cx, cy, cz, node, mom64, cap, mom_a, mom_b, mom_c);
-                if (sizeof(Real) == 4 && node < (uint32_t)nseg)
-                    box[node].r5fit = pc_r5_fits(box[node].k, (float)a.M) ? 1 : 0;
+                if (node < (uint32_t)nseg) box[node].r5fit = pc_r5_fits(box[node].k, (Real)a.M) ? 1 : 0;
             }
         }
         for (;;) {
@@ -335,8 +334,7 @@ __global__ void __launch_bounds__(64) k_moments_climb(
                 }
                 lk = nlink[par];
                 mom_store<Real>(b, cx, cy, cz, node, mom64, cap, mom_a, mom_b, mom_c);
-                if (sizeof(Real) == 4 && node < (uint32_t)nseg)
-                    box[node].r5fit = pc_r5_fits(box[node].k, (float)b.M) ? 1 : 0;
+                if (node < (uint32_t)nseg) box[node].r5fit = pc_r5_fits(box[node].k, (Real)b.M) ? 1 : 0;
             }
         }
     }
@@ -390,13 +388,14 @@ __global__ void __launch_bounds__(256) k_moments_level(
     }
 }
 
-// Per segment b (its root is node b), whether the FP32 walk may take its
-// r^-5 far-cell form: pc_r5_fits of the segment's cube and root mass.
+// Per segment b (its root is node b), whether the walk may take its r^-5
+// far-cell form: pc_r5_fits of the segment's cube and root mass.
+template <typename V4, typename Real>
 __global__ void __launch_bounds__(256) k_r5_flags(const uint32_t *__restrict__ ctr, DevBox *box,
-                                                  const float4 *__restrict__ mom_a, int64_t nseg) {
+                                                  const V4 *__restrict__ mom_a, int64_t nseg) {
     if (aborted(ctr, kStageAfter)) return;
     for (int64_t b = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; b < nseg; b += (int64_t)gridDim.x * blockDim.x)
-        box[b].r5fit = pc_r5_fits(box[b].k, mom_a[b].w) ? 1 : 0;
+        box[b].r5fit = pc_r5_fits(box[b].k, (Real)mom_a[b].w) ? 1 : 0;
 }
 
 template <typename Real>
@@ -434,11 +433,8 @@ static cudaError_t moments_impl(TreeWorkspace *ws, cudaStream_t s) {
                                                  ws->seg_off, ws->nseg, ws->mom64, ws->node_cap, (V4 *)ws->mom_a,
                                                  (V4 *)ws->mom_b, (V2 *)ws->mom_c);
     ws->launches += 3 + kMaxLevel;
-    if (sizeof(Real) == 4) {
-        k_r5_flags<<<grid_for(ws->nseg, 256, 152), 256, 0, s>>>(ws->ctr, ws->box, (const float4 *)ws->mom_a,
-                                                               ws->nseg);
-        ws->launches += 1;
-    }
+    k_r5_flags<V4, Real><<<grid_for(ws->nseg, 256, 152), 256, 0, s>>>(ws->ctr, ws->box, (const V4 *)ws->mom_a, ws->nseg);
+    ws->launches += 1;
     return cudaGetLastError();
 }
 
