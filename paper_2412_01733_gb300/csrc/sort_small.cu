@@ -2,7 +2,7 @@
 // general form: eight onesweep passes, one launch each).
 //
 // Up to kSmallSortMax particles the eight passes are latency: 68 us at N =
-// 1031, 99 at 30011.  Here one cluster of up to eight blocks keeps everything
+// 1031, 99 at 30011.  Here one cluster of up to sixteen blocks keeps everything
 // in its shared memory and sorts in one launch: a stable LSD radix sort by
 // 8-bit digits, positions split evenly over the blocks, digit counts read and
 // keys sent through distributed shared memory.  Only the top five or six
@@ -11,8 +11,9 @@
 // leave such a run in the order of its particles' indices.  A run of more than
 // kRunMax of them sends the cluster through all eight digits instead (a galaxy
 // of 65536 has such runs in the top five digits: 127 us against 86).  Box, keys
-// and sort: N = 1031 96 -> 47 us, 30011 129 -> 69, 65536 136 -> 104 (the
-// ranking of eight keys a thread on eight SMs; beyond, the chip is needed).
+// and sort: N = 1031 96 -> 39 us, 30011 129 -> 61, 65536 136 -> 83.  (Eight
+// blocks of up to eight keys a thread: 47, 75 and 115; a pass is the keys' way
+// through distributed shared memory, which more blocks share.)
 #include <cooperative_groups.h>
 
 #include "common.cuh"
@@ -22,9 +23,9 @@ namespace treegb {
 namespace cg = cooperative_groups;
 
 constexpr int kSmThreads = 1024, kSmWarps = kSmThreads / 32;
-constexpr int kSmItems = 8;                           // keys per thread at most
+constexpr int kSmItems = 4;                           // keys per thread at most
 constexpr int kSmBlock = kSmThreads * kSmItems;       // positions per block at most
-constexpr int kSmCluster = 8;
+constexpr int kSmCluster = 16;
 constexpr int kRunMax = 32;
 constexpr int64_t kTop5Max = 16384;                   // top five digits first up to this size, six above
 static_assert((int64_t)kSmBlock * kSmCluster == kSmallSortMax && kSmallSortMax <= 65536, "indices are 16 bits here");
@@ -229,10 +230,11 @@ cudaError_t launch_small_keys(TreeWorkspace *ws, const void *x, int64_t n, cudaS
 
 cudaError_t launch_small_sort(TreeWorkspace *ws, int64_t n, cudaStream_t s) {
     // more blocks before more keys per thread: a pass is latency, and a block's part of it grows with its keys
-    const uint32_t C = n <= 2048 ? 1 : n <= 4096 ? 2 : n <= 8192 ? 4 : kSmCluster;
+    const uint32_t C = n <= 1024 ? 1 : n <= 2048 ? 2 : n <= 4096 ? 4 : n <= 8192 ? 8 : kSmCluster;
     const uint32_t Q = (uint32_t)((n + C - 1) / C);
     cudaError_t e = cudaFuncSetAttribute(k_small_sort, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          (int)sizeof(SmallSmem));
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(k_small_sort, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
     if (e != cudaSuccess) return e;
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = dim3(C);
