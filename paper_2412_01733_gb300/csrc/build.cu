@@ -17,8 +17,7 @@ namespace treegb {
 template <typename Real>
 __global__ void __launch_bounds__(256) k_box_partial(const Real *__restrict__ x, int64_t n,
                                                      double *__restrict__ part, int32_t *dstatus) {
-    // min/max are exact in the input precision; widen to FP64 once per warp
-    __shared__ double sh[6][8];
+    __shared__ Real sh[6][8];
     const Real big = sizeof(Real) == 4 ? (Real)FLT_MAX : (Real)DBL_MAX;
     Real mn[3] = {big, big, big}, mx[3] = {-big, -big, -big};
     bool bad = false;
@@ -33,64 +32,38 @@ __global__ void __launch_bounds__(256) k_box_partial(const Real *__restrict__ x,
         }
     }
     if (__any_sync(0xffffffffu, bad) && (threadIdx.x & 31) == 0) set_status(dstatus, TREE_DEV_NONFINITE);
-    double dmn[3], dmx[3];
-#pragma unroll
-    for (int d = 0; d < 3; ++d) {
-        dmn[d] = mn[d] == big ? DBL_MAX : (double)mn[d];
-        dmx[d] = mx[d] == -big ? -DBL_MAX : (double)mx[d];
-        for (int o = 16; o > 0; o >>= 1) {
-            dmn[d] = fmin(dmn[d], __shfl_xor_sync(0xffffffffu, dmn[d], o));
-            dmx[d] = fmax(dmx[d], __shfl_xor_sync(0xffffffffu, dmx[d], o));
-        }
-    }
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    if (lane == 0) {
-        for (int d = 0; d < 3; ++d) { sh[d][warp] = dmn[d]; sh[3 + d][warp] = dmx[d]; }
-    }
-    __syncthreads();
-    if (threadIdx.x < 6) {
-        const int c = threadIdx.x;
-        double r = sh[c][0];
-        for (int w = 1; w < (int)(blockDim.x >> 5); ++w) r = c < 3 ? fmin(r, sh[c][w]) : fmax(r, sh[c][w]);
-        part[blockIdx.x * 8 + c] = r;
-    }
+    block_minmax<Real>(mn, mx, big, sh, part + blockIdx.x * 8);
 }
 
 // One block: each thread folds a strided share of the partials, then the
-// block folds the threads (min and max are exact in any order).
+// block folds the threads (min and max are exact in any order, and the
+// partials are values of the input's precision).
+template <typename Real>
 __global__ void __launch_bounds__(256) k_box_final(const double *__restrict__ part, int nblocks, DevBox *box) {
-    __shared__ double sh[6][8];
-    double lo[3] = {DBL_MAX, DBL_MAX, DBL_MAX}, hi[3] = {-DBL_MAX, -DBL_MAX, -DBL_MAX};
+    __shared__ Real sh[6][8];
+    __shared__ double res[6];
+    const Real big = sizeof(Real) == 4 ? (Real)INFINITY : (Real)DBL_MAX;  // (Real)DBL_MAX: an empty partial
+    Real lo[3] = {big, big, big}, hi[3] = {-big, -big, -big};
     for (int b = threadIdx.x; b < nblocks; b += blockDim.x) {
+#pragma unroll
         for (int d = 0; d < 3; ++d) {
-            lo[d] = fmin(lo[d], part[b * 8 + d]);
-            hi[d] = fmax(hi[d], part[b * 8 + 3 + d]);
+            lo[d] = min(lo[d], (Real)part[b * 8 + d]);
+            hi[d] = max(hi[d], (Real)part[b * 8 + 3 + d]);
         }
     }
-    for (int d = 0; d < 3; ++d) {
-        for (int o = 16; o > 0; o >>= 1) {
-            lo[d] = fmin(lo[d], __shfl_xor_sync(0xffffffffu, lo[d], o));
-            hi[d] = fmax(hi[d], __shfl_xor_sync(0xffffffffu, hi[d], o));
-        }
-    }
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    if (lane == 0)
-        for (int d = 0; d < 3; ++d) { sh[d][warp] = lo[d]; sh[3 + d][warp] = hi[d]; }
+    block_minmax<Real>(lo, hi, big, sh, res);
     __syncthreads();
     if (threadIdx.x == 0) {
-        for (int w = 1; w < (int)(blockDim.x >> 5); ++w)
-            for (int d = 0; d < 3; ++d) {
-                lo[d] = fmin(lo[d], sh[d][w]);
-                hi[d] = fmax(hi[d], sh[3 + d][w]);
-            }
-        box_from_minmax(lo, hi, box);
+        double l[3] = {res[0], res[1], res[2]}, h[3] = {res[3], res[4], res[5]};
+        box_from_minmax(l, h, box);
     }
 }
 
 cudaError_t launch_box_final(TreeWorkspace *ws, int nblocks, int64_t n, cudaStream_t s) {
     ws->box_parts = nblocks;
     if (small_sort(ws, n)) return cudaGetLastError();  // k_small_keys folds the partials
-    k_box_final<<<1, 256, 0, s>>>(ws->part, nblocks, ws->box);
+    if (ws->p.precision == TREE_F64) k_box_final<double><<<1, 256, 0, s>>>(ws->part, nblocks, ws->box);
+    else k_box_final<float><<<1, 256, 0, s>>>(ws->part, nblocks, ws->box);
     ws->launches += 1;
     return cudaGetLastError();
 }
@@ -105,9 +78,9 @@ __global__ void __launch_bounds__(256) k_box_chunks(Real *__restrict__ x, Real *
                                                     typename Vec4<Real>::T *__restrict__ xm, Real half_tau, Real tau,
                                                     int64_t n, const uint4 *__restrict__ chunks, int64_t nchunks,
                                                     double *__restrict__ part, int32_t *dstatus) {
-    __shared__ double sh[6][8];
+    __shared__ Real sh[6][8];
     const Real big = sizeof(Real) == 4 ? (Real)FLT_MAX : (Real)DBL_MAX;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int lane = threadIdx.x & 31;
     for (int64_t c = blockIdx.x; c < nchunks; c += gridDim.x) {
         const uint4 ch = chunks[c];
         Real mn[3] = {big, big, big}, mx[3] = {-big, -big, -big};
@@ -137,26 +110,7 @@ __global__ void __launch_bounds__(256) k_box_chunks(Real *__restrict__ x, Real *
             }
         }
         if (__any_sync(0xffffffffu, bad) && lane == 0) set_status(dstatus, TREE_DEV_NONFINITE);
-        double dmn[3], dmx[3];
-#pragma unroll
-        for (int d = 0; d < 3; ++d) {
-            dmn[d] = mn[d] == big ? DBL_MAX : (double)mn[d];
-            dmx[d] = mx[d] == -big ? -DBL_MAX : (double)mx[d];
-            for (int o = 16; o > 0; o >>= 1) {
-                dmn[d] = fmin(dmn[d], __shfl_xor_sync(0xffffffffu, dmn[d], o));
-                dmx[d] = fmax(dmx[d], __shfl_xor_sync(0xffffffffu, dmx[d], o));
-            }
-        }
-        if (lane == 0) {
-            for (int d = 0; d < 3; ++d) { sh[d][warp] = dmn[d]; sh[3 + d][warp] = dmx[d]; }
-        }
-        __syncthreads();
-        if (threadIdx.x < 6) {
-            const int q = threadIdx.x;
-            double r = sh[q][0];
-            for (int w = 1; w < (int)(blockDim.x >> 5); ++w) r = q < 3 ? fmin(r, sh[q][w]) : fmax(r, sh[q][w]);
-            part[c * 8 + q] = r;
-        }
+        block_minmax<Real>(mn, mx, big, sh, part + c * 8);
         __syncthreads();
     }
 }

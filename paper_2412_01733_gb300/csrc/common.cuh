@@ -476,6 +476,30 @@ __device__ __forceinline__ void octant_bounds(const uint64_t *__restrict__ skey,
     b[8] = first + count;
 }
 
+// Folds the threads' minima and maxima of a block of 256 (`big`, -`big`: none)
+// and lets threads 0..5 store them, widened, to part[0..5].  Minima and maxima
+// are exact in the input precision; in FP64 the shuffle steps of FP32 input
+// took longer than the reads (30 compares a thread at 1/64 of the FP32 rate).
+template <typename Real>
+__device__ __forceinline__ void block_minmax(Real (&mn)[3], Real (&mx)[3], Real big, Real (&sh)[6][8], double *part) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+#pragma unroll
+    for (int d = 0; d < 3; ++d) {
+        for (int o = 16; o > 0; o >>= 1) {
+            mn[d] = min(mn[d], __shfl_xor_sync(0xffffffffu, mn[d], o));
+            mx[d] = max(mx[d], __shfl_xor_sync(0xffffffffu, mx[d], o));
+        }
+        if (lane == 0) { sh[d][warp] = mn[d]; sh[3 + d][warp] = mx[d]; }
+    }
+    __syncthreads();
+    if (threadIdx.x < 6) {
+        const int c = threadIdx.x;
+        Real r = sh[c][0];
+        for (int w = 1; w < 8; ++w) r = c < 3 ? min(r, sh[c][w]) : max(r, sh[c][w]);
+        part[c] = c < 3 ? (r == big ? DBL_MAX : (double)r) : (r == -big ? -DBL_MAX : (double)r);
+    }
+}
+
 // lo = min, ext = max_d (hi_d - lo_d) in FP64, L = 2^k the smallest power of
 // two strictly greater than ext (k = 0 when ext = 0): with ext = f 2^e,
 // f in [0.5, 1), that power is 2^e.

@@ -22,7 +22,7 @@ __global__ void __launch_bounds__(256, sizeof(Real) == 4 ? 6 : 3) k_kick_drift_b
                                                         typename Vec4<Real>::T *__restrict__ xm, Real half_tau,
                                                         Real tau, int64_t n, double *__restrict__ part,
                                                         int32_t *dstatus) {
-    __shared__ double sh[6][8];
+    __shared__ Real sh[6][8];
     const Real big = sizeof(Real) == 4 ? (Real)FLT_MAX : (Real)DBL_MAX;
     Real mn[3] = {big, big, big}, mx[3] = {-big, -big, -big};
     bool bad = false;
@@ -45,27 +45,7 @@ __global__ void __launch_bounds__(256, sizeof(Real) == 4 ? 6 : 3) k_kick_drift_b
         xm[i] = p;
     }
     if (__any_sync(0xffffffffu, bad) && (threadIdx.x & 31) == 0) set_status(dstatus, TREE_DEV_NONFINITE);
-    double dmn[3], dmx[3];
-#pragma unroll
-    for (int d = 0; d < 3; ++d) {
-        dmn[d] = mn[d] == big ? DBL_MAX : (double)mn[d];
-        dmx[d] = mx[d] == -big ? -DBL_MAX : (double)mx[d];
-        for (int o = 16; o > 0; o >>= 1) {
-            dmn[d] = fmin(dmn[d], __shfl_xor_sync(0xffffffffu, dmn[d], o));
-            dmx[d] = fmax(dmx[d], __shfl_xor_sync(0xffffffffu, dmx[d], o));
-        }
-    }
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    if (lane == 0) {
-        for (int d = 0; d < 3; ++d) { sh[d][warp] = dmn[d]; sh[3 + d][warp] = dmx[d]; }
-    }
-    __syncthreads();
-    if (threadIdx.x < 6) {
-        const int c = threadIdx.x;
-        double r = sh[c][0];
-        for (int w = 1; w < (int)(blockDim.x >> 5); ++w) r = c < 3 ? fmin(r, sh[c][w]) : fmax(r, sh[c][w]);
-        part[blockIdx.x * 8 + c] = r;
-    }
+    block_minmax<Real>(mn, mx, big, sh, part + blockIdx.x * 8);
 }
 
 cudaError_t launch_kick_drift_box(TreeWorkspace *ws, void *x, void *v, const void *a, const void *m, double tau,

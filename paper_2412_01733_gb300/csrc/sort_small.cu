@@ -49,8 +49,8 @@ __global__ void __launch_bounds__(256) k_small_keys(const Real *__restrict__ x, 
                                                     const double *__restrict__ part, int nparts,
                                                     DevBox *__restrict__ box, uint64_t *__restrict__ key) {
     __shared__ Real sh[6][8];
+    __shared__ double res[6];
     __shared__ DevBox sbox;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     // a part without a finite value on an axis holds (DBL_MAX, -DBL_MAX) there
     const Real big = sizeof(Real) == 4 ? (Real)INFINITY : (Real)DBL_MAX;
     Real mn[3] = {big, big, big}, mx[3] = {-big, -big, -big};
@@ -61,22 +61,10 @@ __global__ void __launch_bounds__(256) k_small_keys(const Real *__restrict__ x, 
             mx[d] = max(mx[d], (Real)part[b * 8 + 3 + d]);
         }
     }
-#pragma unroll
-    for (int d = 0; d < 3; ++d) {
-        for (int o = 16; o > 0; o >>= 1) {
-            mn[d] = min(mn[d], __shfl_xor_sync(0xffffffffu, mn[d], o));
-            mx[d] = max(mx[d], __shfl_xor_sync(0xffffffffu, mx[d], o));
-        }
-        if (lane == 0) { sh[d][warp] = mn[d]; sh[3 + d][warp] = mx[d]; }
-    }
+    block_minmax<Real>(mn, mx, big, sh, res);
     __syncthreads();
     if (threadIdx.x == 0) {
-        double lo[3], hi[3];
-        for (int d = 0; d < 3; ++d) {
-            Real l = sh[d][0], h = sh[3 + d][0];
-            for (int w = 1; w < 8; ++w) { l = min(l, sh[d][w]); h = max(h, sh[3 + d][w]); }
-            lo[d] = l; hi[d] = h;
-        }
+        double lo[3] = {res[0], res[1], res[2]}, hi[3] = {res[3], res[4], res[5]};
         box_from_minmax(lo, hi, &sbox);
         if (blockIdx.x == 0) *box = sbox;
     }
