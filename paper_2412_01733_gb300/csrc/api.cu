@@ -290,8 +290,8 @@ tree_status_t tree_workspace_create(int64_t n_max, const TreeParams *p, TreeWork
              dalloc(&ws->ghead, (size_t)ws->groups_max) && dalloc(&ws->gtiles, (size_t)ws->groups_max);
         ws->tile_cap = ok ? (uint32_t)T : 0u;
     }
-    if (ok && n_max <= flat_octree_max())
-        ok = dalloc(&ws->sdig, N) && dalloc(&ws->flat_cnt, 513 * kLevels) && dalloc(&ws->nraw, NC);
+    ok = ok && dalloc(&ws->sdig, N) && dalloc(&ws->flat_cnt, ((size_t)flat_octree_blocks(n_max) + 1) * kLevels) &&
+         dalloc(&ws->nraw, NC);
     ws->chunks_cap = chunks_max;
     ws->box_cap = 1;
     if (!ok) {
@@ -450,7 +450,7 @@ static cudaError_t clear_build(TreeWorkspace *ws, int64_t n, cudaStream_t s) {
             e = cudaMemset2DAsync(ws->sort_status, (size_t)ws->sort_tiles_max * kRadix * word, 0, tiles * kRadix * word,
                                   (size_t)(kSortPasses + ws->seg_passes), s);
     }
-    if (e == cudaSuccess && !flat_octree(ws, n))
+    if (e == cudaSuccess && !flat_octree(ws))
         e = cudaMemsetAsync(ws->level_status, 0, (size_t)kLevels * ws->level_tiles_max * sizeof(uint32_t), s);
     return e;
 }

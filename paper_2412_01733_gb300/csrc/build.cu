@@ -557,7 +557,7 @@ __global__ void __launch_bounds__(kLevelThreads) k_level(
 }
 
 cudaError_t launch_octree(TreeWorkspace *ws, int64_t n, cudaStream_t s) {
-    if (flat_octree(ws, n)) return launch_octree_flat(ws, n, s);
+    if (flat_octree(ws)) return launch_octree_flat(ws, n, s);
     k_tree_init<<<grid_for(ws->nseg, 128, 1 << 20), 128, 0, s>>>(ws->ctr, ws->nfirst, ws->ncount, ws->nparent, n,
                                                                  ws->seg_off, ws->nseg);
     double maxl = (double)ws->nseg;

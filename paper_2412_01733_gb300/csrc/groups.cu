@@ -175,7 +175,7 @@ cudaError_t launch_groups(TreeWorkspace *ws, int64_t n, cudaStream_t s) {
         const cudaError_t e = cudaMemsetAsync(ws->gscan_status, 0, (size_t)tiles * sizeof(uint32_t), s);
         if (e != cudaSuccess) return e;
     }
-    if (!flat_octree(ws, n)) {
+    if (!flat_octree(ws)) {
         k_leaf_levels<<<grid_for(ws->node_cap, 256, 152 * 8), 256, 0, s>>>(ws->ctr, ws->ngeo, ws->nlink, ws->plev,
                                                                             ws->pleaf);
         ws->launches += 1;

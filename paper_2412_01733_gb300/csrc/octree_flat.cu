@@ -21,19 +21,21 @@
 // (with the walk groups: 144 us at N = 1031, 210 at 30011, 380 at 2^20); this
 // form is bound by latency too, but of three kernels (31, 31 and 87 us).
 // Blocks of kTile positions sum the counts of all blocks before them
-// themselves, which is cheaper than a look-back while there are at most
-// kFlatMaxBlocks of them; beyond (2^20 particles) k_level is 4 % of a force
-// and less, and stays.
+// themselves while there are at most kFlatMaxBlocks of them; beyond (2^20
+// particles) one more launch scans the blocks' counts, level by level.
 #include "common.cuh"
 
 namespace treegb {
 
 constexpr int kFlatThreads = 256;
 constexpr int kFlatMaxBlocks = 512;
-constexpr int kFlatItemsMax = 8;  // positions per thread: kFlatMaxBlocks * 256 * 8 = 2^20 particles
+constexpr int kFlatItemsMax = 8;  // positions per thread
 constexpr int kHalo = 16;         // leaf_cap at most
 
-int64_t flat_octree_max() { return (int64_t)kFlatMaxBlocks * kFlatThreads * kFlatItemsMax; }
+int64_t flat_octree_blocks(int64_t n_max) {
+    const int64_t nb = (n_max + kFlatThreads * kFlatItemsMax - 1) / (kFlatThreads * kFlatItemsMax);
+    return nb > kFlatMaxBlocks ? nb : kFlatMaxBlocks;
+}
 
 // Leading octal digits two keys share (21 if equal).
 __device__ __forceinline__ int shared_digits(uint64_t a, uint64_t b) {
@@ -93,12 +95,34 @@ __global__ void __launch_bounds__(kFlatThreads) k_flat_count(const uint64_t *__r
     }
 }
 
+// Scan of the blocks' counts of one level per block (many blocks): counts
+// become the numbers of nodes of the level in the blocks before; cnt[nblocks]
+// holds the totals.
+__global__ void __launch_bounds__(1024) k_flat_scan(uint32_t *__restrict__ cnt, int nblocks, const uint32_t *ctr) {
+    __shared__ uint32_t wt[32];
+    if (aborted(ctr, kStageAfter)) return;
+    uint32_t *c = cnt + blockIdx.x;  // level
+    const int per = (nblocks + 1023) / 1024;
+    const int b0 = threadIdx.x * per, b1 = min(nblocks, b0 + per);
+    uint32_t sum = 0;
+#pragma unroll 8
+    for (int b = b0; b < b1; ++b) sum += c[(size_t)b * kLevels];
+    uint32_t total;
+    uint32_t run = block_exclusive_scan(sum, wt, &total);
+#pragma unroll 8
+    for (int b = b0; b < b1; ++b) {
+        const uint32_t v = c[(size_t)b * kLevels];
+        c[(size_t)b * kLevels] = run;
+        run += v;
+    }
+    if (threadIdx.x == 0) c[(size_t)nblocks * kLevels] = total;
+}
+
 // The tree when the node array is too small for it: one block builds it level
 // by level, children of a node numbered only while they fit (as k_level).
 __device__ __noinline__ void flat_overflow(const uint64_t *__restrict__ skey, int64_t n, uint32_t *nfirst,
                                            uint32_t *ncount, uint4 *ngeo, uint2 *nlink, uint32_t *nparent,
-                                           uint8_t *plev, uint32_t *pleaf, uint32_t *ctr, uint32_t lcap,
-                                           uint32_t node_cap, int32_t *dstatus) {
+                                           uint32_t *ctr, uint32_t lcap, uint32_t node_cap, int32_t *dstatus) {
     __shared__ uint32_t wt[32], s_trunc;
     const uint32_t tid = threadIdx.x;
     if (tid == 0) {
@@ -135,8 +159,6 @@ __device__ __noinline__ void flat_overflow(const uint64_t *__restrict__ skey, in
                 ngeo[node] = make_uint4(compact3(k0 >> 2) & cmask, compact3(k0 >> 1) & cmask, compact3(k0) & cmask,
                                         (uint32_t)L | (internal ? 0u : 0x100u));
                 nlink[node] = internal ? make_uint2(cf, nch) : make_uint2(first, count);
-                if (!internal)
-                    for (uint32_t j = first; j < first + count; ++j) { plev[j] = (uint8_t)L; pleaf[j] = node; }
             }
             if (internal) {
                 uint32_t c = cf;
@@ -163,10 +185,11 @@ __device__ __noinline__ void flat_overflow(const uint64_t *__restrict__ skey, in
 // Second kernel: numbers, starts, parents and geometry of the nodes that
 // start in the block's positions; ends of the nodes that end there; leaf of
 // every particle.  raw[node] = {first child or first particle, its end}.
-template <int ITEMS>
+// SCANNED: cnt comes from k_flat_scan.
+template <int ITEMS, bool SCANNED>
 __global__ void __launch_bounds__(kFlatThreads) k_flat_nodes(
-    const uint64_t *__restrict__ skey, int64_t n, const uint8_t *__restrict__ sdig, uint8_t *__restrict__ plev,
-    const uint32_t *__restrict__ cnt, int nblocks, uint32_t *__restrict__ nfirst, uint32_t *__restrict__ ncount,
+    const uint64_t *__restrict__ skey, int64_t n, const uint8_t *__restrict__ sdig,
+    const uint8_t *__restrict__ plev, const uint32_t *__restrict__ cnt, int nblocks, uint32_t *__restrict__ nfirst, uint32_t *__restrict__ ncount,
     uint4 *__restrict__ ngeo, uint2 *__restrict__ nlink, uint2 *__restrict__ raw, uint32_t *__restrict__ nparent,
     uint32_t *__restrict__ pleaf, uint32_t *ctr, uint32_t lcap, uint32_t node_cap, int32_t *dstatus) {
     constexpr int kTile = kFlatThreads * ITEMS;
@@ -180,7 +203,12 @@ __global__ void __launch_bounds__(kFlatThreads) k_flat_nodes(
     // nodes per level in the blocks before this one, and in all
     {
         uint32_t before = 0, all = 0;
-        if (lane < kLevels)
+        if (SCANNED) {
+            if (warp == 0 && lane < kLevels) {
+                before = cnt[(size_t)blockIdx.x * kLevels + lane];  // (position n's own block: the totals)
+                all = cnt[(size_t)nblocks * kLevels + lane];
+            }
+        } else if (lane < kLevels)
             for (int b = warp; b < nblocks; b += kWarps) {
                 const uint32_t c = cnt[(size_t)b * kLevels + lane];
                 all += c;
@@ -209,8 +237,8 @@ __global__ void __launch_bounds__(kFlatThreads) k_flat_nodes(
     __syncthreads();
     if (s_end > node_cap) {
         if (blockIdx.x == 0) {
-            if (tid == 0) ctr[kCtrFlatFull] = 1;  // the links below are final: k_flat_links has nothing to do
-            flat_overflow(skey, n, nfirst, ncount, ngeo, nlink, nparent, plev, pleaf, ctr, lcap, node_cap, dstatus);
+            if (tid == 0) ctr[kCtrFlatFull] = 1;  // the links below are final; the leaves' particles follow
+            flat_overflow(skey, n, nfirst, ncount, ngeo, nlink, nparent, ctr, lcap, node_cap, dstatus);
         }
         return;
     }
@@ -287,12 +315,26 @@ __global__ void __launch_bounds__(kFlatThreads) k_flat_nodes(
     }
 }
 
-// Third kernel: ends become counts.
+// Third kernel: ends become counts.  (When the node array was too small, the
+// counts are there, and the particles learn their leaves: a warp per leaf.)
 __global__ void __launch_bounds__(256) k_flat_links(const uint32_t *__restrict__ ctr, const uint2 *__restrict__ raw,
                                                     const uint32_t *__restrict__ nfirst, uint32_t *__restrict__ ncount,
-                                                    uint2 *__restrict__ nlink) {
-    if (aborted(ctr, kStageAfter) || ctr[kCtrFlatFull]) return;
+                                                    const uint4 *__restrict__ ngeo, uint2 *__restrict__ nlink,
+                                                    uint8_t *__restrict__ plev, uint32_t *__restrict__ pleaf) {
+    if (aborted(ctr, kStageAfter)) return;
     const uint32_t nn = ctr[kCtrLevelStart + kLevels];
+    if (ctr[kCtrFlatFull]) {
+        for (uint32_t c = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; c < nn; c += (gridDim.x * blockDim.x) >> 5) {
+            const uint32_t w = ngeo[c].w;
+            if (!((w >> 8) & 1u)) continue;
+            const uint2 l = nlink[c];
+            for (uint32_t j = l.x + (threadIdx.x & 31); j < l.x + l.y; j += 32) {
+                plev[j] = (uint8_t)(w & 0xffu);
+                pleaf[j] = c;
+            }
+        }
+        return;
+    }
     for (uint32_t c = blockIdx.x * blockDim.x + threadIdx.x; c < nn; c += gridDim.x * blockDim.x) {
         const uint2 r = raw[c];
         nlink[c] = make_uint2(r.x, r.y - r.x);
@@ -300,14 +342,16 @@ __global__ void __launch_bounds__(256) k_flat_links(const uint32_t *__restrict__
     }
 }
 
-template <int ITEMS>
+template <int ITEMS, bool SCANNED>
 static void flat_launch(TreeWorkspace *ws, int64_t n, cudaStream_t s) {
     const int nb = (int)((n + kFlatThreads * ITEMS - 1) / (kFlatThreads * ITEMS));
     k_flat_count<ITEMS><<<nb, kFlatThreads, 0, s>>>(ws->key, n, ws->p.leaf_cap, ws->sdig, ws->plev, ws->flat_cnt,
                                                    ws->ctr);
+    if (SCANNED) k_flat_scan<<<kLevels, 1024, 0, s>>>(ws->flat_cnt, nb, ws->ctr);
+    ws->launches += SCANNED ? 3 : 2;
     // position n may need a block of its own
     const int nb1 = (int)((n + kFlatThreads * ITEMS) / (kFlatThreads * ITEMS));
-    k_flat_nodes<ITEMS><<<nb1, kFlatThreads, 0, s>>>(ws->key, n, ws->sdig, ws->plev, ws->flat_cnt, nb, ws->nfirst,
+    k_flat_nodes<ITEMS, SCANNED><<<nb1, kFlatThreads, 0, s>>>(ws->key, n, ws->sdig, ws->plev, ws->flat_cnt, nb, ws->nfirst,
                                                     ws->ncount, ws->ngeo, ws->nlink, ws->nraw, ws->nparent, ws->pleaf,
                                                     ws->ctr, (uint32_t)ws->p.leaf_cap, (uint32_t)ws->node_cap,
                                                     ws->dstatus);
@@ -316,13 +360,14 @@ static void flat_launch(TreeWorkspace *ws, int64_t n, cudaStream_t s) {
 cudaError_t launch_octree_flat(TreeWorkspace *ws, int64_t n, cudaStream_t s) {
     // as few positions per thread as give at most kFlatMaxBlocks blocks
     const int64_t one = (int64_t)kFlatMaxBlocks * kFlatThreads;
-    if (n <= one) flat_launch<1>(ws, n, s);
-    else if (n <= 2 * one) flat_launch<2>(ws, n, s);
-    else if (n <= 4 * one) flat_launch<4>(ws, n, s);
-    else flat_launch<kFlatItemsMax>(ws, n, s);
+    if (n <= one) flat_launch<1, false>(ws, n, s);
+    else if (n <= 2 * one) flat_launch<2, false>(ws, n, s);
+    else if (n <= 4 * one) flat_launch<4, false>(ws, n, s);
+    else if (n <= kFlatItemsMax * one) flat_launch<kFlatItemsMax, false>(ws, n, s);
+    else flat_launch<kFlatItemsMax, true>(ws, n, s);
     k_flat_links<<<grid_for(ws->node_cap, 256, 152 * 8), 256, 0, s>>>(ws->ctr, ws->nraw, ws->nfirst, ws->ncount,
-                                                                      ws->nlink);
-    ws->launches += 3;
+                                                                      ws->ngeo, ws->nlink, ws->plev, ws->pleaf);
+    ws->launches += 1;
     return cudaGetLastError();
 }
 

@@ -1,8 +1,8 @@
 """The octree built straight from adjacent keys equals the level-by-level one.
 
-A workspace made for more particles than the flat form serves builds level by
-level, so the same positions on both are the comparison: every array of the
-tree, the walk groups and the interaction lists, bit for bit.
+A workspace for more than 65536 particles with a node array of its own size
+builds level by level, so the same positions on both are the comparison: every
+array of the tree and the walk groups, bit for bit.
 """
 import pytest
 import torch
@@ -11,7 +11,7 @@ from paper_2412_01733_gb300 import inputs
 
 pytestmark = pytest.mark.gpu
 
-BIG = (1 << 20) + 1  # above the flat form's largest workspace
+BIG = 65537  # the smallest workspace that builds level by level (given a node array's size)
 
 
 def _clumped(n):
@@ -23,7 +23,8 @@ def _clumped(n):
 
 
 # sizes at the edges of a warp, a block, a block of several items, and of leaf_cap
-SIZES = [1, 2, 8, 9, 16, 17, 31, 32, 33, 255, 256, 257, 1023, 131072, 131073, 262145, 524289, 1 << 20]
+SIZES = [1, 2, 8, 9, 16, 17, 31, 32, 33, 255, 256, 257, 1023, 131072, 131073, 262145, 524289, 1 << 20,
+         (1 << 20) + 1, 3000001]
 
 
 @pytest.mark.parametrize("n", SIZES)
@@ -31,7 +32,8 @@ SIZES = [1, 2, 8, 9, 16, 17, 31, 32, 33, 255, 256, 257, 1023, 131072, 131073, 26
 def test_flat_octree_equals_level_by_level(n, leaf_cap):
     from paper_2412_01733_gb300 import treegb as tg
     x = (_clumped(n) if n >= 255 else inputs.plummer(n, 5)[0]).to("cuda", torch.float32).contiguous()
-    with tg.Workspace(n, leaf_cap=leaf_cap) as flat, tg.Workspace(BIG, leaf_cap=leaf_cap) as level:
+    with tg.Workspace(n, leaf_cap=leaf_cap) as flat, tg.Workspace(max(n, BIG), leaf_cap=leaf_cap,
+                                                                     node_cap=max(n, BIG) * 5) as level:
         for ws in (flat, level):
             ws.build(x)
         a, b = flat.export_tree(), level.export_tree()
