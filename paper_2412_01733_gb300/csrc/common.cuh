@@ -583,11 +583,11 @@ inline bool small_sort(const TreeWorkspace *ws, int64_t n) {
 int64_t flat_octree_blocks(int64_t n_max);  // blocks whose counts flat_cnt holds
 cudaError_t launch_octree_flat(TreeWorkspace *ws, int64_t n, cudaStream_t s);
 // Whether launch_octree takes the flat form (leaf levels then come with the
-// octree): one system.  A tree that does not fit the node array is built by
+// octree).  A tree that does not fit the node array is built by
 // one block there, so a workspace with a node array of the caller's own size
 // takes the level-by-level form unless it is small.
 inline bool flat_octree(const TreeWorkspace *ws) {
-    return ws->nseg == 1 && (ws->p.node_cap == 0 || ws->n_max <= 65536);
+    return ws->p.node_cap == 0 || ws->n_max <= 65536;
 }
 // groups.cu
 cudaError_t launch_groups(TreeWorkspace *ws, int64_t n, cudaStream_t s);

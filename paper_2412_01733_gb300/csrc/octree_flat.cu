@@ -1,8 +1,9 @@
-// octree_flat.cu -- the breadth-first octree of one system straight from its
-// sorted keys, in three launches (build.cu builds it level by level).
+// octree_flat.cu -- the breadth-first octree straight from the sorted keys, in
+// three launches (build.cu builds it level by level).
 //
-// With s(i) the number of leading octal digits that keys i-1 and i share
-// (s(0) = -1) and t(j) that of keys j and j + leaf_cap (-1 past the end):
+// With s(i) the number of leading octal digits that keys i-1 and i share (-1
+// where a system starts) and t(j) that of keys j and j + leaf_cap (-1 past the
+// end of j's system):
 //   - a cell of level L > 0 is a node iff its parent holds more than leaf_cap
 //     particles, i.e. iff some leaf_cap + 1 consecutive particles of the
 //     parent share L - 1 digits; so the leaf that holds particle i has level
@@ -45,16 +46,30 @@ __device__ __forceinline__ int shared_digits(uint64_t a, uint64_t b) {
 
 // First kernel: s(i) + 1 and lev(i) of every particle, and each block's
 // number of nodes per level.
-template <int ITEMS>
+template <int ITEMS, bool SEG>
 __global__ void __launch_bounds__(kFlatThreads) k_flat_count(const uint64_t *__restrict__ skey, int64_t n, int lcap,
+                                                             const int64_t *__restrict__ seg_off, int64_t nseg,
                                                              uint8_t *__restrict__ sdig, uint8_t *__restrict__ plev,
                                                              uint32_t *__restrict__ cnt, const uint32_t *ctr) {
     constexpr int kTile = kFlatThreads * ITEMS;
     __shared__ uint64_t key[kTile + 2 * kHalo + 1];  // key[k]: particle b0 - kHalo + k
     __shared__ int8_t t[kTile + kHalo];              // t[k]: of particle b0 - kHalo + k
+    __shared__ uint8_t bnd[SEG ? kTile + 2 * kHalo + 1 : 1];  // a system starts at particle b0 - kHalo + k
     __shared__ uint32_t diff[24];
     if (aborted(ctr, kStageAfter)) return;
     const int64_t b0 = (int64_t)blockIdx.x * kTile;
+    if constexpr (SEG) {
+        for (int k = threadIdx.x; k < kTile + 2 * kHalo + 1; k += kFlatThreads) bnd[k] = 0;
+        __syncthreads();
+        // the systems that start inside the tile and its halo
+        const int64_t lo = b0 - kHalo, hi = b0 + kTile + kHalo;
+        for (int64_t b = (lo > 0 ? seg_find(seg_off, nseg, lo < n ? lo : n - 1) : 0) + threadIdx.x; b < nseg;
+             b += kFlatThreads) {
+            const int64_t o = seg_off[b];
+            if (o >= hi) break;
+            if (o >= lo) bnd[o - lo] = 1;
+        }
+    }
     if (threadIdx.x < 24) diff[threadIdx.x] = 0;
     for (int k = threadIdx.x; k < kTile + 2 * kHalo; k += kFlatThreads) {
         const int64_t i = b0 - kHalo + k;
@@ -63,7 +78,10 @@ __global__ void __launch_bounds__(kFlatThreads) k_flat_count(const uint64_t *__r
     __syncthreads();
     for (int k = threadIdx.x; k < kTile + kHalo; k += kFlatThreads) {
         const int64_t j = b0 - kHalo + k;
-        t[k] = j >= 0 && j + lcap < n ? (int8_t)shared_digits(key[k], key[k + lcap]) : (int8_t)-1;
+        bool same = j >= 0 && j + lcap < n;
+        if constexpr (SEG)
+            for (int o = 1; o <= lcap; ++o) same &= bnd[k + o] == 0;
+        t[k] = same ? (int8_t)shared_digits(key[k], key[k + lcap]) : (int8_t)-1;
     }
     __syncthreads();
 #pragma unroll
@@ -74,7 +92,9 @@ __global__ void __launch_bounds__(kFlatThreads) k_flat_count(const uint64_t *__r
         int m = -1;
         for (int o = 0; o <= lcap; ++o) m = max(m, (int)t[k + kHalo - o]);
         const int lev = min(kMaxLevel, 1 + m);
-        const int sd = i > 0 ? shared_digits(key[k + kHalo - 1], key[k + kHalo]) + 1 : 0;
+        bool head = i == 0;
+        if constexpr (SEG) head = bnd[k + kHalo] != 0;
+        const int sd = head ? 0 : shared_digits(key[k + kHalo - 1], key[k + kHalo]) + 1;
         sdig[i] = (uint8_t)sd;
         plev[i] = (uint8_t)lev;
         if (sd <= lev) {  // nodes start here at levels sd .. lev
@@ -120,16 +140,19 @@ __global__ void __launch_bounds__(1024) k_flat_scan(uint32_t *__restrict__ cnt, 
 
 // The tree when the node array is too small for it: one block builds it level
 // by level, children of a node numbered only while they fit (as k_level).
-__device__ __noinline__ void flat_overflow(const uint64_t *__restrict__ skey, int64_t n, uint32_t *nfirst,
+__device__ __noinline__ void flat_overflow(const uint64_t *__restrict__ skey, int64_t n,
+                                           const int64_t *__restrict__ seg_off, int64_t nseg, uint32_t *nfirst,
                                            uint32_t *ncount, uint4 *ngeo, uint2 *nlink, uint32_t *nparent,
                                            uint32_t *ctr, uint32_t lcap, uint32_t node_cap, int32_t *dstatus) {
     __shared__ uint32_t wt[32], s_trunc;
     const uint32_t tid = threadIdx.x;
-    if (tid == 0) {
-        nfirst[0] = 0; ncount[0] = (uint32_t)n; nparent[0] = 0;
-        ctr[kCtrLevelStart] = 0;
+    for (int64_t b = tid; b < nseg; b += kFlatThreads) {
+        nfirst[b] = nseg > 1 ? (uint32_t)seg_off[b] : 0u;
+        ncount[b] = nseg > 1 ? (uint32_t)(seg_off[b + 1] - seg_off[b]) : (uint32_t)n;
+        nparent[b] = (uint32_t)b;
     }
-    uint32_t start = 0, end = 1;
+    if (tid == 0) ctr[kCtrLevelStart] = 0;
+    uint32_t start = 0, end = (uint32_t)nseg;
     for (int L = 0; L < kLevels; ++L) {
         if (tid == 0) s_trunc = 0xffffffffu;
         __syncthreads();
@@ -191,7 +214,8 @@ __global__ void __launch_bounds__(kFlatThreads) k_flat_nodes(
     const uint64_t *__restrict__ skey, int64_t n, const uint8_t *__restrict__ sdig,
     const uint8_t *__restrict__ plev, const uint32_t *__restrict__ cnt, int nblocks, uint32_t *__restrict__ nfirst, uint32_t *__restrict__ ncount,
     uint4 *__restrict__ ngeo, uint2 *__restrict__ nlink, uint2 *__restrict__ raw, uint32_t *__restrict__ nparent,
-    uint32_t *__restrict__ pleaf, uint32_t *ctr, uint32_t lcap, uint32_t node_cap, int32_t *dstatus) {
+    uint32_t *__restrict__ pleaf, uint32_t *ctr, uint32_t lcap, uint32_t node_cap, int32_t *dstatus,
+    const int64_t *__restrict__ seg_off, int64_t nseg) {
     constexpr int kTile = kFlatThreads * ITEMS;
     constexpr int kChunks = kTile / 32, kWarps = kFlatThreads / 32;
     __shared__ uint32_t base[kChunks][24];  // per chunk of 32 positions: number of its first node of each level
@@ -238,7 +262,7 @@ __global__ void __launch_bounds__(kFlatThreads) k_flat_nodes(
     if (s_end > node_cap) {
         if (blockIdx.x == 0) {
             if (tid == 0) ctr[kCtrFlatFull] = 1;  // the links below are final; the leaves' particles follow
-            flat_overflow(skey, n, nfirst, ncount, ngeo, nlink, nparent, ctr, lcap, node_cap, dstatus);
+            flat_overflow(skey, n, seg_off, nseg, nfirst, ncount, ngeo, nlink, nparent, ctr, lcap, node_cap, dstatus);
         }
         return;
     }
@@ -303,7 +327,7 @@ __global__ void __launch_bounds__(kFlatThreads) k_flat_nodes(
             if (starts) {
                 const uint32_t cmask = ~((1u << (kBits - L)) - 1u);
                 nfirst[id] = (uint32_t)i;
-                nparent[id] = L == 0 ? 0u : L == sd[q] ? prev - 1u : up;
+                nparent[id] = L == 0 ? id : L == sd[q] ? prev - 1u : up;
                 ngeo[id] = make_uint4(qx & cmask, qy & cmask, qz & cmask, (uint32_t)L | (L == lv[q] ? 0x100u : 0u));
                 if (L > sd[q]) raw[up].x = id;
                 if (L == lv[q]) raw[id].x = (uint32_t)i;
@@ -345,8 +369,12 @@ __global__ void __launch_bounds__(256) k_flat_links(const uint32_t *__restrict__
 template <int ITEMS, bool SCANNED>
 static void flat_launch(TreeWorkspace *ws, int64_t n, cudaStream_t s) {
     const int nb = (int)((n + kFlatThreads * ITEMS - 1) / (kFlatThreads * ITEMS));
-    k_flat_count<ITEMS><<<nb, kFlatThreads, 0, s>>>(ws->key, n, ws->p.leaf_cap, ws->sdig, ws->plev, ws->flat_cnt,
-                                                   ws->ctr);
+    if (ws->nseg > 1)
+        k_flat_count<ITEMS, true><<<nb, kFlatThreads, 0, s>>>(ws->key, n, ws->p.leaf_cap, ws->seg_off, ws->nseg,
+                                                             ws->sdig, ws->plev, ws->flat_cnt, ws->ctr);
+    else
+        k_flat_count<ITEMS, false><<<nb, kFlatThreads, 0, s>>>(ws->key, n, ws->p.leaf_cap, nullptr, 1, ws->sdig,
+                                                              ws->plev, ws->flat_cnt, ws->ctr);
     if (SCANNED) k_flat_scan<<<kLevels, 1024, 0, s>>>(ws->flat_cnt, nb, ws->ctr);
     ws->launches += SCANNED ? 3 : 2;
     // position n may need a block of its own
@@ -354,7 +382,7 @@ static void flat_launch(TreeWorkspace *ws, int64_t n, cudaStream_t s) {
     k_flat_nodes<ITEMS, SCANNED><<<nb1, kFlatThreads, 0, s>>>(ws->key, n, ws->sdig, ws->plev, ws->flat_cnt, nb, ws->nfirst,
                                                     ws->ncount, ws->ngeo, ws->nlink, ws->nraw, ws->nparent, ws->pleaf,
                                                     ws->ctr, (uint32_t)ws->p.leaf_cap, (uint32_t)ws->node_cap,
-                                                    ws->dstatus);
+                                                    ws->dstatus, ws->seg_off, ws->nseg);
 }
 
 cudaError_t launch_octree_flat(TreeWorkspace *ws, int64_t n, cudaStream_t s) {

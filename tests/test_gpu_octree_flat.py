@@ -59,3 +59,28 @@ def test_flat_octree_out_of_nodes_equals_level_by_level(n, cap):
             assert torch.equal(a[k], b[k]), k
         assert torch.equal(flat.export_groups(), level.export_groups())
         assert all(torch.equal(s, t) for s, t in zip(*out))
+
+
+@pytest.mark.parametrize("sizes", [[1, 1], [1, 2, 17, 33, 700, 4101, 9000], [1] * 600 + [16] * 40 + [17, 3000],
+                                   [255, 1, 256, 1, 2048, 16, 2032], [140000, 5, 140000]])
+@pytest.mark.parametrize("leaf_cap,cap", [(16, 0), (1, 0), (4, 700)])
+def test_flat_octree_of_systems(sizes, leaf_cap, cap):
+    """Several systems (boundaries inside tiles, halos and leaves); cap: also when the node array is too small."""
+    from paper_2412_01733_gb300 import treegb as tg
+    off = [0]
+    for k in sizes:
+        off.append(off[-1] + k)
+    n = off[-1]
+    x = torch.cat([inputs.plummer(k, 70 + b % 7)[0] for b, k in enumerate(sizes)], 1).to("cuda", torch.float32).contiguous()
+    if cap and len(sizes) >= cap:
+        pytest.skip("more systems than nodes")
+    with tg.Workspace(n, leaf_cap=leaf_cap, **(dict(node_cap=cap) if cap and n <= 65536 else {})) as flat, \
+            tg.Workspace(max(n, BIG), leaf_cap=leaf_cap, node_cap=cap if cap and n <= 65536 else 5 * max(n, BIG)) as level:
+        for ws in (flat, level):
+            ws.set_segments(off)
+            ws.build(x)
+        a, b = flat.export_tree(), level.export_tree()
+        assert flat.status() == level.status()
+        for k in ("keys", "perm", "level", "corner", "first", "count", "child", "nchild"):
+            assert torch.equal(a[k], b[k]), k
+        assert torch.equal(flat.export_groups(), level.export_groups())
