@@ -69,16 +69,11 @@ int64_t default_node_cap(int64_t n_max, int leaf_cap) {
 }
 
 void free_all(TreeWorkspace *ws) {
-    void *ptrs[] = {ws->key, ws->key_alt, ws->idx, ws->idx_alt, ws->hist, ws->sort_status, ws->level_status,
-                    ws->ctr, ws->part, ws->box, ws->spos, ws->nfirst, ws->ncount, ws->ngeo, ws->nlink,
-                    ws->mom64, ws->mom_a, ws->mom_b, ws->mom_c, ws->dstatus, ws->stats, ws->gstat,
-                    ws->list_cnt, ws->pc_list, ws->pp_list, ws->direct_part, ws->dmac, ws->gorder,
-                    ws->gkey, ws->gbucket, ws->gfirst, ws->plev, ws->ccount, ws->coff, ws->gscan_status,
-                    ws->adj_cot, ws->adj_xg, ws->adj_mg, ws->adj_ccot, ws->pleaf, ws->nparent,
-                    ws->seg_off, ws->seg_cstart, ws->seg_bchunk, ws->seg_bfirst, ws->seg_part,
-                    ws->seg_digit_off, ws->cmask, ws->morder, ws->mbucket, ws->xm, ws->hs_x, ws->hs_v,
-                    ws->hs_m, ws->hs_a, ws->hs_phi, ws->hs_diag, ws->dctl, ws->tile_hdr, ws->tile_idx,
-                    ws->tile_part, ws->tile_next, ws->ghead, ws->gtiles, ws->sdig, ws->flat_cnt, ws->nraw, ws->marrived};
+    // (everything else lies in the arena)
+    void *ptrs[] = {ws->arena, ws->box, ws->ccount, ws->coff, ws->cmask, ws->gscan_status, ws->list_cnt, ws->pc_list,
+                    ws->pp_list, ws->direct_part, ws->adj_cot, ws->adj_xg, ws->adj_mg, ws->adj_ccot, ws->seg_off,
+                    ws->seg_cstart, ws->seg_bchunk, ws->seg_bfirst, ws->seg_part, ws->seg_digit_off, ws->hs_x,
+                    ws->hs_v, ws->hs_m, ws->hs_a, ws->hs_phi, ws->hs_diag};
     for (void *p : ptrs)
         if (p) cudaFree(p);
     if (ws->graph_exec) cudaGraphExecDestroy(ws->graph_exec);
@@ -101,6 +96,19 @@ void free_all(TreeWorkspace *ws) {
     ws->ev.clear();
     ws->ev_phase.clear();
 }
+
+// Arrays of a workspace laid out in one allocation: a first pass with no base
+// adds up the sizes, a second one hands out the addresses.
+struct Arena {
+    unsigned char *base = nullptr;
+    size_t size = 0;
+    template <typename T>
+    void take(T **p, size_t count, size_t elem = sizeof(T)) {
+        if (base) *p = reinterpret_cast<T *>(base + size);
+        size += ((count ? count : 1) * elem + 255) & ~(size_t)255;
+    }
+    void take(void **p, size_t count, size_t elem) { take((unsigned char **)p, count, elem); }
+};
 
 template <typename T>
 bool dalloc(T **p, size_t count) {
@@ -263,35 +271,73 @@ tree_status_t tree_workspace_create(int64_t n_max, const TreeParams *p, TreeWork
     const int64_t chunks_max = (n_max + 15) / 16 + 1;
     const size_t v4 = p->precision == TREE_F64 ? sizeof(double4a) : sizeof(float4);
     const size_t v2 = p->precision == TREE_F64 ? sizeof(double2a) : sizeof(float2);
-    bool ok = dalloc(&ws->key, N) && dalloc(&ws->key_alt, N) && dalloc(&ws->idx, N) && dalloc(&ws->idx_alt, N) &&
-              dalloc(&ws->hist, 2 * kSortPasses * kRadix) &&
-              dalloc(&ws->sort_status, (size_t)(kSortPasses + kSegPassesMax) * ws->sort_tiles_max * kRadix) &&
-              dalloc(&ws->level_status, (size_t)kLevels * ws->level_tiles_max) && dalloc(&ws->ctr, kCtrCount) &&
-              dalloc(&ws->part, (size_t)kMaxBlocksReduce * 8) && dalloc(&ws->box, 1) &&
-              dalloc((unsigned char **)&ws->spos, N * v4) && dalloc((unsigned char **)&ws->xm, N * v4) &&
-              dalloc(&ws->nfirst, NC) && dalloc(&ws->ncount, NC) &&
-              dalloc(&ws->ngeo, NC) && dalloc(&ws->nlink, NC) && dalloc(&ws->mom64, 10 * NC) &&
-              dalloc(&ws->morder, NC) && dalloc(&ws->mbucket, 3 * kMomBuckets + 1) && dalloc(&ws->marrived, NC) &&
-              dalloc((unsigned char **)&ws->mom_a, NC * v4) && dalloc((unsigned char **)&ws->mom_b, NC * v4) &&
-              dalloc((unsigned char **)&ws->mom_c, NC * v2) && dalloc(&ws->dstatus, 1) &&
-              dalloc(&ws->stats, kStatCount) && dalloc(&ws->gstat, (size_t)ws->groups_max) &&
-              dalloc(&ws->gorder, (size_t)ws->groups_max) && dalloc(&ws->gkey, (size_t)ws->groups_max) &&
-              dalloc(&ws->gbucket, 64) && dalloc(&ws->gfirst, (size_t)ws->groups_max + 1) &&
-              dalloc(&ws->plev, N) && dalloc(&ws->pleaf, N) && dalloc(&ws->nparent, NC) &&
-              dalloc(&ws->ccount, (size_t)chunks_max) && dalloc(&ws->coff, (size_t)chunks_max) &&
-              dalloc(&ws->cmask, 2 * (size_t)chunks_max) &&
-              dalloc(&ws->gscan_status, (size_t)(chunks_max / 2048 + 2)) &&
-              dalloc(&ws->dmac, kLevels) && dalloc(&ws->dctl, 1);
-    if (ok && n_max > 0 && n_max <= (p->precision == TREE_F64 ? kSplitMaxN64 : kSplitMaxN32)) {
-        // tile slots of the split walk (groups of 64 use half of them: two targets per lane)
-        const size_t T = (((size_t)n_max * kTilesPer + 4096) / kTileChunk) * kTileChunk;
-        ok = dalloc(&ws->tile_hdr, T) && dalloc(&ws->tile_idx, T * 32) && dalloc(&ws->tile_next, T / kTileChunk) &&
-             dalloc((unsigned char **)&ws->tile_part, T * 32 * v4) &&
-             dalloc(&ws->ghead, (size_t)ws->groups_max) && dalloc(&ws->gtiles, (size_t)ws->groups_max);
-        ws->tile_cap = ok ? (uint32_t)T : 0u;
+    // tile slots of the split walk (groups of 64 use half of them: two targets per lane)
+    size_t T = 0;
+    if (n_max > 0 && n_max <= (p->precision == TREE_F64 ? kSplitMaxN64 : kSplitMaxN32))
+        T = (((size_t)n_max * kTilesPer + 4096) / kTileChunk) * kTileChunk;
+    auto lay_out = [&](Arena &A) {
+        const size_t G = (size_t)ws->groups_max;
+        // these four start at zero
+        A.take(&ws->dctl, 1);
+        A.take(&ws->dstatus, 1);
+        A.take(&ws->stats, kStatCount);
+        A.take(&ws->marrived, NC);
+        const size_t zeroed = A.size;
+        A.take(&ws->ctr, kCtrCount);
+        A.take(&ws->hist, 2 * kSortPasses * kRadix);
+        A.take(&ws->part, (size_t)kMaxBlocksReduce * 8);
+        A.take(&ws->mbucket, 3 * kMomBuckets + 1);
+        A.take(&ws->gbucket, 64);
+        A.take(&ws->dmac, kLevels);
+        A.take(&ws->key, N);
+        A.take(&ws->key_alt, N);
+        A.take(&ws->idx, N);
+        A.take(&ws->idx_alt, N);
+        A.take(&ws->sort_status, (size_t)(kSortPasses + kSegPassesMax) * ws->sort_tiles_max * kRadix);
+        A.take(&ws->level_status, (size_t)kLevels * ws->level_tiles_max);
+        A.take(&ws->spos, N, v4);
+        A.take(&ws->xm, N, v4);
+        A.take(&ws->plev, N);
+        A.take(&ws->pleaf, N);
+        A.take(&ws->sdig, N);
+        A.take(&ws->flat_cnt, ((size_t)flat_octree_blocks(n_max) + 1) * kLevels);
+        A.take(&ws->nfirst, NC);
+        A.take(&ws->ncount, NC);
+        A.take(&ws->nparent, NC);
+        A.take(&ws->ngeo, NC);
+        A.take(&ws->nlink, NC);
+        A.take(&ws->nraw, NC);
+        A.take(&ws->mom64, 10 * NC);
+        A.take(&ws->morder, NC);
+        A.take(&ws->mom_a, NC, v4);
+        A.take(&ws->mom_b, NC, v4);
+        A.take(&ws->mom_c, NC, v2);
+        A.take(&ws->gstat, G);
+        A.take(&ws->gorder, G);
+        A.take(&ws->gkey, G);
+        A.take(&ws->gfirst, G + 1);
+        if (T > 0) {
+            A.take(&ws->tile_hdr, T);
+            A.take(&ws->tile_idx, T * 32);
+            A.take(&ws->tile_next, T / kTileChunk);
+            A.take(&ws->tile_part, T * 32, v4);
+            A.take(&ws->ghead, G);
+            A.take(&ws->gtiles, G);
+        }
+        return zeroed;
+    };
+    Arena A;
+    const size_t zeroed = lay_out(A);
+    // the arrays that tree_set_segments may replace are allocations of their own
+    const bool ok = dalloc((unsigned char **)&ws->arena, A.size) && dalloc(&ws->box, 1) &&
+                    dalloc(&ws->ccount, (size_t)chunks_max) && dalloc(&ws->coff, (size_t)chunks_max) &&
+                    dalloc(&ws->cmask, 2 * (size_t)chunks_max) &&
+                    dalloc(&ws->gscan_status, (size_t)(chunks_max / 2048 + 2));
+    if (ok) {
+        A = Arena{static_cast<unsigned char *>(ws->arena), 0};
+        lay_out(A);
+        ws->tile_cap = (uint32_t)T;
     }
-    ok = ok && dalloc(&ws->sdig, N) && dalloc(&ws->flat_cnt, ((size_t)flat_octree_blocks(n_max) + 1) * kLevels) &&
-         dalloc(&ws->nraw, NC);
     ws->chunks_cap = chunks_max;
     ws->box_cap = 1;
     if (!ok) {
@@ -301,9 +347,7 @@ tree_status_t tree_workspace_create(int64_t n_max, const TreeParams *p, TreeWork
         return TREE_ERR_ALLOC;
     }
     const DevCtl ctl{kWaitCycles, -1};
-    if (cudaMemset(ws->dstatus, 0, sizeof(int32_t)) != cudaSuccess ||
-        cudaMemset(ws->marrived, 0, NC * sizeof(uint32_t)) != cudaSuccess ||
-        cudaMemset(ws->stats, 0, kStatCount * sizeof(unsigned long long)) != cudaSuccess ||
+    if (cudaMemset(ws->arena, 0, zeroed) != cudaSuccess ||
         cudaMemcpy(ws->dctl, &ctl, sizeof(ctl), cudaMemcpyHostToDevice) != cudaSuccess) {
         free_all(ws);
         delete ws;

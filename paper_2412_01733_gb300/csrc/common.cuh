@@ -130,6 +130,7 @@ struct TreeWorkspace {
     int64_t sort_tiles_max = 0;
     int64_t level_tiles_max = 0;
     size_t real_size = 4;
+    void *arena = nullptr;             // one allocation for the arrays that live as long as the workspace
 
     // sort
     uint64_t *key = nullptr, *key_alt = nullptr;
