@@ -446,12 +446,14 @@ __device__ __forceinline__ void part_pc(const Stage<Real> &S, const Targets<Real
     }
 }
 
-// Resident blocks per SM the registers are held to.  kWalkFold keeps two
+// Resident blocks per SM the registers are held to.  FP32: 5 (96 registers, no
+// spills): galaxy of 1e7 41.8 ms against 42.0 at 6 blocks (80) and 42.4 at 4,
+// Plummer 2^20 at theta = 0.5 7.25 against 7.33 and 7.27.  kWalkFold keeps two
 // batches of partial sums in registers (the fold of the longest group is a
 // chain of loads: 65 us at N = 16384 with one batch that spilled, 20 with two
 // that fit) and runs few groups: 3 blocks.
 constexpr int walk_blocks(int mode, int tpl, size_t real) {
-    return mode == kWalkFold ? 3 : tpl == 2 ? 4 : real == 4 ? 6 : 5;
+    return mode == kWalkFold ? 3 : tpl == 2 ? 4 : 5;
 }
 
 template <typename Real, int TPL, bool QUAD, bool KAHAN, bool SOFT, int MODE>
