@@ -85,10 +85,10 @@ void free_all(TreeWorkspace *ws) {
     ws->copy_stream = nullptr;
     ws->ev_drift = ws->ev_xback = nullptr;
     if (ws->side_stream) cudaStreamDestroy(ws->side_stream);
-    if (ws->ev_fork) cudaEventDestroy(ws->ev_fork);
-    if (ws->ev_join) cudaEventDestroy(ws->ev_join);
+    for (cudaEvent_t e : {ws->ev_sort, ws->ev_gather, ws->ev_fork, ws->ev_join})
+        if (e) cudaEventDestroy(e);
     ws->side_stream = nullptr;
-    ws->ev_fork = ws->ev_join = nullptr;
+    ws->ev_sort = ws->ev_gather = ws->ev_fork = ws->ev_join = nullptr;
     ws->graph_exec = nullptr;
     ws->graph = nullptr;
     ws->cap_stream = nullptr;
@@ -499,29 +499,23 @@ static cudaError_t clear_build(TreeWorkspace *ws, int64_t n, cudaStream_t s) {
     return e;
 }
 
-// Keys, sort and octree of positions whose box (or its partials) is known.
-static tree_status_t sort_and_octree(TreeWorkspace *ws, const void *x, int64_t n, cudaStream_t s) {
+// Keys and sort of positions whose box (or its partials) is known.
+static tree_status_t keys_and_sort(TreeWorkspace *ws, const void *x, int64_t n, cudaStream_t s) {
     {
         PhaseScope ph(ws, TREE_PHASE_KEYS, s);
         TRY_CUDA(launch_keys(ws, x, n, s));
     }
-    {
-        PhaseScope ph(ws, TREE_PHASE_SORT, s);
-        TRY_CUDA(launch_sort(ws, n, s));
-    }
-    PhaseScope ph(ws, TREE_PHASE_OCTREE, s);
-    TRY_CUDA(launch_octree(ws, n, s));
+    PhaseScope ph(ws, TREE_PHASE_SORT, s);
+    TRY_CUDA(launch_sort(ws, n, s));
     return TREE_OK;
 }
 
-// Everything of a build but the walk groups.
-static tree_status_t build_octree(TreeWorkspace *ws, const void *x, int64_t n, cudaStream_t s) {
+// The start of a build, up to the box.
+static tree_status_t build_begin(TreeWorkspace *ws, const void *x, int64_t n, cudaStream_t s) {
     TRY_CUDA(clear_build(ws, n, s));
-    {
-        PhaseScope ph(ws, TREE_PHASE_BOX, s);
-        TRY_CUDA(launch_box(ws, x, n, s));
-    }
-    return sort_and_octree(ws, x, n, s);
+    PhaseScope ph(ws, TREE_PHASE_BOX, s);
+    TRY_CUDA(launch_box(ws, x, n, s));
+    return TREE_OK;
 }
 
 tree_status_t tree_build(TreeWorkspace *ws, const void *x, int64_t n, int32_t dtype, void *stream) {
@@ -536,9 +530,11 @@ tree_status_t tree_build(TreeWorkspace *ws, const void *x, int64_t n, int32_t dt
     ws->has_moments = false;
     ws->list_groups = -1;
     if (n == 0) { ws->built = true; return TREE_OK; }
-    tree_status_t st = build_octree(ws, x, n, s);
+    tree_status_t st = build_begin(ws, x, n, s);
+    if (st == TREE_OK) st = keys_and_sort(ws, x, n, s);
     if (st != TREE_OK) return st;
     PhaseScope ph(ws, TREE_PHASE_OCTREE, s);
+    TRY_CUDA(launch_octree(ws, n, s));
     TRY_CUDA(launch_groups(ws, n, s));
     ws->built = true;
     return TREE_OK;
@@ -687,8 +683,8 @@ tree_status_t tree_energy_vjp(TreeWorkspace *ws, const void *m, const void *phi,
 // onto (created outside any stream capture).
 static tree_status_t ensure_side_stream(TreeWorkspace *ws) {
     if (!ws->side_stream) TRY_CUDA(cudaStreamCreateWithFlags(&ws->side_stream, cudaStreamNonBlocking));
-    if (!ws->ev_fork) TRY_CUDA(cudaEventCreateWithFlags(&ws->ev_fork, cudaEventDisableTiming));
-    if (!ws->ev_join) TRY_CUDA(cudaEventCreateWithFlags(&ws->ev_join, cudaEventDisableTiming));
+    for (cudaEvent_t *e : {&ws->ev_sort, &ws->ev_gather, &ws->ev_fork, &ws->ev_join})
+        if (!*e) TRY_CUDA(cudaEventCreateWithFlags(e, cudaEventDisableTiming));
     return TREE_OK;
 }
 
@@ -700,46 +696,60 @@ static cudaError_t launch_groups_timed(TreeWorkspace *ws, int64_t n, cudaStream_
     return e;
 }
 
-// From the octree to the forces: walk groups, gather, moments and walk.  x and
-// m: the caller's arrays, or NULL to gather from the packed copy of the
-// kick-drift pass.
+// From the box to the forces: keys, sort, octree, walk groups, gather, moments
+// and walk.  gx and gm: the caller's arrays to gather from, or NULL to gather
+// from the packed copy of the kick-drift pass.
 //
-// The walk groups need the octree only, and the gather and the moments do not
-// need the groups, so one of the two runs on the side stream beside the other
-// and is joined before whatever needs both.  A split walk's traversal reads
-// cells and groups but neither particles nor moments: there the gather and the
-// moments (FP64 latency) go aside and the groups and the traversal (dependent
-// loads) go on, up to the evaluation of the tiles (force at N = 1031 186 ->
-// 152 us, step at 30011 453 -> 369).  Otherwise the groups go aside.  The phase events of what
-// runs aside are on the side stream.
-static tree_status_t finish_forces(TreeWorkspace *ws, const void *x, const void *m, const WalkOut &out, int64_t n,
-                                   cudaStream_t s) {
+// The gather needs the sort only and runs on the side stream beside the
+// octree.  The walk groups need the octree only, and the gather and the
+// moments do not need the groups, so one of the two runs on the side stream
+// beside the other and is joined before whatever needs both.  A split walk's
+// traversal reads cells and groups but neither particles nor moments: there
+// the moments (FP64 latency) go aside and the groups and the traversal
+// (dependent loads) go on, up to the evaluation of the tiles (force at N =
+// 1031 186 -> 152 us, step at 30011 453 -> 369).  Otherwise the groups go
+// aside.  The phase events of what runs aside are on the side stream.
+static tree_status_t forces_from_box(TreeWorkspace *ws, const void *x, const void *gx, const void *gm,
+                                     const WalkOut &out, int64_t n, cudaStream_t s) {
     tree_status_t st = upload_mac(ws, s);
+    if (st == TREE_OK) st = ensure_side_stream(ws);
+    if (st == TREE_OK) st = keys_and_sort(ws, x, n, s);
     if (st != TREE_OK) return st;
-    st = ensure_side_stream(ws);
-    if (st != TREE_OK) return st;
-    const bool split = walk_splits(ws);
-    const cudaStream_t side = ws->side_stream, sg = split ? s : side, sm = split ? side : s;
+    const cudaStream_t side = ws->side_stream;
+    TRY_CUDA(cudaEventRecord(ws->ev_sort, s));
+    TRY_CUDA(cudaStreamWaitEvent(side, ws->ev_sort, 0));
+    {
+        PhaseScope ph(ws, TREE_PHASE_GATHER, side);
+        TRY_CUDA(gx ? launch_gather(ws, gx, gm, n, side) : launch_gather_packed(ws, n, side));
+    }
+    TRY_CUDA(cudaEventRecord(ws->ev_gather, side));
+    {
+        PhaseScope ph(ws, TREE_PHASE_OCTREE, s);
+        TRY_CUDA(launch_octree(ws, n, s));
+    }
     TRY_CUDA(cudaEventRecord(ws->ev_fork, s));
     TRY_CUDA(cudaStreamWaitEvent(side, ws->ev_fork, 0));
-    if (!split) TRY_CUDA(launch_groups_timed(ws, n, sg));
-    {
-        PhaseScope ph(ws, TREE_PHASE_GATHER, sm);
-        TRY_CUDA(x ? launch_gather(ws, x, m, n, sm) : launch_gather_packed(ws, n, sm));
-    }
-    {
-        PhaseScope ph(ws, TREE_PHASE_MOMENTS, sm);
-        TRY_CUDA(launch_moments(ws, sm));
-    }
-    TRY_CUDA(cudaEventRecord(ws->ev_join, side));
+    const bool split = walk_splits(ws);
     if (split) {
-        TRY_CUDA(launch_groups_timed(ws, n, sg));
+        {
+            PhaseScope ph(ws, TREE_PHASE_MOMENTS, side);
+            TRY_CUDA(launch_moments(ws, side));
+        }
+        TRY_CUDA(cudaEventRecord(ws->ev_join, side));
+        TRY_CUDA(launch_groups_timed(ws, n, s));
         PhaseScope ph(ws, TREE_PHASE_WALK, s);
         TRY_CUDA(launch_walk_split(ws, kWalkTiles, out, s));
         TRY_CUDA(cudaStreamWaitEvent(s, ws->ev_join, 0));
         ws->built = ws->has_moments = true;
         TRY_CUDA(launch_walk_split(ws, kWalkFold, out, s));
         return TREE_OK;
+    }
+    TRY_CUDA(launch_groups_timed(ws, n, side));
+    TRY_CUDA(cudaEventRecord(ws->ev_join, side));
+    TRY_CUDA(cudaStreamWaitEvent(s, ws->ev_gather, 0));
+    {
+        PhaseScope ph(ws, TREE_PHASE_MOMENTS, s);
+        TRY_CUDA(launch_moments(ws, s));
     }
     TRY_CUDA(cudaStreamWaitEvent(s, ws->ev_join, 0));
     ws->built = ws->has_moments = true;
@@ -757,9 +767,9 @@ tree_status_t tree_accel(TreeWorkspace *ws, const void *x, const void *m, int64_
     ws->built = ws->has_moments = n == 0;
     ws->list_groups = -1;
     if (n == 0) return TREE_OK;
-    st = build_octree(ws, x, n, s);
+    st = build_begin(ws, x, n, s);
     if (st != TREE_OK) return st;
-    return finish_forces(ws, x, m, WalkOut{a, phi, nullptr, 0.0}, n, s);
+    return forces_from_box(ws, x, x, m, WalkOut{a, phi, nullptr, 0.0}, n, s);
 }
 
 // First part of a step: the first kick and the drift (Eqs. 2-3), fused with
@@ -782,12 +792,10 @@ static tree_status_t leapfrog_begin(TreeWorkspace *ws, void *x, void *v, const v
 static tree_status_t leapfrog_finish(TreeWorkspace *ws, const void *x, void *v, void *a, void *phi, double tau,
                                      int64_t n, cudaStream_t s, void *v_mirror = nullptr,
                                      void *phi_mirror = nullptr) {
-    tree_status_t st = sort_and_octree(ws, x, n, s);
-    if (st != TREE_OK) return st;
     WalkOut out{a, phi, v, 0.5 * tau};
     out.v_mirror = v_mirror;
     out.phi_mirror = phi_mirror;
-    return finish_forces(ws, nullptr, nullptr, out, n, s);
+    return forces_from_box(ws, x, nullptr, nullptr, out, n, s);
 }
 
 tree_status_t leapfrog_step(TreeWorkspace *ws, void *x, void *v, const void *m, void *a, void *phi, double tau,

@@ -164,8 +164,8 @@ struct TreeWorkspace {
     double *hs_diag = nullptr;
     cudaStream_t copy_stream = nullptr;  // copies back that overlap the rest of the step
     cudaEvent_t ev_drift = nullptr, ev_xback = nullptr;
-    cudaStream_t side_stream = nullptr;  // part of a force evaluation beside the rest (finish_forces)
-    cudaEvent_t ev_fork = nullptr, ev_join = nullptr;
+    cudaStream_t side_stream = nullptr;  // part of a force evaluation beside the rest (forces_from_box)
+    cudaEvent_t ev_sort = nullptr, ev_gather = nullptr, ev_fork = nullptr, ev_join = nullptr;
     // one captured leapfrog step (leapfrog_graph_capture)
     cudaStream_t cap_stream = nullptr;
     cudaGraph_t graph = nullptr;
