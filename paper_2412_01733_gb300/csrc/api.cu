@@ -273,8 +273,10 @@ tree_status_t tree_workspace_create(int64_t n_max, const TreeParams *p, TreeWork
     const size_t v2 = p->precision == TREE_F64 ? sizeof(double2a) : sizeof(float2);
     // tile slots of the split walk (groups of 64 use half of them: two targets per lane)
     size_t T = 0;
-    if (n_max > 0 && n_max <= (p->precision == TREE_F64 ? kSplitMaxN64 : kSplitMaxN32))
-        T = (((size_t)n_max * kTilesPer + 4096) / kTileChunk) * kTileChunk;
+    if (n_max > 0 && n_max <= (p->precision == TREE_F64 ? kSplitMaxN64 : kSplitMaxN32)) {
+        const double need = split_slots(n_max, p->theta, p->group_size) * 1.2 + 4096.0;
+        if (need <= (double)n_max * kTilesPer + 4096.0) T = ((size_t)need / kTileChunk) * kTileChunk;
+    }
     auto lay_out = [&](Arena &A) {
         const size_t G = (size_t)ws->groups_max;
         // these four start at zero
@@ -327,12 +329,20 @@ tree_status_t tree_workspace_create(int64_t n_max, const TreeParams *p, TreeWork
         return zeroed;
     };
     Arena A;
-    const size_t zeroed = lay_out(A);
+    size_t zeroed = lay_out(A);
+    bool ok = dalloc((unsigned char **)&ws->arena, A.size);
+    if (!ok && T > 0) {  // a full device does without the split walk
+        cudaGetLastError();
+        T = 0;
+        A = Arena{};
+        zeroed = lay_out(A);
+        ok = dalloc((unsigned char **)&ws->arena, A.size);
+    }
     // the arrays that tree_set_segments may replace are allocations of their own
-    const bool ok = dalloc((unsigned char **)&ws->arena, A.size) && dalloc(&ws->box, 1) &&
-                    dalloc(&ws->ccount, (size_t)chunks_max) && dalloc(&ws->coff, (size_t)chunks_max) &&
-                    dalloc(&ws->cmask, 2 * (size_t)chunks_max) &&
-                    dalloc(&ws->gscan_status, (size_t)(chunks_max / 2048 + 2));
+    ok = ok && dalloc(&ws->box, 1) &&
+         dalloc(&ws->ccount, (size_t)chunks_max) && dalloc(&ws->coff, (size_t)chunks_max) &&
+         dalloc(&ws->cmask, 2 * (size_t)chunks_max) &&
+         dalloc(&ws->gscan_status, (size_t)(chunks_max / 2048 + 2));
     if (ok) {
         A = Arena{static_cast<unsigned char *>(ws->arena), 0};
         lay_out(A);

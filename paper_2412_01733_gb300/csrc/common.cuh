@@ -38,9 +38,10 @@ constexpr int64_t kMaxNodes = (int64_t)1 << 29;  // node indices fit 29 bits (wa
 constexpr int64_t kWalkOrderMaxN = (int64_t)1 << 22;
 
 // Split walk (walk.cuh): workspaces of at most this many particles (FP32,
-// FP64; the measured lines are in walk.cuh) keep tile slots for it, kTilesPer
-// for each particle, handed out kTileChunk at a time.  12 a particle serve
-// theta >= 0.45 at N = 131072 (660 B a slot in FP32).
+// FP64; the measured lines are in walk.cuh) keep the tile slots that their
+// parameters are expected to need (split_slots), unless that is more than
+// kTilesPer for each particle (theta below 0.45 at N = 131072; 660 B a slot in
+// FP32).  Slots are handed out kTileChunk at a time.
 constexpr int64_t kSplitMaxN32 = (int64_t)1 << 17, kSplitMaxN64 = (int64_t)1 << 17;
 constexpr int kTilesPer = 12;
 constexpr int kTileChunk = 16;
@@ -240,19 +241,23 @@ struct TreeWorkspace {
 
 namespace treegb {
 
-// Whether the force walk is split: the workspace keeps tile slots, and the
-// lists are expected to fit them.  A particle meets about 95 log2(n) / theta^2
-// sources (Plummer spheres and the galaxy, within a tenth), at most n; groups
-// hold 28 or more on average, and a chunk's unused slots come to about one per
-// particle.  Lists that do not fit after all are walked by one warp as ever,
-// but only after the traversal has been tried in vain, hence the line.
-inline bool walk_splits(const TreeWorkspace *ws) {
-    if (ws->tile_cap == 0) return false;
-    const double n = (double)ws->n, th = ws->p.theta;
+// Tile slots that a split walk is expected to take.  A particle meets about 95
+// log2(n) / theta^2 sources (Plummer spheres and the galaxy, within a tenth),
+// at most n; groups hold 28 or more on average (groups of 64 put two targets
+// to a lane of a slot twice the size), and a chunk's unused slots come to
+// about one per particle.
+inline double split_slots(int64_t particles, double theta, int group_size) {
+    const double n = (double)particles;
     double src = n;
-    if (th > 0.0 && 95.0 * log2(n + 2.0) / (th * th) < n) src = 95.0 * log2(n + 2.0) / (th * th);
-    const double lanes = ws->p.group_size == 16 ? 14.0 : 28.0;  // groups of 64 share a slot two targets to a lane
-    return n * (src / (32.0 * lanes) + 1.0) <= 0.9 * (double)ws->tile_cap;
+    if (theta > 0.0 && 95.0 * log2(n + 2.0) / (theta * theta) < n) src = 95.0 * log2(n + 2.0) / (theta * theta);
+    return n * (src / (32.0 * (group_size == 16 ? 14.0 : 28.0)) + 1.0);
+}
+// Whether the force walk is split: the workspace keeps tile slots, and the
+// lists are expected to fit them.  Lists that do not fit after all are walked
+// by one warp as ever, but only after the traversal has been tried in vain,
+// hence the line.
+inline bool walk_splits(const TreeWorkspace *ws) {
+    return ws->tile_cap > 0 && split_slots(ws->n, ws->p.theta, ws->p.group_size) <= 0.9 * (double)ws->tile_cap;
 }
 inline bool walk_widest_first(const TreeWorkspace *ws) { return ws->n < kWalkOrderMaxN; }
 

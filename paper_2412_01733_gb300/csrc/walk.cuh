@@ -15,8 +15,8 @@
 // moments then beside the traversal): FP32 N = 16384 455 -> 221 us, 65536 742
 // -> 528, 131072 987 -> 917, but 262144 1585 -> 1649 (1.25 KB of slot traffic
 // per tile, and the traversal no longer hides behind the arithmetic); FP64
-// walk alone N = 16384 12.8 -> 2.7 ms, 65536 21.6 -> 13.1, 131072 32.6 ->
-// 28.7.  walk_splits() draws the lines there.
+// walk alone, full far-cell form, N = 16384 12.8 -> 2.7 ms, 65536 21.6 ->
+// 13.1, 131072 32.6 -> 28.7.  walk_splits() draws the lines there.
 //
 // Traversal (per warp, depth first, stack in shared memory):
 //   the stack holds ranges of sibling nodes (children are contiguous in the
