@@ -208,18 +208,24 @@ __global__ void __launch_bounds__(kAdjWarps * 32, 4) k_force_vjp(const AdjArgs A
     }
     __syncwarp();
     double xt[2][3] = {{0, 0, 0}, {0, 0, 0}};
-    const Real px0 = spos[s0].x, py0 = spos[s0].y, pz0 = spos[s0].z;
 
     // All pairs of the lanes' sources with the group's targets: the source-side
     // sums stay in the lane, the targets' partial sums travel with them (one
-    // shuffle per step passes each on to the lane that meets it next).
+    // shuffle per step passes each on to the lane that meets it next).  Lanes
+    // without a source and places without a target take part with zero weights,
+    // at the position of the tile's first source and of the group's first
+    // particle: pairs that are there anyway, so a stand-in's powers of 1/r are
+    // finite (and its terms zero) wherever theirs are.  At a distance of their
+    // own they might not be: at r = 3e-6 a cell's 5/r^7 is past the FP32 range,
+    // and 0 times it a NaN.  The self pair, which nothing else meets, is left
+    // out for stand-ins too.
     auto meet = [&](const AdjSource<Real> &S, auto quad, bool own, uint32_t sj, V(&acc)[11]) {
 #pragma unroll
         for (int h = 0; h < 2; ++h) {
             if (h >= halves) break;
             V t[3] = {P::dup(Real(0)), P::dup(Real(0)), P::dup(Real(0))};
             const V(*st)[L] = s_t[w][h];
-            const uint32_t first = s0 + 32u * (uint32_t)h;
+            auto target = [&](int j) { return s0 + (uint32_t)(32 * h + j < cnt ? 32 * h + j : 0); };
 #pragma unroll W
             for (int k = 0; k < L; ++k) {
                 if (k > 0) {
@@ -228,8 +234,8 @@ __global__ void __launch_bounds__(kAdjWarps * 32, 4) k_force_vjp(const AdjArgs A
                 }
                 const int j = (lane + k) & (L - 1);
                 pair_vjp<Real, decltype(quad)::value, SOFT>(S, st[0][j], st[1][j], st[2][j], st[3][j], st[4][j],
-                                                            st[5][j], st[6][j], eps2, own, first + j == sj,
-                                                            first + j + L == sj, acc, t);
+                                                            st[5][j], st[6][j], eps2, own, target(j) == sj,
+                                                            target(j + L) == sj, acc, t);
             }
 #pragma unroll
             for (int c = 0; c < 3; ++c) {
@@ -249,22 +255,18 @@ __global__ void __launch_bounds__(kAdjWarps * 32, 4) k_force_vjp(const AdjArgs A
     const int64_t pc0 = A.list_off[g], pc1 = A.list_off[g + 1];
     for (int64_t base = pc0 + 32 * part; base < pc1; base += 32 * A.parts) {
         const int nt = (int)min((int64_t)32, pc1 - base);
-        uint32_t cid = 0;
+        const uint32_t cid = (uint32_t)A.pc_list[base + (lane < nt ? lane : 0)];
+        const V4 a = momA[cid];
         AdjSource<Real> S;
-        S.x = P::dup(px0); S.y = P::dup(py0); S.z = P::dup(pz0); S.nm = P::dup(Real(0));
+        S.x = P::dup(a.x); S.y = P::dup(a.y); S.z = P::dup(a.z); S.nm = P::dup(lane < nt ? -a.w : Real(0));
 #pragma unroll
         for (int q = 0; q < 6; ++q) S.q[q] = P::dup(Real(0));
-        if (lane < nt) {
-            cid = (uint32_t)A.pc_list[base + lane];
-            const V4 a = momA[cid];
-            S.x = P::dup(a.x); S.y = P::dup(a.y); S.z = P::dup(a.z); S.nm = P::dup(-a.w);
-            if (QUAD) {
-                const V4 b = momB[cid];
-                const V2 c = momC[cid];
-                const Real qs = sizeof(Real) == 4 ? Real(1) : Real(-1);  // the FP32 walk copies hold -Q
-                S.q[0] = P::dup(qs * b.x); S.q[1] = P::dup(qs * b.y); S.q[2] = P::dup(qs * b.z);
-                S.q[3] = P::dup(qs * b.w); S.q[4] = P::dup(qs * c.x); S.q[5] = P::dup(qs * c.y);
-            }
+        if (QUAD && lane < nt) {
+            const V4 b = momB[cid];
+            const V2 c = momC[cid];
+            const Real qs = sizeof(Real) == 4 ? Real(1) : Real(-1);  // the FP32 walk copies hold -Q
+            S.q[0] = P::dup(qs * b.x); S.q[1] = P::dup(qs * b.y); S.q[2] = P::dup(qs * b.z);
+            S.q[3] = P::dup(qs * b.w); S.q[4] = P::dup(qs * c.x); S.q[5] = P::dup(qs * c.y);
         }
         // the group's (at most 64) targets are summed in the working precision;
         // the per-group totals go to the FP64 accumulators (G comes with the scatter)
@@ -286,18 +288,17 @@ __global__ void __launch_bounds__(kAdjWarps * 32, 4) k_force_vjp(const AdjArgs A
     // ---- near leaves: expand particles into the buffer, tiles of 32 ----
     const int64_t pp0 = A.list_off[A.ngroups + 1 + g], pp1 = A.list_off[A.ngroups + 1 + g + 1];
     auto pp_tile = [&](uint32_t sj, int nt) {
+        const uint32_t s1 = __shfl_sync(0xffffffffu, sj, 0);
+        if (lane >= nt) sj = s1;
+        const V4 a = spos[sj];
         AdjSource<Real> S;
-        S.x = P::dup(px0); S.y = P::dup(py0); S.z = P::dup(pz0); S.nm = P::dup(Real(0));
-        if (lane < nt) {
-            const V4 a = spos[sj];
-            S.x = P::dup(a.x); S.y = P::dup(a.y); S.z = P::dup(a.z); S.nm = P::dup(-a.w);
-        }
-        const bool own = __any_sync(0xffffffffu, lane < nt && sj - s0 < (uint32_t)cnt);
+        S.x = P::dup(a.x); S.y = P::dup(a.y); S.z = P::dup(a.z); S.nm = P::dup(lane < nt ? -a.w : Real(0));
+        const bool own = __any_sync(0xffffffffu, sj - s0 < (uint32_t)cnt);
         V acc[11];
 #pragma unroll
         for (int q = 0; q < 5; ++q) acc[q] = P::dup(Real(0));
         // the self pair is excluded by index
-        if (own) meet(S, std::false_type{}, true, lane < nt ? sj : 0xffffffffu, acc);
+        if (own) meet(S, std::false_type{}, true, sj, acc);
         else meet(S, std::false_type{}, false, 0u, acc);
         if (lane < nt) {
             atomicAdd(A.xg + sj, (double)P::total(acc[2]));
