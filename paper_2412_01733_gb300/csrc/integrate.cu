@@ -236,9 +236,11 @@ __device__ __forceinline__ void direct_term(float px, float py, float pz, float4
 // Bound by the FMA pipe: 8192 targets of 2^20 particles 7.29 -> 4.13 ms
 // (2.1e12 pairs/s; one pair at a time, with two branches each, 1.2e12).  SOFT: eps^2 is a normal FP32 number (rsqrt_pair);
 // otherwise a pair at r^2 = 0 contributes nothing.  In tiles that hold one of
-// the block's targets, a target's own mass counts as zero; tiles with a
-// coordinate that is not finite go through direct_term itself, which skips
-// pairs whose r^2 is a NaN.
+// the block's targets, a target's own mass counts as zero; without SOFT its 1/r
+// to itself does, because r^-2 = eps^-2 may be past the FP32 range there (eps
+// below 5.4e-20; the mass is off the chain of the terms: 4.13 ms against 4.24);
+// tiles with a coordinate or mass that is not finite go through
+// direct_term itself, which skips pairs whose r^2 is zero or a NaN.
 template <bool SOFT, int P>
 __global__ void __launch_bounds__(kDirThreads) k_direct_f32(const float *__restrict__ x, const float *__restrict__ m,
                                                             int64_t n, int64_t jbeg, int64_t jend,
@@ -272,7 +274,7 @@ __global__ void __launch_bounds__(kDirThreads) k_direct_f32(const float *__restr
         const int ns = (int)min((int64_t)kDirThreads, j1 - jb);
         float4 q = make_float4(0.f, 0.f, 0.f, 0.f);
         if (j < j1) q = make_float4(x[j], x[n + j], x[2 * n + j], m[j]);
-        int kind = odd || !(isfinite(q.x) && isfinite(q.y) && isfinite(q.z)) ? 2 : 0;
+        int kind = odd || !(isfinite(q.x) && isfinite(q.y) && isfinite(q.z) && isfinite(q.w)) ? 2 : 0;
         int me[T];  // the target's own place in this tile
 #pragma unroll
         for (int i = 0; i < T; ++i) {
@@ -299,11 +301,11 @@ __global__ void __launch_bounds__(kDirThreads) k_direct_f32(const float *__restr
                     const float2 dz = __fadd2_rn(make_float2(b.x, b.y), nz[i]);
                     const float2 r2 =
                         __fadd2_rn(__ffma2_rn(dz, dz, __ffma2_rn(dx, dx, __fmul2_rn(dy, dy))), eps2v);
-                    const float2 ri = rsqrt_pair<SOFT>(r2);
+                    float2 ri = rsqrt_pair<SOFT>(r2);
                     float2 mk = make_float2(b.z, b.w);
                     if (skip) {
-                        if (k == me[2 * i]) mk.x = 0.f;
-                        if (k == me[2 * i + 1]) mk.y = 0.f;
+                        if (k == me[2 * i]) (SOFT ? mk : ri).x = 0.f;
+                        if (k == me[2 * i + 1]) (SOFT ? mk : ri).y = 0.f;
                     }
                     const float2 mr = __fmul2_rn(mk, ri);
                     const float2 w = __fmul2_rn(mr, __fmul2_rn(ri, ri));
