@@ -556,6 +556,7 @@ __global__ void __launch_bounds__(256) k_group_key(const uint64_t *__restrict__ 
                                                    const uint32_t *__restrict__ ctr, uint32_t *__restrict__ gkey,
                                                    uint32_t *bucket) {
     __shared__ uint32_t h[32];
+    if (aborted(ctr, kStageAfter)) return;  // (a group count whose gfirst has not been written)
     if (threadIdx.x < 32) h[threadIdx.x] = 0;
     __syncthreads();
     const uint32_t ng = ctr[kCtrGroups];
@@ -589,6 +590,7 @@ __global__ void k_group_scan(uint32_t *bucket) {
 
 __global__ void __launch_bounds__(256) k_group_scatter(const uint32_t *__restrict__ gkey, const uint32_t *__restrict__ ctr,
                                                        uint32_t *bucket, uint32_t *__restrict__ order) {
+    if (aborted(ctr, kStageAfter)) return;
     const uint32_t ng = ctr[kCtrGroups];
     const int lane = threadIdx.x & 31;
     // warp-uniform trip count, one atomic per distinct key in a warp
@@ -656,7 +658,7 @@ cudaError_t noalloc_scratch(double **out) {
 __global__ void __launch_bounds__(256) k_gstat_reduce(const uint4 *__restrict__ gstat, const uint32_t *__restrict__ gfirst,
                                                       const uint32_t *__restrict__ ctr, unsigned long long *stats) {
     unsigned long long pp = 0, pc = 0, ms = 0;
-    const uint32_t ng = ctr[kCtrGroups];
+    const uint32_t ng = aborted(ctr, kStageAfter) ? 0u : ctr[kCtrGroups];
     for (uint32_t g = blockIdx.x * blockDim.x + threadIdx.x; g < ng; g += gridDim.x * blockDim.x) {
         const uint4 r = gstat[g];
         const unsigned long long c = (unsigned long long)(gfirst[g + 1] - gfirst[g]);
@@ -678,14 +680,15 @@ __global__ void __launch_bounds__(256) k_gstat_reduce(const uint4 *__restrict__ 
 }
 
 // Exclusive scans of the per-group list lengths (x: PC cells, w: PP leaves)
-// into list_off[0..ng] and list_off[ng+1 .. 2ng+1]; sizes: ng and both totals.  Single block: the list
+// into list_off[0..ng] and list_off[ng+1 .. 2ng+1]; sizes: ng and both totals.  (After a given-up wait the
+// list lengths have not been written: no groups, empty lists.)  Single block: the list
 // path is a test/adjoint path, not the force hot path.
 __global__ void __launch_bounds__(1024) k_list_scan(const uint4 *__restrict__ gstat, const uint32_t *__restrict__ ctr,
                                                     int64_t *__restrict__ off, int64_t *__restrict__ sizes) {
     __shared__ unsigned long long wt[2][32];
     __shared__ unsigned long long carry[2];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const int64_t ng = ctr[kCtrGroups];
+    const int64_t ng = aborted(ctr, kStageAfter) ? 0 : ctr[kCtrGroups];
     if (tid < 2) carry[tid] = 0;
     __syncthreads();
     for (int64_t b = 0; b < ng; b += 1024) {

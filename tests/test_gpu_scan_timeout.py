@@ -1,0 +1,64 @@
+"""Builds whose group scan gives up a wait: nothing reads the walk groups that were not written, and nothing stays
+behind for the next build.
+
+With 65536 particles in groups of 16 the scan has two tiles and no other kernel of the build waits, so under a limit of
+one clock cycle it is the scan that gives up, whenever its second tile looks before the first has published: alone that
+never happens, beside another system's steps it does in one build of some dozens.  Afterwards, with the limit
+restored, the workspace must give the bits of an undisturbed one.
+"""
+import pytest
+import torch
+
+from paper_2412_01733_gb300 import inputs
+
+pytestmark = pytest.mark.gpu
+
+N = 65536
+
+
+def _disturbed(ws, work):
+    """Runs work() many times under a limit of one cycle beside other work; the status bits seen."""
+    from paper_2412_01733_gb300 import treegb as tg
+    y, _, k = (t.to("cuda", torch.float32).contiguous() for t in inputs.plummer(1 << 20, 13))
+    side, seen, hits = torch.cuda.Stream(), 0, 0
+    ws.set_waits(wait_cycles=1)
+    with tg.Workspace(1 << 20) as other:
+        for _ in range(40):
+            side.wait_stream(torch.cuda.current_stream())
+            with torch.cuda.stream(side):
+                for _ in range(5):
+                    other.accel(y, k)
+            for _ in range(40):
+                work()
+            st = ws.status(clear=True)
+            seen |= st
+            hits += st != 0
+            if hits == 4:
+                break
+        assert other.status() == 0
+    ws.set_waits(wait_cycles=2_000_000_000)
+    assert seen in (0, tg.DEV_TIMEOUT)
+    return seen
+
+
+@pytest.mark.parametrize("theta", [0.3, 0.7])  # 0.3: the one-warp walk, which orders the groups first
+def test_lists_and_gradients_of_builds_without_groups(theta):
+    from paper_2412_01733_gb300 import treegb as tg
+    x, _, m = (t.to("cuda", torch.float32).contiguous() for t in inputs.plummer(N, 12))
+    a, f = torch.empty_like(x), torch.empty_like(m)
+    p = dict(group_size=16, theta=theta)
+    with tg.Workspace(N, **p) as ws, tg.Workspace(N, **p) as ref:
+        def work():
+            ws.build(x); ws.moments(x, m)
+            ws.forces(a, f, emit_lists=True)
+            ws.forces_adjoint(x, m)
+
+        seen = _disturbed(ws, work)
+        for w in (ws, ref):
+            w.build(x); w.moments(x, m)
+        got, want = (w.forces(emit_lists=True) for w in (ws, ref))
+        assert ws.status() == ref.status() == 0
+        assert all(torch.equal(s, t) for s, t in zip(got, want))
+        assert ws.info()["list_pc"] == ref.info()["list_pc"] > 0
+        if not seen:
+            pytest.skip("no wait ran out")
