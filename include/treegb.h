@@ -370,8 +370,10 @@ tree_status_t tree_direct_forces_noalloc(const void *x, const void *m, int64_t n
  * walk-group scan) gives up after a limit of clock cycles: it then sets
  * TREE_DEV_TIMEOUT, the rest of its own kernel writes only in bounds, and
  * every later kernel of that build, force or gradient call returns without
- * touching the tree -- the call's results are invalid, the context stays
- * usable and the next build starts clean.  wait_cycles > 0 sets the limit
+ * touching the tree (the gather and the moments, which run beside the group
+ * scan and do not need it, complete when that one gives up) -- the call's
+ * results are invalid, the context stays usable and the next build starts
+ * clean.  wait_cycles > 0 sets the limit
  * (default 2e9 cycles, about 1 s); 0 keeps it.  withhold_pass and
  * withhold_tile >= 0 make that tile of that sort pass (0..9) skip publishing
  * its look-back words, so the tiles after it run into the limit: a test of

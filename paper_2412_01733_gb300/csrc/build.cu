@@ -575,12 +575,14 @@ cudaError_t launch_octree(TreeWorkspace *ws, int64_t n, cudaStream_t s) {
 }
 
 // ============================================================== gather
+// (A given-up wait of the group scan, which may run meanwhile, does not stop
+// the gather: the moments that follow run on too, see moments.cu.)
 template <typename Real>
 __global__ void __launch_bounds__(256) k_gather(const Real *__restrict__ x, const Real *__restrict__ m,
                                                 const uint32_t *__restrict__ idx, int64_t n,
                                                 typename Vec4<Real>::T *__restrict__ spos,
                                                 const uint32_t *__restrict__ ctr) {
-    if (aborted(ctr, kStageAfter)) return;
+    if (aborted(ctr, kStageGroupScan)) return;
     for (int64_t s = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; s < n; s += (int64_t)gridDim.x * blockDim.x) {
         const uint32_t i = idx[s];
         typename Vec4<Real>::T p;
@@ -598,7 +600,7 @@ template <typename V4>
 __global__ void __launch_bounds__(256) k_gather_packed(const V4 *__restrict__ xm, const uint32_t *__restrict__ idx,
                                                        int64_t n, V4 *__restrict__ spos,
                                                        const uint32_t *__restrict__ ctr) {
-    if (aborted(ctr, kStageAfter)) return;
+    if (aborted(ctr, kStageGroupScan)) return;
     for (int64_t s = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; s < n; s += (int64_t)gridDim.x * blockDim.x)
         spos[s] = xm[idx[s]];
 }

@@ -103,7 +103,9 @@ enum CounterSlots {
 // Stages that wait on other blocks (decoupled look-backs).  When a wait of
 // stage S gives up, S is recorded in the counter block; the rest of S still
 // writes only in bounds, and every later kernel of the build (any other stage)
-// returns at once, so no kernel consumes the inconsistent data.
+// returns at once, so no kernel consumes the inconsistent data.  (The gather
+// and the moments run beside the group scan and consume nothing of it: they
+// complete when it gives up, see moments.cu.)
 constexpr uint32_t kStageSort0 = 1;        // sort pass p: 1 + p
 constexpr uint32_t kStageLevel0 = 16;      // octree level L: 16 + L
 constexpr uint32_t kStageGroupScan = 48;   // walk-group count scan

@@ -21,6 +21,14 @@
 // level, finest first).  A warp then mostly holds cells with equal trip
 // counts.  The order inside a bucket is arbitrary; every cell's arithmetic
 // is its own, so the results do not depend on it.
+//
+// Given-up waits.  The walk groups are made beside the moments, which do not
+// need them, so a wait of the group scan may give up while these kernels run.
+// They run on then (aborted(ctr, kStageGroupScan)): returning half-way would
+// leave arrival counters behind that the next build's climb starts from, and
+// slots of `order` unwritten.  The waits of the sort and the octree are over
+// before the moments start; after one of those gave up, none of these kernels
+// does anything.
 #include "common.cuh"
 
 namespace treegb {
@@ -35,8 +43,8 @@ __device__ __forceinline__ uint32_t mom_bucket(uint4 g, uint2 l) {
 // Bucket counts of all nodes.
 __global__ void __launch_bounds__(256) k_mom_hist(const uint32_t *__restrict__ ctr, const uint4 *__restrict__ ngeo,
                                                   const uint2 *__restrict__ nlink, uint32_t *__restrict__ cnt) {
-    // after a given-up wait the buckets stay empty, so no later moment kernel does any work
-    if (aborted(ctr, kStageAfter)) return;
+    // after a given-up wait of the sort or the octree the buckets stay empty, so no later moment kernel does any work
+    if (aborted(ctr, kStageGroupScan)) return;
     __shared__ uint32_t sh[kMomBuckets];
     for (int i = threadIdx.x; i < kMomBuckets; i += blockDim.x) sh[i] = 0;
     __syncthreads();
@@ -55,7 +63,7 @@ __global__ void __launch_bounds__(256) k_mom_scatter(const uint32_t *__restrict_
                                                      const uint2 *__restrict__ nlink, const uint32_t *__restrict__ cnt,
                                                      uint32_t *__restrict__ off, uint32_t *__restrict__ cursor,
                                                      uint32_t *__restrict__ order) {
-    if (aborted(ctr, kStageAfter)) return;
+    if (aborted(ctr, kStageGroupScan)) return;
     __shared__ uint32_t s_off[kMomBuckets + 1], s_cnt[kMomBuckets], s_base[kMomBuckets];
     for (int b = threadIdx.x; b < kMomBuckets; b += blockDim.x) s_cnt[b] = cnt[b];
     __syncthreads();
@@ -266,7 +274,7 @@ __global__ void __launch_bounds__(64) k_moments_climb(
     const uint32_t *__restrict__ nfirst, const int64_t *__restrict__ seg_off, int64_t nseg, double *mom64, int64_t cap,
     typename Vec4<Real>::T *__restrict__ mom_a, typename Vec4<Real>::T *__restrict__ mom_b,
     typename Vec2<Real>::T *__restrict__ mom_c) {
-    if (aborted(ctr, kStageAfter)) return;
+    if (aborted(ctr, kStageGroupScan)) return;
     const int lane = threadIdx.x & 31;
     const uint32_t end = BUCKETS ? off[kMomLeafBuckets] : ctr[kCtrLevelStart + kLevels];
     const uint32_t stride = gridDim.x * blockDim.x;
@@ -393,7 +401,7 @@ __global__ void __launch_bounds__(256) k_moments_level(
 template <typename V4, typename Real>
 __global__ void __launch_bounds__(256) k_r5_flags(const uint32_t *__restrict__ ctr, DevBox *box,
                                                   const V4 *__restrict__ mom_a, int64_t nseg) {
-    if (aborted(ctr, kStageAfter)) return;
+    if (aborted(ctr, kStageGroupScan)) return;
     for (int64_t b = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; b < nseg; b += (int64_t)gridDim.x * blockDim.x)
         box[b].r5fit = pc_r5_fits(box[b].k, (Real)mom_a[b].w) ? 1 : 0;
 }

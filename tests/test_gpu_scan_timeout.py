@@ -62,3 +62,20 @@ def test_lists_and_gradients_of_builds_without_groups(theta):
         assert ws.info()["list_pc"] == ref.info()["list_pc"] > 0
         if not seen:
             pytest.skip("no wait ran out")
+
+
+def test_moments_beside_a_scan_that_gives_up():
+    """accel runs the moments beside the scan; their arrival counters must come back to zero all the same."""
+    from paper_2412_01733_gb300 import treegb as tg
+    x, _, m = (t.to("cuda", torch.float32).contiguous() for t in inputs.plummer(N, 12))
+    a, f = torch.empty_like(x), torch.empty_like(m)
+    p = dict(group_size=16, theta=1.0)
+    with tg.Workspace(N, **p) as ws, tg.Workspace(N, **p) as ref:
+        want = ref.accel(x, m) + ref.export_moments()
+        seen = _disturbed(ws, lambda: ws.accel(x, m, a, f))
+        for _ in range(2):
+            got = ws.accel(x, m) + ws.export_moments()
+            assert ws.status() == ref.status() == 0
+            assert all(torch.equal(s, t) for s, t in zip(got, want))
+        if not seen:
+            pytest.skip("no wait ran out")
