@@ -302,7 +302,7 @@ tree_status_t tree_workspace_create(int64_t n_max, const TreeParams *p, TreeWork
         A.take(&ws->plev, N);
         A.take(&ws->pleaf, N);
         A.take(&ws->sdig, N);
-        A.take(&ws->flat_cnt, ((size_t)flat_octree_blocks(n_max) + 1) * kLevels);
+        A.take(&ws->flat_cnt, ((size_t)flat_octree_blocks(n_max) + 2) * kLevels);  // (totals, and a cut tree's record)
         A.take(&ws->nfirst, NC);
         A.take(&ws->ncount, NC);
         A.take(&ws->nparent, NC);

@@ -96,7 +96,7 @@ enum CounterSlots {
     kCtrAbort = kCtrGroups + 2,               // stage whose bounded wait gave up (0: none)
     kCtrWalkTicket = kCtrGroups + 3,          // walk: next group slot (reset before every walk)
     kCtrTiles = kCtrGroups + 4,               // split walk: tile slots handed out (reset with the ticket)
-    kCtrFlatFull = kCtrGroups + 5,            // octree_flat.cu: the node array was too small
+    kCtrFlatCut = kCtrGroups + 5,             // octree_flat.cu: level at which the node array was too small (0: none)
     kCtrCount = kCtrGroups + 8
 };
 
@@ -591,9 +591,8 @@ inline bool small_sort(const TreeWorkspace *ws, int64_t n) {
 int64_t flat_octree_blocks(int64_t n_max);  // blocks whose counts flat_cnt holds
 cudaError_t launch_octree_flat(TreeWorkspace *ws, int64_t n, cudaStream_t s);
 // Whether launch_octree takes the flat form (leaf levels then come with the
-// octree).  A tree that does not fit the node array is built by
-// one block there, so a workspace with a node array of the caller's own size
-// takes the level-by-level form unless it is small.
+// octree).  A workspace with a node array of the caller's own size takes the
+// level-by-level form unless it is small.
 inline bool flat_octree(const TreeWorkspace *ws) {
     return ws->p.node_cap == 0 || ws->n_max <= 65536;
 }

@@ -24,6 +24,19 @@
 // Blocks of kTile positions sum the counts of all blocks before them
 // themselves while there are at most kFlatMaxBlocks of them; beyond (2^20
 // particles) one more launch scans the blocks' counts, level by level.
+//
+// A node array that is too small cuts the tree as the level-by-level build
+// does: children are numbered in order while they fit, and a cell whose
+// children do not stays a leaf.  With X the first level whose nodes do not all
+// fit, the levels before it are whole, and level X keeps the children of the
+// cells before P, the parent of the node whose number is the array's capacity:
+// numbers below `trunc`, P's first child.  At most seven slots are left, for
+// the children of the first cells of level X (the first kCutKids nodes of
+// level X + 1 tell which) and theirs in turn; everything else of level X is a
+// leaf.  So the same kernels cut the tree, in parallel too; one thread follows
+// the last seven.  Build of tight pairs with leaf_cap 1, which need 1.2 times
+// the default array: N = 1048577 0.39 ms (level by level 0.90; one block
+// building the whole tree 31.7), 1e7 2.4 (4.8).
 #include "common.cuh"
 
 namespace treegb {
@@ -138,92 +151,111 @@ __global__ void __launch_bounds__(1024) k_flat_scan(uint32_t *__restrict__ cnt, 
     if (threadIdx.x == 0) c[(size_t)nblocks * kLevels] = total;
 }
 
-// The tree when the node array is too small for it: one block builds it level
-// by level, children of a node numbered only while they fit (as k_level).
-__device__ __noinline__ void flat_overflow(const uint64_t *__restrict__ skey, int64_t n,
-                                           const int64_t *__restrict__ seg_off, int64_t nseg, uint32_t *nfirst,
-                                           uint32_t *ncount, uint4 *ngeo, uint2 *nlink, uint32_t *nparent,
-                                           uint32_t *ctr, uint32_t lcap, uint32_t node_cap, int32_t *dstatus) {
-    __shared__ uint32_t wt[32], s_trunc;
-    const uint32_t tid = threadIdx.x;
-    for (int64_t b = tid; b < nseg; b += kFlatThreads) {
-        nfirst[b] = nseg > 1 ? (uint32_t)seg_off[b] : 0u;
-        ncount[b] = nseg > 1 ? (uint32_t)(seg_off[b + 1] - seg_off[b]) : (uint32_t)n;
-        nparent[b] = (uint32_t)b;
-    }
-    if (tid == 0) ctr[kCtrLevelStart] = 0;
-    uint32_t start = 0, end = (uint32_t)nseg;
-    for (int L = 0; L < kLevels; ++L) {
-        if (tid == 0) s_trunc = 0xffffffffu;
-        __syncthreads();
-        const int shift = 3 * (kMaxLevel - 1 - L);
-        const uint32_t cmask = ~((1u << (kBits - L)) - 1u);
-        uint32_t base = end;  // first free node
-        for (uint32_t t0 = start; t0 < end; t0 += kFlatThreads) {
-            const uint32_t node = t0 + tid;
-            const bool valid = node < end;
-            const uint32_t first = valid ? nfirst[node] : 0u, count = valid ? ncount[node] : 0u;
-            const uint64_t k0 = valid ? skey[first] : 0u;
-            bool internal = valid && count > lcap && L < kMaxLevel;
-            uint32_t b[9], nch = 0;
-            if (internal) {
-                octant_bounds(skey, first, count, shift, b);
+// A cut tree (see above): what k_flat_nodes leaves for k_flat_links.
+constexpr int kCutKids = 8;
+struct FlatCut {
+    uint32_t first[kCutKids], parent[kCutKids];  // the first nodes of level X + 1: first particle, parent
+    uint32_t kids;                               // how many of them there are
+    uint32_t P;
+};
+static_assert(sizeof(FlatCut) <= kLevels * sizeof(uint32_t), "kept in the row of flat_cnt after the totals");
+constexpr uint32_t kCutInParent = 1u << 31;      // leaf of a particle: not its node of level X, but the one above
+
+// A thread's positions: s, lev and lev of the position before.
+template <int ITEMS>
+struct FlatItems {
+    int sd[ITEMS], lv[ITEMS], pv[ITEMS];
+};
+
+// Numbers, starts, parents and geometry of the nodes that start in the block's
+// positions; ends of the nodes that end there; leaf of every particle.
+// raw[node] = {first child or first particle, its end}.  CUT: the tree is cut
+// at level X (nodes of that level are leaves here, T: number of the first one
+// of the next level).
+template <int ITEMS, bool CUT>
+__device__ __forceinline__ void flat_number(const FlatItems<ITEMS> &it, const uint32_t (*base)[24], int64_t b0,
+                                            int64_t last, int64_t n, const uint64_t *__restrict__ skey,
+                                            uint32_t *__restrict__ nfirst, uint32_t *__restrict__ ncount,
+                                            uint4 *__restrict__ ngeo, uint2 *__restrict__ raw,
+                                            uint32_t *__restrict__ nparent, uint32_t *__restrict__ pleaf, int X,
+                                            uint32_t T, uint32_t cap, FlatCut *cut) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const uint32_t lt = lanemask_lt();
 #pragma unroll
-                for (int o = 0; o < 8; ++o) nch += b[o + 1] > b[o] ? 1u : 0u;
+    for (int q = 0; q < ITEMS; ++q) {
+        const int sd = it.sd[q], lv = it.lv[q], pv = it.pv[q];
+        const int chunk = warp * ITEMS + q, k = chunk * 32 + lane;
+        const int64_t i = b0 + k;
+        const uint64_t k0 = k < last && i < n ? skey[i] : 0u;
+        const uint32_t qx = compact3(k0 >> 2), qy = compact3(k0 >> 1), qz = compact3(k0);
+        uint32_t prev = 0;        // number of the next node of level L - 1 at i
+        uint32_t up = 0;          // node of level L - 1 that starts at i
+        uint32_t closing = 0;     // node of level L - 1 that ends at i
+        uint32_t above = 0;       // CUT: node of level L - 1 that holds i
+        // the levels at which something starts or ends among the warp's positions, or is a leaf, and
+        // the level before them
+        const int top = max(lv, pv);
+        int l0 = (int)__reduce_min_sync(0xffffffffu, (unsigned)min(sd, lv >= 0 ? lv : 64));
+        int l1 = (int)__reduce_max_sync(0xffffffffu, (unsigned)max(top, 0));
+        if (CUT) { l0 = min(l0, X); l1 = min(l1, X + 1); }
+#pragma unroll 1
+        for (int L = max(l0 - 1, 0); L <= l1; ++L) {
+            const bool starts = sd <= L && L <= lv;
+            const bool ends = sd <= L && L <= pv;
+            const uint32_t b = __ballot_sync(0xffffffffu, starts);
+            const uint32_t id = base[chunk][L] + __popc(b & lt);
+            const uint32_t par = L == sd ? prev - 1u : up;  // (of a node that starts here, L > 0)
+            if (CUT && L > X) {
+                if (starts && id - T < (uint32_t)kCutKids) {
+                    cut->first[id - T] = (uint32_t)i;
+                    cut->parent[id - T] = par;
+                }
+                break;
             }
-            uint32_t tot;
-            const uint32_t cf = base + block_exclusive_scan(nch, wt, &tot);
-            if (internal && (uint64_t)cf + nch > node_cap) {
-                internal = false;
-                atomicMin(&s_trunc, cf);
-                set_status(dstatus, TREE_DEV_NODES);
+            if (ends) {
+                const uint32_t c = id - 1u;
+                if (L > sd) raw[closing].y = id;       // the children of the node above end here too
+                if (!CUT || c < cap) {
+                    if (L == pv || (CUT && L == X)) raw[c].y = (uint32_t)i;  // a leaf: its particles end
+                    ncount[c] = (uint32_t)i;           // (its end; k_flat_links subtracts the start)
+                }
+                closing = c;
             }
-            if (valid) {
-                ngeo[node] = make_uint4(compact3(k0 >> 2) & cmask, compact3(k0 >> 1) & cmask, compact3(k0) & cmask,
-                                        (uint32_t)L | (internal ? 0u : 0x100u));
-                nlink[node] = internal ? make_uint2(cf, nch) : make_uint2(first, count);
+            const bool leaf = L == lv || (CUT && L == X);
+            if (starts) {
+                const uint32_t cmask = ~((1u << (kBits - L)) - 1u);
+                if (!CUT || id < cap) {
+                    nfirst[id] = (uint32_t)i;
+                    nparent[id] = L == 0 ? id : par;
+                    ngeo[id] = make_uint4(qx & cmask, qy & cmask, qz & cmask, (uint32_t)L | (leaf ? 0x100u : 0u));
+                    if (leaf) raw[id].x = (uint32_t)i;
+                }
+                if (L > sd) raw[up].x = id;
+                if (CUT && id == cap) cut->P = par;    // (level X: the numbers before it fit)
+                up = id;
             }
-            if (internal) {
-                uint32_t c = cf;
-#pragma unroll
-                for (int o = 0; o < 8; ++o)
-                    if (b[o + 1] > b[o]) {
-                        nfirst[c] = b[o];
-                        ncount[c] = b[o + 1] - b[o];
-                        nparent[c] = node;
-                        ++c;
-                    }
-            }
-            base += tot;
-            __syncthreads();
+            const uint32_t in = starts ? id : id - 1u;
+            if (L == (CUT ? min(lv, X) : lv)) pleaf[i] = CUT && in >= cap ? above | kCutInParent : in;
+            if (CUT) above = in;
+            prev = id;
         }
-        const uint32_t next = min(base, s_trunc);
-        start = end;
-        end = next;
-        if (tid == 0) ctr[kCtrLevelStart + L + 1] = start;
-        __syncthreads();
     }
 }
 
-// Second kernel: numbers, starts, parents and geometry of the nodes that
-// start in the block's positions; ends of the nodes that end there; leaf of
-// every particle.  raw[node] = {first child or first particle, its end}.
-// SCANNED: cnt comes from k_flat_scan.
+// Second kernel: the nodes (flat_number).  SCANNED: cnt comes from k_flat_scan.
 template <int ITEMS, bool SCANNED>
 __global__ void __launch_bounds__(kFlatThreads) k_flat_nodes(
     const uint64_t *__restrict__ skey, int64_t n, const uint8_t *__restrict__ sdig,
-    const uint8_t *__restrict__ plev, const uint32_t *__restrict__ cnt, int nblocks, uint32_t *__restrict__ nfirst, uint32_t *__restrict__ ncount,
-    uint4 *__restrict__ ngeo, uint2 *__restrict__ nlink, uint2 *__restrict__ raw, uint32_t *__restrict__ nparent,
-    uint32_t *__restrict__ pleaf, uint32_t *ctr, uint32_t lcap, uint32_t node_cap, int32_t *dstatus,
-    const int64_t *__restrict__ seg_off, int64_t nseg) {
+    const uint8_t *__restrict__ plev, const uint32_t *__restrict__ cnt, int nblocks, uint32_t *__restrict__ nfirst,
+    uint32_t *__restrict__ ncount, uint4 *__restrict__ ngeo, uint2 *__restrict__ raw, uint32_t *__restrict__ nparent,
+    uint32_t *__restrict__ pleaf, uint32_t *ctr, uint32_t node_cap, FlatCut *cut) {
     constexpr int kTile = kFlatThreads * ITEMS;
     constexpr int kChunks = kTile / 32, kWarps = kFlatThreads / 32;
     __shared__ uint32_t base[kChunks][24];  // per chunk of 32 positions: number of its first node of each level
     __shared__ uint32_t part[kWarps][2][24];
-    __shared__ uint32_t s_end;
+    __shared__ uint32_t s_cut, s_next;      // level at which the tree is cut (kLevels: it fits), T of flat_number
     if (aborted(ctr, kStageAfter)) return;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const uint32_t lt = lanemask_lt();
     // nodes per level in the blocks before this one, and in all
     {
         uint32_t before = 0, all = 0;
@@ -254,35 +286,38 @@ __global__ void __launch_bounds__(kFlatThreads) k_flat_nodes(
         }
         myoff = incl - all + before;
         const uint32_t total = __shfl_sync(0xffffffffu, incl, 31);
-        if (lane == 0) s_end = total;
-        if (blockIdx.x == 0 && total <= node_cap && lane <= kLevels)
-            ctr[kCtrLevelStart + lane] = lane < kLevels ? incl - all : total;
+        // (levels after the first one that does not fit play no part)
+        const uint32_t over = __ballot_sync(0xffffffffu, incl > node_cap);
+        const int X = over ? __ffs(over) - 1 : kLevels;
+        if (lane == 0) s_cut = (uint32_t)X;
+        if (lane == X) s_next = incl;
+        if (blockIdx.x == 0) {
+            if (lane <= min(X, kLevels)) ctr[kCtrLevelStart + lane] = lane < kLevels ? incl - all : total;
+            const uint32_t kids = __shfl_down_sync(0xffffffffu, all, 1);  // nodes of the next level
+            if (lane == X && over) {
+                ctr[kCtrFlatCut] = (uint32_t)X;
+                cut->kids = min(kids, (uint32_t)kCutKids);
+            }
+        }
     }
     __syncthreads();
-    if (s_end > node_cap) {
-        if (blockIdx.x == 0) {
-            if (tid == 0) ctr[kCtrFlatFull] = 1;  // the links below are final; the leaves' particles follow
-            flat_overflow(skey, n, seg_off, nseg, nfirst, ncount, ngeo, nlink, nparent, ctr, lcap, node_cap, dstatus);
-        }
-        return;
-    }
     const int64_t b0 = (int64_t)blockIdx.x * kTile;
     const int64_t last = min((int64_t)kTile, n + 1 - b0);  // position n ends what is still open
-    int sd[ITEMS], lv[ITEMS], pv[ITEMS];
+    FlatItems<ITEMS> it;
 #pragma unroll
     for (int q = 0; q < ITEMS; ++q) {
         const int chunk = warp * ITEMS + q, k = chunk * 32 + lane;
         const int64_t i = b0 + k;
-        sd[q] = 64; lv[q] = -1; pv[q] = -1;
+        it.sd[q] = 64; it.lv[q] = -1; it.pv[q] = -1;
         if (k < last) {
-            sd[q] = i < n ? sdig[i] : 0;
-            lv[q] = i < n ? plev[i] : -1;
-            pv[q] = i > 0 ? plev[i - 1] : -1;
+            it.sd[q] = i < n ? sdig[i] : 0;
+            it.lv[q] = i < n ? plev[i] : -1;
+            it.pv[q] = i > 0 ? plev[i - 1] : -1;
         }
         uint32_t mine = 0;
 #pragma unroll
         for (int L = 0; L < kLevels; ++L) {
-            const uint32_t c = __popc(__ballot_sync(0xffffffffu, sd[q] <= L && L <= lv[q]));
+            const uint32_t c = __popc(__ballot_sync(0xffffffffu, it.sd[q] <= L && L <= it.lv[q]));
             if (lane == L) mine = c;
         }
         if (lane < 24) base[chunk][lane] = mine;
@@ -297,73 +332,132 @@ __global__ void __launch_bounds__(kFlatThreads) k_flat_nodes(
         }
     }
     __syncthreads();
-#pragma unroll
-    for (int q = 0; q < ITEMS; ++q) {
-        const int chunk = warp * ITEMS + q, k = chunk * 32 + lane;
-        const int64_t i = b0 + k;
-        const uint64_t k0 = k < last && i < n ? skey[i] : 0u;
-        const uint32_t qx = compact3(k0 >> 2), qy = compact3(k0 >> 1), qz = compact3(k0);
-        uint32_t prev = 0;        // number of the next node of level L - 1 at i
-        uint32_t up = 0;          // node of level L - 1 that starts at i
-        uint32_t closing = 0;     // node of level L - 1 that ends at i
-        // the levels at which something starts or ends among the warp's positions, or is a leaf, and
-        // the level before them
-        const int top = max(lv[q], pv[q]);
-        const int l0 = (int)__reduce_min_sync(0xffffffffu, (unsigned)min(sd[q], lv[q] >= 0 ? lv[q] : 64));
-        const int l1 = (int)__reduce_max_sync(0xffffffffu, (unsigned)max(top, 0));
-#pragma unroll 1
-        for (int L = max(l0 - 1, 0); L <= l1; ++L) {
-            const bool starts = sd[q] <= L && L <= lv[q];
-            const bool ends = sd[q] <= L && L <= pv[q];
-            const uint32_t b = __ballot_sync(0xffffffffu, starts);
-            const uint32_t id = base[chunk][L] + __popc(b & lt);
-            if (ends) {
-                const uint32_t c = id - 1u;
-                if (L > sd[q]) raw[closing].y = id;       // the children of the node above end here too
-                if (L == pv[q]) raw[c].y = (uint32_t)i;   // a leaf: its particles end
-                ncount[c] = (uint32_t)i;                  // (its end; k_flat_links subtracts the start)
-                closing = c;
-            }
-            if (starts) {
-                const uint32_t cmask = ~((1u << (kBits - L)) - 1u);
-                nfirst[id] = (uint32_t)i;
-                nparent[id] = L == 0 ? id : L == sd[q] ? prev - 1u : up;
-                ngeo[id] = make_uint4(qx & cmask, qy & cmask, qz & cmask, (uint32_t)L | (L == lv[q] ? 0x100u : 0u));
-                if (L > sd[q]) raw[up].x = id;
-                if (L == lv[q]) raw[id].x = (uint32_t)i;
-                up = id;
-            }
-            if (L == lv[q]) pleaf[i] = starts ? id : id - 1u;
-            prev = id;
+    if (s_cut == (uint32_t)kLevels)
+        flat_number<ITEMS, false>(it, base, b0, last, n, skey, nfirst, ncount, ngeo, raw, nparent, pleaf, 0, 0u, 0u,
+                                  nullptr);
+    else
+        flat_number<ITEMS, true>(it, base, b0, last, n, skey, nfirst, ncount, ngeo, raw, nparent, pleaf, (int)s_cut,
+                                 s_next, node_cap, cut);
+}
+
+// Third kernel for a tree that is cut at level X: links, leaf flags, the nodes
+// in the slots that are left, and the leaves of the particles.
+__device__ __noinline__ void flat_links_cut(const uint64_t *__restrict__ skey, int64_t n, uint32_t *ctr,
+                                            const FlatCut *cut, const uint2 *raw, uint32_t *nfirst, uint32_t *ncount,
+                                            uint4 *ngeo, uint2 *nlink, uint32_t *nparent, uint8_t *plev,
+                                            uint32_t *pleaf, uint32_t lcap, uint32_t cap, int32_t *dstatus) {
+    // the last nodes, numbers trunc + q, in order, and the cells of level X that have children
+    struct Node { uint32_t first, end, parent, level, child, nchild; };
+    __shared__ Node tail[kCutKids];
+    __shared__ uint32_t s_cell[kCutKids], s_child[kCutKids], s_nchild[kCutKids], s_tail, s_cells;
+    const uint32_t X = ctr[kCtrFlatCut], P = cut->P, trunc = raw[P].x;
+    if (threadIdx.x == 0) {
+        const bool store = blockIdx.x == 0;
+        uint32_t free = trunc, cells = 0;
+        for (uint32_t k = 0; k < cut->kids;) {
+            const uint32_t p = cut->parent[k];
+            uint32_t m = 1;
+            while (k + m < cut->kids && cut->parent[k + m] == p) ++m;
+            if (p >= trunc || free + m > cap) break;
+            s_cell[cells] = p; s_child[cells] = free; s_nchild[cells] = m;
+            ++cells;
+            for (uint32_t j = 0; j < m; ++j)
+                tail[free - trunc + j] =
+                    Node{cut->first[k + j], j + 1 < m ? cut->first[k + j + 1] : raw[p].y, p, X + 1u, 0u, 0u};
+            free += m;
+            k += m;
         }
+        if (store) ctr[kCtrLevelStart + X + 1] = trunc;
+        uint32_t q = 0;
+        for (uint32_t L = X + 1; L < (uint32_t)kLevels; ++L) {
+            const uint32_t end = free - trunc;
+            if (store) ctr[kCtrLevelStart + L + 1] = free;
+            bool fits = true;
+            for (; q < end; ++q) {
+                const Node c = tail[q];
+                if (!fits || c.end - c.first <= lcap || L == (uint32_t)kMaxLevel) continue;
+                uint32_t b[9], m = 0;
+                octant_bounds(skey, c.first, c.end - c.first, 3 * (kMaxLevel - 1 - (int)L), b);
+                for (int o = 0; o < 8; ++o) m += b[o + 1] > b[o] ? 1u : 0u;
+                if (free + m > cap) { fits = false; continue; }
+                tail[q].child = free;
+                tail[q].nchild = m;
+                for (int o = 0; o < 8; ++o)
+                    if (b[o + 1] > b[o]) tail[free++ - trunc] = Node{b[o], b[o + 1], trunc + q, L + 1u, 0u, 0u};
+            }
+        }
+        s_tail = free - trunc;
+        s_cells = cells;
+        if (store) set_status(dstatus, TREE_DEV_NODES);
+    }
+    __syncthreads();
+    const uint32_t ntail = s_tail, ncells = s_cells;
+    const uint32_t t0 = blockIdx.x * blockDim.x + threadIdx.x, stride = gridDim.x * blockDim.x;
+    if (t0 < ntail) {
+        const Node c = tail[t0];
+        const uint32_t id = trunc + t0, cmask = ~((1u << (kBits - c.level)) - 1u);
+        const uint64_t k0 = skey[c.first];
+        nfirst[id] = c.first;
+        ncount[id] = c.end - c.first;
+        nparent[id] = c.parent;
+        ngeo[id] = make_uint4(compact3(k0 >> 2) & cmask, compact3(k0 >> 1) & cmask, compact3(k0) & cmask,
+                              c.level | (c.nchild ? 0u : 0x100u));
+        nlink[id] = c.nchild ? make_uint2(c.child, c.nchild) : make_uint2(c.first, c.end - c.first);
+    }
+    for (uint32_t c = t0; c < trunc; c += stride) {
+        const uint2 r = raw[c];
+        const uint32_t w = ngeo[c].w, lev = w & 0xffu, first = nfirst[c], count = ncount[c] - first;
+        ncount[c] = count;
+        uint2 l = make_uint2(r.x, r.y - r.x);
+        if (lev == X) {
+            for (uint32_t k = 0; k < ncells; ++k)
+                if (s_cell[k] == c) {
+                    l = make_uint2(s_child[k], s_nchild[k]);
+                    ngeo[c].w = lev;
+                }
+        } else if (!(w & 0x100u) && lev + 1u == X && r.x >= trunc) {
+            l = make_uint2(first, count);  // P and the cells after it
+            ngeo[c].w = w | 0x100u;
+        }
+        nlink[c] = l;
+    }
+    for (int64_t i = t0; i < n; i += stride) {
+        if (plev[i] < X) continue;
+        uint32_t a = pleaf[i], lev = X;
+        if (a >= trunc) {  // (numbers from trunc to the capacity: children of P)
+            a = a & kCutInParent ? a & ~kCutInParent : P;
+            lev = X - 1u;
+        } else {
+            for (uint32_t q = 0; q < ntail; ++q)
+                if (tail[q].parent == a && tail[q].first <= i && i < tail[q].end) { a = trunc + q; lev = tail[q].level; }
+        }
+        pleaf[i] = a;
+        plev[i] = (uint8_t)lev;
     }
 }
 
-// Third kernel: ends become counts.  (When the node array was too small, the
-// counts are there, and the particles learn their leaves: a warp per leaf.)
-__global__ void __launch_bounds__(256) k_flat_links(const uint32_t *__restrict__ ctr, const uint2 *__restrict__ raw,
-                                                    const uint32_t *__restrict__ nfirst, uint32_t *__restrict__ ncount,
-                                                    const uint4 *__restrict__ ngeo, uint2 *__restrict__ nlink,
-                                                    uint8_t *__restrict__ plev, uint32_t *__restrict__ pleaf) {
+// Third kernel: ends become counts.
+__global__ void __launch_bounds__(256) k_flat_links(const uint64_t *__restrict__ skey, int64_t n, uint32_t *ctr,
+                                                    const FlatCut *cut, const uint2 *raw, uint32_t *nfirst,
+                                                    uint32_t *ncount, uint4 *ngeo, uint2 *nlink, uint32_t *nparent,
+                                                    uint8_t *plev, uint32_t *pleaf, uint32_t lcap, uint32_t node_cap,
+                                                    int32_t *dstatus) {
     if (aborted(ctr, kStageAfter)) return;
-    const uint32_t nn = ctr[kCtrLevelStart + kLevels];
-    if (ctr[kCtrFlatFull]) {
-        for (uint32_t c = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; c < nn; c += (gridDim.x * blockDim.x) >> 5) {
-            const uint32_t w = ngeo[c].w;
-            if (!((w >> 8) & 1u)) continue;
-            const uint2 l = nlink[c];
-            for (uint32_t j = l.x + (threadIdx.x & 31); j < l.x + l.y; j += 32) {
-                plev[j] = (uint8_t)(w & 0xffu);
-                pleaf[j] = c;
-            }
-        }
+    if (ctr[kCtrFlatCut]) {
+        flat_links_cut(skey, n, ctr, cut, raw, nfirst, ncount, ngeo, nlink, nparent, plev, pleaf, lcap, node_cap,
+                       dstatus);
         return;
     }
+    const uint32_t nn = ctr[kCtrLevelStart + kLevels];
     for (uint32_t c = blockIdx.x * blockDim.x + threadIdx.x; c < nn; c += gridDim.x * blockDim.x) {
         const uint2 r = raw[c];
         nlink[c] = make_uint2(r.x, r.y - r.x);
         ncount[c] -= nfirst[c];
     }
+}
+
+static FlatCut *flat_cut(TreeWorkspace *ws) {
+    return reinterpret_cast<FlatCut *>(ws->flat_cnt + (size_t)(flat_octree_blocks(ws->n_max) + 1) * kLevels);
 }
 
 template <int ITEMS, bool SCANNED>
@@ -379,10 +473,9 @@ static void flat_launch(TreeWorkspace *ws, int64_t n, cudaStream_t s) {
     ws->launches += SCANNED ? 3 : 2;
     // position n may need a block of its own
     const int nb1 = (int)((n + kFlatThreads * ITEMS) / (kFlatThreads * ITEMS));
-    k_flat_nodes<ITEMS, SCANNED><<<nb1, kFlatThreads, 0, s>>>(ws->key, n, ws->sdig, ws->plev, ws->flat_cnt, nb, ws->nfirst,
-                                                    ws->ncount, ws->ngeo, ws->nlink, ws->nraw, ws->nparent, ws->pleaf,
-                                                    ws->ctr, (uint32_t)ws->p.leaf_cap, (uint32_t)ws->node_cap,
-                                                    ws->dstatus, ws->seg_off, ws->nseg);
+    k_flat_nodes<ITEMS, SCANNED><<<nb1, kFlatThreads, 0, s>>>(ws->key, n, ws->sdig, ws->plev, ws->flat_cnt, nb,
+                                                              ws->nfirst, ws->ncount, ws->ngeo, ws->nraw, ws->nparent,
+                                                              ws->pleaf, ws->ctr, (uint32_t)ws->node_cap, flat_cut(ws));
 }
 
 cudaError_t launch_octree_flat(TreeWorkspace *ws, int64_t n, cudaStream_t s) {
@@ -393,8 +486,9 @@ cudaError_t launch_octree_flat(TreeWorkspace *ws, int64_t n, cudaStream_t s) {
     else if (n <= 4 * one) flat_launch<4, false>(ws, n, s);
     else if (n <= kFlatItemsMax * one) flat_launch<kFlatItemsMax, false>(ws, n, s);
     else flat_launch<kFlatItemsMax, true>(ws, n, s);
-    k_flat_links<<<grid_for(ws->node_cap, 256, 152 * 8), 256, 0, s>>>(ws->ctr, ws->nraw, ws->nfirst, ws->ncount,
-                                                                      ws->ngeo, ws->nlink, ws->plev, ws->pleaf);
+    k_flat_links<<<grid_for(ws->node_cap, 256, 152 * 8), 256, 0, s>>>(
+        ws->key, n, ws->ctr, flat_cut(ws), ws->nraw, ws->nfirst, ws->ncount, ws->ngeo, ws->nlink, ws->nparent, ws->plev,
+        ws->pleaf, (uint32_t)ws->p.leaf_cap, (uint32_t)ws->node_cap, ws->dstatus);
     ws->launches += 1;
     return cudaGetLastError();
 }
