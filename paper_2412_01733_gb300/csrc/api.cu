@@ -268,6 +268,7 @@ tree_status_t tree_workspace_create(int64_t n_max, const TreeParams *p, TreeWork
     ws->sort_tiles_max = (n_max + kSortTile - 1) / kSortTile + 1;
     ws->level_tiles_max = (ws->node_cap + kLevelThreads - 1) / kLevelThreads + 1;
     ws->groups_max = n_max + 1;  // a group holds at least one particle
+    ws->small_max = small_sort_limit(n_max);
     const int64_t chunks_max = (n_max + 15) / 16 + 1;
     const size_t v4 = p->precision == TREE_F64 ? sizeof(double4a) : sizeof(float4);
     const size_t v2 = p->precision == TREE_F64 ? sizeof(double2a) : sizeof(float2);

@@ -143,6 +143,7 @@ struct TreeWorkspace {
     uint32_t *level_status = nullptr;  // [22][level_tiles]
     uint32_t *ctr = nullptr;           // kCtrCount words
     // box
+    int64_t small_max = 0;             // particles of one system that one cluster sorts, at most (small_sort_limit)
     int box_parts = 0;                 // partial boxes of the last box reduction
     bool withhold = false;             // tree_set_waits has a sort tile withhold its words (test injection)
     double *part = nullptr;            // reduction partials [kMaxBlocksReduce][8]
@@ -582,10 +583,11 @@ cudaError_t launch_octree(TreeWorkspace *ws, int64_t n, cudaStream_t s);
 // sort_small.cu
 cudaError_t launch_small_keys(TreeWorkspace *ws, const void *x, int64_t n, cudaStream_t s);
 cudaError_t launch_small_sort(TreeWorkspace *ws, int64_t n, cudaStream_t s);
+int64_t small_sort_limit(int64_t n_max);  // largest system of a workspace that the device has room to sort so
 // Whether keys and sort take the one-cluster form: one small system, and no
 // onesweep tile to withhold.
 inline bool small_sort(const TreeWorkspace *ws, int64_t n) {
-    return ws->nseg == 1 && n <= kSmallSortMax && !ws->withhold;
+    return ws->nseg == 1 && n <= ws->small_max && !ws->withhold;
 }
 // octree_flat.cu
 int64_t flat_octree_blocks(int64_t n_max);  // blocks whose counts flat_cnt holds

@@ -10,7 +10,7 @@
 // keys that agree in them are put in order by insertion, since LSD passes
 // leave such a run in the order of its particles' indices.  A run of more than
 // kRunMax of them sends the cluster through all eight digits instead (a galaxy
-// of 65536 has such runs in the top five digits: 127 us against 86).  Box, keys
+// of 65536 has such runs in the top five digits).  Box, keys
 // and sort: N = 1031 96 -> 39 us, 30011 129 -> 61, 65536 136 -> 83.  (Eight
 // blocks of up to eight keys a thread: 47, 75 and 115; a pass is the keys' way
 // through distributed shared memory, which more blocks share.)
@@ -216,25 +216,53 @@ cudaError_t launch_small_keys(TreeWorkspace *ws, const void *x, int64_t n, cudaS
     return cudaGetLastError();
 }
 
-cudaError_t launch_small_sort(TreeWorkspace *ws, int64_t n, cudaStream_t s) {
-    // more blocks before more keys per thread: a pass is latency, and a block's part of it grows with its keys
-    const uint32_t C = n <= 1024 ? 1 : n <= 2048 ? 2 : n <= 4096 ? 4 : n <= 8192 ? 8 : kSmCluster;
-    const uint32_t Q = (uint32_t)((n + C - 1) / C);
+// Launch of n particles: more blocks before more keys per thread (a pass is
+// latency, and a block's part of it grows with its keys).
+static uint32_t cluster_blocks(int64_t n) {
+    return n <= 1024 ? 1 : n <= 2048 ? 2 : n <= 4096 ? 4 : n <= 8192 ? 8 : kSmCluster;
+}
+
+static cudaError_t cluster_config(uint32_t C, cudaStream_t s, cudaLaunchConfig_t &cfg, cudaLaunchAttribute &at) {
     cudaError_t e = cudaFuncSetAttribute(k_small_sort, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          (int)sizeof(SmallSmem));
     if (e == cudaSuccess) e = cudaFuncSetAttribute(k_small_sort, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
-    if (e != cudaSuccess) return e;
-    cudaLaunchConfig_t cfg{};
+    cfg = cudaLaunchConfig_t{};
     cfg.gridDim = dim3(C);
     cfg.blockDim = dim3(kSmThreads);
     cfg.dynamicSmemBytes = sizeof(SmallSmem);
     cfg.stream = s;
-    cudaLaunchAttribute at{};
+    at = cudaLaunchAttribute{};
     at.id = cudaLaunchAttributeClusterDimension;
     at.val.clusterDim.x = C;
     at.val.clusterDim.y = at.val.clusterDim.z = 1;
     cfg.attrs = &at;
     cfg.numAttrs = 1;
+    return e;
+}
+
+// A device that is partitioned, or restricted to some of its SMs, may have no
+// room for a cluster of sixteen blocks of 100 KB: larger systems then take the
+// general passes.
+int64_t small_sort_limit(int64_t n_max) {
+    for (uint32_t C = cluster_blocks(n_max < kSmallSortMax ? n_max : kSmallSortMax); C > 0; C /= 2) {
+        cudaLaunchConfig_t cfg;
+        cudaLaunchAttribute at;
+        int clusters = 0;
+        if (cluster_config(C, nullptr, cfg, at) == cudaSuccess &&
+            cudaOccupancyMaxActiveClusters(&clusters, k_small_sort, &cfg) == cudaSuccess && clusters > 0)
+            return C == kSmCluster ? kSmallSortMax : 1024 * (int64_t)C;
+        cudaGetLastError();
+    }
+    return 0;
+}
+
+cudaError_t launch_small_sort(TreeWorkspace *ws, int64_t n, cudaStream_t s) {
+    const uint32_t C = cluster_blocks(n);
+    const uint32_t Q = (uint32_t)((n + C - 1) / C);
+    cudaLaunchConfig_t cfg;
+    cudaLaunchAttribute at;
+    cudaError_t e = cluster_config(C, s, cfg, at);
+    if (e != cudaSuccess) return e;
     e = cudaLaunchKernelEx(&cfg, k_small_sort, (const uint64_t *)ws->key_alt, ws->key, ws->idx, (uint32_t)n, Q,
                            n <= kTop5Max ? 3 : 2);
     ws->launches += 1;
