@@ -152,7 +152,14 @@ tree_status_t tree_params_default(TreeParams *p);
 
 /* Allocates a workspace for up to n_max particles on the current device.
  * p (host) is copied.  On success *out owns device memory until
- * tree_workspace_destroy.  Errors: TREE_ERR_ARG (bad parameter, n_max < 0),
+ * tree_workspace_destroy.  A workspace of up to 131072 particles also holds
+ * tile slots that spread its force walk over the whole GPU, as many as its
+ * theta and group_size are expected to need: 0.6 GB in FP32 and 1.1 GB in FP64
+ * at 131072 particles and theta = 0.7, in proportion to n_max log(n_max) /
+ * theta^2, none where theta is small (below 0.45 at 131072) or the device has
+ * no room for them.  Without them, or when tree_set_params asks for a walk
+ * that needs more (a smaller theta, groups of 16), the walk gives the same
+ * bits, one warp to a group.  Errors: TREE_ERR_ARG (bad parameter, n_max < 0),
  * TREE_ERR_ALLOC. */
 tree_status_t tree_workspace_create(int64_t n_max, const TreeParams *p, TreeWorkspace **out);
 tree_status_t tree_workspace_destroy(TreeWorkspace *ws);
@@ -297,8 +304,8 @@ tree_status_t leapfrog_graph_launch(TreeWorkspace *ws, void *stream);
  * ([3][n], [n] of base->precision; with nseg > 1 the ensemble given by
  * offsets as in tree_set_segments) for every leaf_cap in {4, 8, 16},
  * group_size in {16, 32, 64} and stack_depth in {512, 1024}, the other
- * parameters taken from base, each leaf_cap in a temporary workspace of
- * n_max = n.  Leaf capacity and group size change the cells that pass the
+ * parameters taken from base, each leaf_cap and group_size in a temporary
+ * workspace of n_max = n.  Leaf capacity and group size change the cells that pass the
  * opening criterion of Sec. 2, so they change the force error: every
  * candidate's accelerations are compared with the FP64 direct sum of Eq. 1
  * (each target against its own system) on a fixed sample of up to 512

@@ -1087,16 +1087,17 @@ tree_status_t tree_autotune(const TreeParams *base, int64_t nseg, const int64_t 
     }
     tree_status_t ret = TREE_OK;
     for (int li = 0; li < 3 && ret == TREE_OK; ++li) {
-        TreeParams p = *base;
-        p.leaf_cap = lcaps[li];
-        p.node_cap = 0;
-        TreeWorkspace *ws = nullptr;
-        st = tree_workspace_create(n, &p, &ws);
-        if (st != TREE_OK) { ret = st; break; }
-        if (nseg > 1) st = tree_set_segments(ws, nseg, offsets);
-        for (int gi = 0; gi < 3 && st == TREE_OK; ++gi) {
+        for (int gi = 0; gi < 3 && ret == TREE_OK; ++gi) {
+            // a workspace as the caller would create it: its tile slots, and with them the walk, follow the group size
+            TreeParams p = *base;
+            p.leaf_cap = lcaps[li];
+            p.group_size = gss[gi];
+            p.node_cap = 0;
+            TreeWorkspace *ws = nullptr;
+            st = tree_workspace_create(n, &p, &ws);
+            if (st != TREE_OK) { ret = st; break; }
+            if (nseg > 1) st = tree_set_segments(ws, nseg, offsets);
             for (int si = 0; si < 2 && st == TREE_OK; ++si) {
-                p.group_size = gss[gi];
                 p.stack_depth = stacks[si];
                 st = tree_set_params(ws, &p);
                 if (st != TREE_OK) break;
@@ -1135,9 +1136,9 @@ tree_status_t tree_autotune(const TreeParams *base, int64_t nseg, const int64_t 
                     *best = p;
                 }
             }
+            if (st != TREE_OK) ret = st;
+            tree_workspace_destroy(ws);
         }
-        if (st != TREE_OK) ret = st;
-        tree_workspace_destroy(ws);
     }
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
