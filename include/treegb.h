@@ -128,11 +128,14 @@ typedef struct {
     int64_t n_segments;         /* independent systems (tree_set_segments); 1 = a single system */
 } TreeInfo;
 
-/* Phases timed by tree_timing_read (indices into its ms[] output). */
+/* Phases timed by tree_timing_read (indices into its ms[] output).  In a force
+ * evaluation and a step the gather runs beside the octree, and the moments
+ * beside the walk groups and, in small systems, part of the walk, so the
+ * phases' times may add up to more than the call's. */
 #define TREE_PHASE_BOX 0     /* box reduction; in leapfrog_step: kick + drift + box (Eqs. 2-3) */
 #define TREE_PHASE_KEYS 1    /* Morton keys + radix histograms */
-#define TREE_PHASE_SORT 2    /* eight onesweep passes */
-#define TREE_PHASE_OCTREE 3  /* level-by-level octree */
+#define TREE_PHASE_SORT 2    /* radix sort of the keys */
+#define TREE_PHASE_OCTREE 3  /* octree (tree_build: and walk groups) */
 #define TREE_PHASE_GATHER 4  /* positions/masses into key order */
 #define TREE_PHASE_MOMENTS 5 /* FP64 moments, bottom-up */
 #define TREE_PHASE_WALK 6    /* tree walk + forces (+ fused write-back and Eq. 5 kick) */

@@ -38,7 +38,7 @@ constexpr int64_t kMaxNodes = (int64_t)1 << 29;  // node indices fit 29 bits (wa
 constexpr int64_t kWalkOrderMaxN = (int64_t)1 << 22;
 
 // Split walk (walk.cuh): workspaces of at most this many particles (FP32,
-// FP64; the measured lines are in walk.cuh) keep the tile slots that their
+// FP64; measured on both sides in walk.cuh) keep the tile slots that their
 // parameters are expected to need (split_slots), unless that is more than
 // kTilesPer for each particle (theta below 0.45 at N = 131072; 660 B a slot in
 // FP32).  Slots are handed out kTileChunk at a time.
@@ -48,10 +48,12 @@ constexpr int kTileChunk = 16;
 constexpr uint32_t kTilesFull = 0xffffffffu;     // group whose tiles found no slot
 
 // Moments up to kClimbMaxN particles climb the tree in one launch, up to
-// kClimbPlainN without sorting the leaves by their particle counts first
-// (Plummer spheres, all moments, level by level -> climbing: N = 1031 182 ->
-// 53 us, 30011 241 -> 83, 131072 272 -> 88 plain; 2^20 355 -> 220 sorted;
-// beyond, the level-by-level form's full warps gain on it).
+// kClimbPlainN without sorting the leaves by their particle counts first.
+// Plummer spheres, FP32, all moments in us (plain / sorted / level by level):
+// N = 30011 77 / 94 / 232, 131072 90 / 102 / 257, 200000 116 / 112 / 277, 2^20
+// 286 / 206 / 346, 2^21 535 / 335 / 419, 4e6 1009 / 555 / 568, 1e7 - / 1320 /
+// 1000.  So sorting pays from about 170000 on, and climbing until about 4e6;
+// between kClimbMaxN and there level by level costs 0.1 ms at most, of 10.
 constexpr int64_t kClimbMaxN = (int64_t)1 << 20, kClimbPlainN = (int64_t)1 << 17;
 
 // lookback status words: 2-bit flag + 30-bit value
@@ -334,8 +336,6 @@ struct WaitCtx {
     long long limit;       // clock cycles
 };
 
-// True when a bounded wait of an earlier stage of this build gave up: the
-// calling kernel (of stage `stage`) must return without touching the data.
 // Whether the FP32 walk's quadrupole far-cell term with r^-5 taken out of the
 // acceleration (pc_pair's R5 form) stays in the normal FP32 range for every
 // far cell of a segment whose tree is the cube of side L = 2^k and whose total
@@ -357,6 +357,8 @@ __device__ __forceinline__ bool pc_r5_fits(int k, double m_root) {
     return fabs(m_root) * span * span * span <= 1e300;
 }
 
+// True when a bounded wait of an earlier stage of this build gave up: the
+// calling kernel (of stage `stage`) must return without touching the data.
 __device__ __forceinline__ bool aborted(const uint32_t *ctr, uint32_t stage) {
     const uint32_t a = ctr[kCtrAbort];
     return a != 0u && a != stage;

@@ -11,12 +11,14 @@
 // the partial sums are folded, group by group, in the order of the tiles
 // (kWalkFold).  Each tile's partial sums and the order of the folds are those
 // of the one-warp walk, so the results are the same bits, alone or in an
-// ensemble.  Force on a Plummer sphere, theta = 0.7 (one-warp -> split, the
-// moments then beside the traversal): FP32 N = 16384 455 -> 221 us, 65536 742
-// -> 528, 131072 987 -> 917, but 262144 1585 -> 1649 (1.25 KB of slot traffic
-// per tile, and the traversal no longer hides behind the arithmetic); FP64
-// walk alone, full far-cell form, N = 16384 12.8 -> 2.7 ms, 65536 21.6 ->
-// 13.1, 131072 32.6 -> 28.7.  walk_splits() draws the lines there.
+// ensemble.  Force on a Plummer sphere, theta = 0.7, in ms (one-warp -> split,
+// the moments then beside the traversal): FP32 N = 16384 0.455 -> 0.221, 65537
+// 0.659 -> 0.558, 100000 0.749 -> 0.712, 131072 0.872 -> 0.919, 200000 1.21 ->
+// 1.29 (1.25 KB of slot traffic per tile, and the traversal no longer hides
+// behind the arithmetic: the two cross near 115000); FP64 16384 12.8 -> 2.7
+// (walk alone), 65537 19.7 -> 12.9, 131072 29.7 -> 27.2, 200000 45.7 -> 43.8,
+// 262144 58.6 -> 57.8, 400000 91.6 -> 93.0 (above 2^17 a few percent for twice
+// the slots and more).  walk_splits() draws the lines, at 2^17 in both.
 //
 // Traversal (per warp, depth first, stack in shared memory):
 //   the stack holds ranges of sibling nodes (children are contiguous in the
@@ -452,12 +454,12 @@ __device__ __forceinline__ void part_pc(const Stage<Real> &S, const Targets<Real
 // batches of partial sums in registers (the fold of the longest group is a
 // chain of loads: 65 us at N = 16384 with one batch that spilled, 20 with two
 // that fit) and runs few groups: 3 blocks.
-constexpr int walk_blocks(int mode, int tpl, size_t real) {
+constexpr int walk_blocks(int mode, int tpl) {
     return mode == kWalkFold ? 3 : tpl == 2 ? 4 : 5;
 }
 
 template <typename Real, int TPL, bool QUAD, bool KAHAN, bool SOFT, int MODE>
-__global__ void __launch_bounds__(kWalkWarps * 32, walk_blocks(MODE, TPL, sizeof(Real))) k_walk(const WalkArgs A) {
+__global__ void __launch_bounds__(kWalkWarps * 32, walk_blocks(MODE, TPL)) k_walk(const WalkArgs A) {
     using V4 = typename Vec4<Real>::T;
     using V2 = typename Vec2<Real>::T;
     extern __shared__ __align__(32) unsigned char smem[];
