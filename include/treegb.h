@@ -218,8 +218,8 @@ tree_status_t tree_forces(TreeWorkspace *ws, void *a, void *phi, int32_t flags, 
  * accelerations) and phi_bar [n] or NULL (of the potentials), ADDS the
  * gradient to x_bar [3][n] and m_bar [n] (either may be NULL), all in the
  * caller's order and the workspace precision.  FP64 accumulation of the
- * cotangents.  Scratch is allocated on the first call (about 56 B per
- * particle + 80 B per node).  Errors: TREE_ERR_STATE without stored lists. */
+ * cotangents.  Scratch is allocated on the first call (48 B per particle in
+ * FP32, 64 in FP64, + 80 B per node).  Errors: TREE_ERR_STATE without stored lists. */
 tree_status_t tree_forces_adjoint(TreeWorkspace *ws, const void *a_bar, const void *phi_bar, void *x_bar,
                                   void *m_bar, void *stream);
 
